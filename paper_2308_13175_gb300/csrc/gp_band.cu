@@ -262,9 +262,12 @@ void band_free(gp_band* b) {
   gp_free(b->tv_inv);
   gp_free(b->pts);
   gp_free(b->pts_sorted);
-  gp_free(b->cell_start);
+  gp_free(b->cell_table);
+  gp_free(b->cell_sup);
+  gp_free(b->cell_blk);
+  gp_free(b->cell_occ);
   gp_free(b->sigma);
-  gp_free(b->normals);
+  gp_free(b->seeds);
   gp_free(b->perm);
   gp_free(b->inv_perm);
   gp_free(b->order_tiles);

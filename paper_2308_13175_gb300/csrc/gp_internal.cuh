@@ -81,10 +81,14 @@ struct gp_band {
 
   // Point cloud: original order copy, cell list sorted copy, sigma, permutation.
   float* pts = nullptr;            // J x 3
-  float4* pts_sorted = nullptr;    // J: x, y, z, original index (int bits)
-  int32_t* cell_start = nullptr;   // G^3 + 1
+  float4* pts_sorted = nullptr;    // the points in chunks of four, by search cell (4 per chunk)
+  int64_t n_chunks = 0;
+  int32_t* cell_table = nullptr;   // record of each block of 4^3 search cells, -1 where it holds no point
+  unsigned long long* cell_sup = nullptr;  // which blocks of each 4^3 blocks hold points
+  float4* cell_blk = nullptr;      // two per stored block: its plane, cells and first occupied cell
+  int32_t* cell_occ = nullptr;     // first chunk of each occupied cell, one more entry per block
   float* sigma = nullptr;          // J
-  float* normals = nullptr;        // J x 3: unit normal estimate (PCA of the sigma-ball), seeds gp_nn
+  float4* seeds = nullptr;         // J: x, y, z and a packed normal estimate (PCA of the sigma-ball; 0 without sigma), seeds gp_nn
   int32_t* perm = nullptr;         // J: Pi_e of the cached epoch
   int32_t* inv_perm = nullptr;     // J: Pi_e^-1 (point -> pool slot within a replica)
   int32_t* order_tiles = nullptr;  // per-tile counts / offsets of the spatial batch order

@@ -10,15 +10,15 @@
 // The scan works in float32.  With E_j the exact squared distance, the float32
 // value is within a relative 5u (u = 2^-24) of E_j (plus an absolute 1e-30
 // covering underflow) and the float64 value within 3*2^-53.  Keeping the
-// smallest float32 distance b1 (index j1) and the second smallest b2 over all
-// scanned points: if b2 > b1 (1 + 2 eps) + 1e-30 with eps = 2^-18 >> 5u, every
-// other point has E_k > E_j1 (1 + eps), hence a larger float64 value, so j1 is
-// the float64 answer.  Otherwise (a near tie, e.g. duplicate points) the
-// scanned cells are visited again and every point within that margin is ranked
-// by its float64 value and index.  Rings of cells are scanned around the
-// query's cell until the distance from q to the scanned box, less a rounding
-// margin of 1e-5 (1 + |q|_inf), exceeds sqrt(b1 (1 + 8 eps)), so no unscanned
-// point can enter the comparison.
+// smallest float32 distance b1 and the second smallest b2 over all scanned
+// points: if b2 > b1 (1 + 2 eps) + 1e-30 with eps = 2^-18 >> 5u, every other
+// point has E_k > E_j1 (1 + eps), hence a larger float64 value, so the point of
+// b1 is the float64 answer.  Otherwise (a near tie, e.g. duplicate points) the
+// cells within the margin are visited again and every point within it is
+// ranked by its float64 value and index.  A cell is left out only if no point
+// of it can be within sqrt(b1 (1 + 8 eps)) of q: its super-block or block does
+// not meet that ball, or the plane of its block keeps its points out of it
+// (nn_block_cells), each taken with a rounding margin of 1e-5 (2 + |q|_inf).
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -28,47 +28,260 @@
 
 namespace {
 
-__global__ void k_point_cells(const float* __restrict__ pts, int64_t J, NNGrid g, int32_t* __restrict__ cid,
-                              int32_t* __restrict__ counts) {
+__device__ __forceinline__ int nn_local_cell(float4 p, const NNGrid& g) {
+  return (nn_cell(p.x, g) & 3) | ((nn_cell(p.y, g) & 3) << 2) | ((nn_cell(p.z, g) & 3) << 4);
+}
+
+__global__ void k_point_blocks(const float* __restrict__ pts, int64_t J, NNGrid g, int32_t* __restrict__ bid,
+                               int32_t* __restrict__ counts) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= J) return;
-  int cx = nn_cell(pts[3 * j], g), cy = nn_cell(pts[3 * j + 1], g), cz = nn_cell(pts[3 * j + 2], g);
-  int32_t c = (int32_t)(((int64_t)cz * g.G + cy) * g.G + cx);
-  cid[j] = c;
+  const int bx = nn_cell(pts[3 * j], g) >> 2, by = nn_cell(pts[3 * j + 1], g) >> 2, bz = nn_cell(pts[3 * j + 2], g) >> 2;
+  const int32_t c = (int32_t)(((int64_t)bz * g.nbk + by) * g.nbk + bx);
+  bid[j] = c;
   atomicAdd(counts + c, 1);
 }
 
-__global__ void k_point_scatter(const float* __restrict__ pts, int64_t J, const int32_t* __restrict__ cid,
+__global__ void k_point_scatter(const float* __restrict__ pts, int64_t J, const int32_t* __restrict__ bid,
                                 const int32_t* __restrict__ start, int32_t* __restrict__ cursor,
-                                float4* __restrict__ sorted) {
+                                float4* __restrict__ by_block) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= J) return;
-  int32_t c = cid[j];
+  int32_t c = bid[j];
   int32_t pos = start[c] + atomicAdd(cursor + c, 1);
-  sorted[pos] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], __int_as_float((int)j));
+  by_block[pos] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], __int_as_float((int)j));
+}
+
+// A vector of least spread of the points with covariance S (00, 01, 02, 11,
+// 12, 22): cyclic Jacobi rotations (Golub and Van Loan, "Matrix Computations",
+// the two-sided 2 x 2 rotation that zeroes one off-diagonal entry), then the
+// column of the smallest diagonal entry.  Any vector serves: it only shapes
+// bounds and seeds.
+__device__ __forceinline__ void least_spread(const float S[6], float n[3]) {
+  float A[3][3] = {{S[0], S[1], S[2]}, {S[1], S[3], S[4]}, {S[2], S[4], S[5]}};
+  float V[3][3] = {{1.f, 0.f, 0.f}, {0.f, 1.f, 0.f}, {0.f, 0.f, 1.f}};
+  const float scale = fabsf(S[0]) + fabsf(S[3]) + fabsf(S[5]);
+#pragma unroll 1
+  for (int sweep = 0; sweep < 6; ++sweep) {
+#pragma unroll
+    for (int e = 0; e < 3; ++e) {
+      const int p = e == 2 ? 1 : 0, q = e == 0 ? 1 : 2, r = 3 - p - q;
+      const float apq = A[p][q];
+      if (!(fabsf(apq) > 1e-9f * scale)) continue;
+      const float tau = (A[q][q] - A[p][p]) / (2.f * apq);
+      const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+      const float c = rsqrtf(1.f + t * t), s = t * c;
+      A[p][p] -= t * apq;
+      A[q][q] += t * apq;
+      A[p][q] = A[q][p] = 0.f;
+      const float arp = A[r][p], arq = A[r][q];
+      A[r][p] = A[p][r] = c * arp - s * arq;
+      A[r][q] = A[q][r] = s * arp + c * arq;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float vp = V[k][p], vq = V[k][q];
+        V[k][p] = c * vp - s * vq;
+        V[k][q] = s * vp + c * vq;
+      }
+    }
+  }
+  const int m = A[0][0] <= A[1][1] ? (A[0][0] <= A[2][2] ? 0 : 2) : (A[1][1] <= A[2][2] ? 1 : 2);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) n[k] = m == 0 ? V[k][0] : m == 1 ? V[k][1] : V[k][2];
+  const float len = sqrtf(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
+  const float inv = len > 0.5f && len < 2.f ? 1.f / len : 0.f;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) n[k] = inv > 0.f ? n[k] * inv : 0.f;
+}
+
+// A block's 64 cell counts, in shared memory, from its points [first, last).
+__device__ __forceinline__ void block_histogram(const NNGrid& g, const float4* __restrict__ by_block, int first,
+                                                int last, int* cell) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  cell[lane] = 0;
+  cell[lane + 32] = 0;
+  __syncwarp();
+  for (int p = first + lane; p < last; p += 32) atomicAdd(cell + nn_local_cell(by_block[p], g), 1);
+  __syncwarp();
+}
+
+constexpr int NN_BUILD_WARPS = 4;
+enum { NN_C_BLOCKS, NN_C_OCC, NN_C_CHUNKS, NN_C_ALL };
+
+// Each warp takes 32 consecutive blocks of the grid and works through those
+// with points.  Pass 1: gives them their records' numbers and counts their
+// occupied cells (one more each) and chunks.
+__global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_count(NNGrid g, const int32_t* __restrict__ start,
+                                                                     const float4* __restrict__ by_block, int64_t nblk,
+                                                                     int32_t* __restrict__ table,
+                                                                     int32_t* __restrict__ totals) {
+  __shared__ int s_cell[NN_BUILD_WARPS][64];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int64_t b0 = ((int64_t)blockIdx.x * NN_BUILD_WARPS + w) * 32; b0 < nblk;
+       b0 += (int64_t)gridDim.x * NN_BUILD_WARPS * 32) {
+    const int64_t mine = b0 + lane;
+    const int f = mine < nblk ? start[mine] : 0, l = mine < nblk ? start[mine + 1] : 0;
+    const unsigned some = __ballot_sync(0xffffffffu, l > f);
+    int base = 0, occ = 0, chunks = 0;
+    if (lane == 0 && some) base = atomicAdd(totals + NN_C_BLOCKS, __popc(some));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (mine < nblk) table[mine] = l > f ? base + __popc(some & ((1u << lane) - 1u)) : -1;
+    for (unsigned left = some; left; left &= left - 1u) {
+      const int k = __ffs(left) - 1;
+      block_histogram(g, by_block, __shfl_sync(0xffffffffu, f, k), __shfl_sync(0xffffffffu, l, k), s_cell[w]);
+      const int n0 = s_cell[w][lane], n1 = s_cell[w][lane + 32];
+      occ += (n0 > 0) + (n1 > 0) + (lane == 0);
+      chunks += ((n0 + 3) >> 2) + ((n1 + 3) >> 2);
+    }
+    occ = gp_warp_sum_i(occ);
+    chunks = gp_warp_sum_i(chunks);
+    if (lane == 0 && some) {
+      atomicAdd(totals + NN_C_OCC, occ);
+      atomicAdd(totals + NN_C_CHUNKS, chunks);
+    }
+  }
+}
+
+// Pass 2: the chunks of the cells, the first chunk of each occupied cell, the
+// occupancy, and the plane the points lie along.  Blocks with a point outside
+// the grid's cube (kept in the boundary cells) get no plane, so that every
+// coordinate of a bounded block is at most 1.01.
+__global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
+    NNGrid g, const int32_t* __restrict__ start, const float4* __restrict__ by_block, int64_t nblk,
+    const int32_t* __restrict__ table, int32_t* __restrict__ totals, float* __restrict__ pts, int32_t* __restrict__ occ,
+    float4* __restrict__ blk, unsigned long long* __restrict__ sup) {
+  __shared__ int s_cell[NN_BUILD_WARPS][64];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int* cell = s_cell[w];
+  for (int64_t b0 = ((int64_t)blockIdx.x * NN_BUILD_WARPS + w) * 32; b0 < nblk;
+       b0 += (int64_t)gridDim.x * NN_BUILD_WARPS * 32) {
+    const int64_t mine = b0 + lane;
+    const int fl = mine < nblk ? start[mine] : 0, ll = mine < nblk ? start[mine + 1] : 0;
+    for (unsigned left = __ballot_sync(0xffffffffu, ll > fl); left; left &= left - 1u) {
+      const int kb = __ffs(left) - 1;
+      const int first = __shfl_sync(0xffffffffu, fl, kb), last = __shfl_sync(0xffffffffu, ll, kb);
+      const int64_t b = b0 + kb;
+      const int bi = table[b];
+      const int bx = (int)(b % g.nbk), by = (int)((b / g.nbk) % g.nbk), bz = (int)(b / ((int64_t)g.nbk * g.nbk));
+      const float c0 = -1.0f + (4 * bx + 2) * g.cs, c1 = -1.0f + (4 * by + 2) * g.cs, c2 = -1.0f + (4 * bz + 2) * g.cs;
+      block_histogram(g, by_block, first, last, cell);
+      // Exclusive scans of the cells' chunks and occupancy, two consecutive
+      // cells per lane, and the block's share of the arrays.
+      const int n0 = cell[2 * lane], n1 = cell[2 * lane + 1];
+      const int h0 = (n0 + 3) >> 2, h1 = (n1 + 3) >> 2;
+      int incl = h0 + h1;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+      }
+      const unsigned e = __ballot_sync(0xffffffffu, n0 > 0), d = __ballot_sync(0xffffffffu, n1 > 0);
+      const int nocc = __popc(e) + __popc(d);
+      int base = 0, o0 = 0;
+      if (lane == 31) base = atomicAdd(totals + NN_C_CHUNKS, incl);
+      if (lane == 31) o0 = atomicAdd(totals + NN_C_OCC, nocc + 1);
+      base = __shfl_sync(0xffffffffu, base, 31);
+      o0 = __shfl_sync(0xffffffffu, o0, 31);
+      const int at0 = base + incl - h0 - h1, at1 = at0 + h0;
+      const unsigned below = (1u << lane) - 1u;
+      const int k0 = __popc(e & below) + __popc(d & below);
+      if (n0) occ[o0 + k0] = at0;
+      if (n1) occ[o0 + k0 + (n0 > 0)] = at1;
+      if (lane == 31) occ[o0 + nocc] = base + incl;
+      __syncwarp();
+      cell[2 * lane] = 4 * at0;
+      cell[2 * lane + 1] = 4 * at1;
+      __syncwarp();
+      float m[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+      bool inside = true;
+      for (int p = first + lane; p < last; p += 32) {
+        const float4 P = by_block[p];
+        const int at = atomicAdd(cell + nn_local_cell(P, g), 1);
+        const float v[4] = {P.x, P.y, P.z, P.w};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) pts[4 * nn_part(at >> 2, k) + (at & 3)] = v[k];
+        inside = inside && fabsf(P.x) <= 1.01f && fabsf(P.y) <= 1.01f && fabsf(P.z) <= 1.01f;
+        const float x = P.x - c0, y = P.y - c1, z = P.z - c2;
+        m[0] += x;
+        m[1] += y;
+        m[2] += z;
+        m[3] += x * x;
+        m[4] += x * y;
+        m[5] += x * z;
+        m[6] += y * y;
+        m[7] += y * z;
+        m[8] += z * z;
+      }
+      __syncwarp();
+      // The places left in each cell's last chunk.
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int end = 4 * (k ? at1 + h1 : at0 + h0);
+        for (int at = cell[2 * lane + k]; at < end; ++at) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            pts[4 * nn_part(at >> 2, j) + (at & 3)] = j < 3 ? INFINITY : __int_as_float(-1);
+        }
+      }
+      inside = __all_sync(0xffffffffu, inside);
+      float n[3] = {0.f, 0.f, 0.f};
+      if (inside) {
+        const float inv = 1.0f / (float)(last - first);
+#pragma unroll
+        for (int k = 0; k < 9; ++k) m[k] = gp_warp_sum(m[k]) * inv;
+        const float S[6] = {m[3] - m[0] * m[0], m[4] - m[0] * m[1], m[5] - m[0] * m[2],
+                            m[6] - m[1] * m[1], m[7] - m[1] * m[2], m[8] - m[2] * m[2]};
+        least_spread(S, n);
+      }
+      float lo = INFINITY, hi = -INFINITY;
+      for (int p = first + lane; p < last; p += 32) {
+        const float4 P = by_block[p];
+        const float v = n[0] * P.x + n[1] * P.y + n[2] * P.z;
+        lo = fminf(lo, v);
+        hi = fmaxf(hi, v);
+      }
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, k));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, k));
+      }
+      if (lane == 0) {
+        if (!inside) lo = hi = 0.f;
+        unsigned long long mask = 0ull;
+        for (int k = 0; k < 32; ++k)
+          mask |= ((unsigned long long)((e >> k) & 1u) | ((unsigned long long)((d >> k) & 1u) << 1)) << (2 * k);
+        blk[2 * (int64_t)bi] = make_float4(n[0], n[1], n[2], lo);
+        blk[2 * (int64_t)bi + 1] = make_float4(hi, __int_as_float(o0), __uint_as_float((uint32_t)mask),
+                                               __uint_as_float((uint32_t)(mask >> 32)));
+        atomicOr(sup + ((int64_t)(bz >> 2) * g.nsup + (by >> 2)) * g.nsup + (bx >> 2),
+                 1ull << ((bx & 3) | ((by & 3) << 2) | ((bz & 3) << 4)));
+      }
+    }
+  }
 }
 
 // sigma_j: distance to the k-th nearest other point, by a bounded max-heap.
-__global__ void __launch_bounds__(128) k_knn_sigma(NNGrid g, int64_t J, int k, float* __restrict__ sigma) {
+__global__ void __launch_bounds__(128) k_knn_sigma(NNGrid g, int64_t chunks, int k, float* __restrict__ sigma) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= J) return;
-  float4 me = g.pts[t];
-  int self = __float_as_int(me.w);
+  if (t >= 4 * chunks) return;
+  const int self = __float_as_int(nn_value(g.pts, t, 3));
+  if (self < 0) return;
   float heap[64];
   int cnt = 0;
   if (k <= 0) {
     sigma[self] = 0.f;
     return;
   }
-  float q[3] = {me.x, me.y, me.z};
+  float q[3] = {nn_value(g.pts, t, 0), nn_value(g.pts, t, 1), nn_value(g.pts, t, 2)};
   int c[3] = {nn_cell(q[0], g), nn_cell(q[1], g), nn_cell(q[2], g)};
   float margin = nn_margin(q);
+  const int64_t me = t;
   for (int r = 0; r <= g.G; ++r) {
     nn_ring(c, r, g, [&](int a, int b) {
-      for (int p = a; p < b; ++p) {
-        float4 P = g.pts[p];
-        if (__float_as_int(P.w) == self) continue;
-        float dx = q[0] - P.x, dy = q[1] - P.y, dz = q[2] - P.z;
+      for (int64_t p = 4 * (int64_t)a; p < 4 * (int64_t)b; ++p) {
+        if (p == me || __float_as_int(nn_value(g.pts, p, 3)) < 0) continue;
+        float dx = q[0] - nn_value(g.pts, p, 0), dy = q[1] - nn_value(g.pts, p, 1), dz = q[2] - nn_value(g.pts, p, 2);
         float d = dx * dx + dy * dy + dz * dz;
         if (cnt < k) {
           // sift up
@@ -107,245 +320,116 @@ __global__ void __launch_bounds__(128) k_knn_sigma(NNGrid g, int64_t J, int k, f
   sigma[self] = cnt > 0 ? sqrtf(heap[0]) : 0.f;
 }
 
-// Smallest-eigenvalue eigenvector of a symmetric 3x3 matrix (Smith, "Eigenvalues
-// of a symmetric 3x3 matrix", CACM 1961: the characteristic cubic solved by
-// trigonometry), then a null vector of A - l I from the largest cross product
-// of its rows.  Returns false when the matrix is (nearly) isotropic.
-__device__ bool smallest_eigvec(const double A[6], double v[3]) {
-  // A = [a00 a01 a02; . a11 a12; . . a22] packed as a00, a01, a02, a11, a12, a22
-  const double a00 = A[0], a01 = A[1], a02 = A[2], a11 = A[3], a12 = A[4], a22 = A[5];
-  const double p1 = a01 * a01 + a02 * a02 + a12 * a12;
-  const double qm = (a00 + a11 + a22) / 3.0;
-  const double p2 = (a00 - qm) * (a00 - qm) + (a11 - qm) * (a11 - qm) + (a22 - qm) * (a22 - qm) + 2.0 * p1;
-  if (!(p2 > 1e-300)) return false;
-  const double p = sqrt(p2 / 6.0);
-  const double b00 = (a00 - qm) / p, b11 = (a11 - qm) / p, b22 = (a22 - qm) / p;
-  const double b01 = a01 / p, b02 = a02 / p, b12 = a12 / p;
-  double r = 0.5 * (b00 * (b11 * b22 - b12 * b12) - b01 * (b01 * b22 - b12 * b02) + b02 * (b01 * b12 - b11 * b02));
-  r = fmin(1.0, fmax(-1.0, r));
-  const double phi = acos(r) / 3.0;
-  const double lmin = qm + 2.0 * p * cos(phi + 2.0943951023931954923);  // + 2 pi / 3
-  const double r0[3] = {a00 - lmin, a01, a02}, r1[3] = {a01, a11 - lmin, a12}, r2[3] = {a02, a12, a22 - lmin};
-  double c[3][3] = {{r0[1] * r1[2] - r0[2] * r1[1], r0[2] * r1[0] - r0[0] * r1[2], r0[0] * r1[1] - r0[1] * r1[0]},
-                    {r0[1] * r2[2] - r0[2] * r2[1], r0[2] * r2[0] - r0[0] * r2[2], r0[0] * r2[1] - r0[1] * r2[0]},
-                    {r1[1] * r2[2] - r1[2] * r2[1], r1[2] * r2[0] - r1[0] * r2[2], r1[0] * r2[1] - r1[1] * r2[0]}};
-  int best = 0;
-  double bn = -1.0;
-  for (int k = 0; k < 3; ++k) {
-    double nk = c[k][0] * c[k][0] + c[k][1] * c[k][1] + c[k][2] * c[k][2];
-    if (nk > bn) {
-      bn = nk;
-      best = k;
-    }
-  }
-  if (!(bn > 1e-300)) return false;
-  const double inv = 1.0 / sqrt(bn);
-  v[0] = c[best][0] * inv;
-  v[1] = c[best][1] * inv;
-  v[2] = c[best][2] * inv;
-  return true;
-}
-
 // Normal of each point: direction of least spread of the points within
-// sigma_j (its k-nearest-neighbour ball), by PCA.  Used only to seed gp_nn.
-__global__ void __launch_bounds__(128) k_normals(NNGrid g, int64_t J, const float* __restrict__ sigma,
-                                                 float* __restrict__ normals) {
+// sigma_j (its k-nearest-neighbour ball), by PCA.  Used only to seed gp_nn:
+// written with the point, packed, as its record of `seeds`.
+__global__ void __launch_bounds__(128) k_normals(NNGrid g, int64_t chunks, const float* __restrict__ sigma,
+                                                 float4* __restrict__ seeds) {
   int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= J) return;
-  const float4 me = g.pts[t];
-  const int self = __float_as_int(me.w);
-  const float q[3] = {me.x, me.y, me.z};
+  if (t >= 4 * chunks) return;
+  const int self = __float_as_int(nn_value(g.pts, t, 3));
+  if (self < 0) return;
+  const float q[3] = {nn_value(g.pts, t, 0), nn_value(g.pts, t, 1), nn_value(g.pts, t, 2)};
   const int c[3] = {nn_cell(q[0], g), nn_cell(q[1], g), nn_cell(q[2], g)};
   const float rad = sigma[self];
   const float r2 = rad * rad * 1.000001f;
   const float margin = nn_margin(q);
-  double m[3] = {0, 0, 0}, S[6] = {0, 0, 0, 0, 0, 0};
+  float m[3] = {0, 0, 0}, S[6] = {0, 0, 0, 0, 0, 0};
   int cnt = 0;
   for (int r = 0; r <= g.G; ++r) {
     nn_ring(c, r, g, [&](int a, int b) {
-      for (int p = a; p < b; ++p) {
-        float4 P = g.pts[p];
-        float dx = P.x - q[0], dy = P.y - q[1], dz = P.z - q[2];
+      for (int64_t p = 4 * (int64_t)a; p < 4 * (int64_t)b; ++p) {
+        float dx = nn_value(g.pts, p, 0) - q[0], dy = nn_value(g.pts, p, 1) - q[1], dz = nn_value(g.pts, p, 2) - q[2];
         if (dx * dx + dy * dy + dz * dz > r2) continue;
         m[0] += dx;
         m[1] += dy;
         m[2] += dz;
-        S[0] += (double)dx * dx;
-        S[1] += (double)dx * dy;
-        S[2] += (double)dx * dz;
-        S[3] += (double)dy * dy;
-        S[4] += (double)dy * dz;
-        S[5] += (double)dz * dz;
+        S[0] += dx * dx;
+        S[1] += dx * dy;
+        S[2] += dx * dz;
+        S[3] += dy * dy;
+        S[4] += dy * dz;
+        S[5] += dz * dz;
         ++cnt;
       }
     });
     float gap = nn_gap(q, c, r, g);
     if (gap == INFINITY || gap - margin > rad) break;
   }
-  float nv[3] = {0.f, 0.f, 0.f};
+  float n[3] = {0.f, 0.f, 0.f};
   if (cnt >= 3) {
-    for (int a = 0; a < 3; ++a) m[a] /= cnt;
-    double C[6] = {S[0] / cnt - m[0] * m[0], S[1] / cnt - m[0] * m[1], S[2] / cnt - m[0] * m[2],
-                   S[3] / cnt - m[1] * m[1], S[4] / cnt - m[1] * m[2], S[5] / cnt - m[2] * m[2]};
-    double v[3];
-    if (smallest_eigvec(C, v)) {
-      nv[0] = (float)v[0];
-      nv[1] = (float)v[1];
-      nv[2] = (float)v[2];
-    }
+    const float inv = 1.0f / (float)cnt;
+    for (int a = 0; a < 3; ++a) m[a] *= inv;
+    const float C[6] = {S[0] * inv - m[0] * m[0], S[1] * inv - m[0] * m[1], S[2] * inv - m[0] * m[2],
+                        S[3] * inv - m[1] * m[1], S[4] * inv - m[1] * m[2], S[5] * inv - m[2] * m[2]};
+    least_spread(C, n);
   }
-  normals[3 * (int64_t)self + 0] = nv[0];
-  normals[3 * (int64_t)self + 1] = nv[1];
-  normals[3 * (int64_t)self + 2] = nv[2];
+  seeds[self] = make_float4(q[0], q[1], q[2], __int_as_float(nn_pack_normal(n[0], n[1], n[2])));
 }
 
-__device__ __forceinline__ void nn_add_work(unsigned long long* total, int v) {
-  unsigned long long w = (unsigned long long)v;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
-  if ((threadIdx.x & 31) == 0 && w) atomicAdd(total, w);
+// Records of a cloud without normals: the points themselves.
+__global__ void k_seed_points(const float* __restrict__ pts, int64_t J, float4* __restrict__ seeds) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < J) seeds[j] = make_float4(pts[3 * j], pts[3 * j + 1], pts[3 * j + 2], 0.f);
 }
 
-// One thread per query.  Queries with a NaN, infinite or huge coordinate (whose
-// squared distances would overflow float32) get -1 and a NaN surface point.
-#ifndef GP_NN_BLOCK
-#define GP_NN_BLOCK 256
-#endif
-#ifdef GP_NN_MIN_BLOCKS
-#define GP_NN_BOUNDS __launch_bounds__(GP_NN_BLOCK, GP_NN_MIN_BLOCKS)
-#else
-#define GP_NN_BOUNDS __launch_bounds__(GP_NN_BLOCK)
-#endif
-// COUNT: also add the number of point distances evaluated (seeds, walk and
+// Four warps a block, 8 blocks an SM at 64 registers; 64 or 256 threads, and
+// 10 blocks an SM at fewer registers, were within 2% on every batch measured.
+constexpr int NN_THREADS = 128;
+
+// One lane per query (nn_search works on a warp's 32 together).  Queries with a
+// NaN, infinite or huge coordinate (whose squared distances would overflow
+// float32) get -1 and a NaN surface point.  COUNT: also add the number of point distances evaluated (seeds, cells and
 // tie-break) to *work_total, for measurement; the search is the same.
 template <bool COUNT>
-__global__ void GP_NN_BOUNDS k_nn(NNGrid g, const float* __restrict__ qin, int64_t n,
-                                            const int32_t* __restrict__ hint, int64_t J,
-                                            const float* __restrict__ pts_orig, int32_t* __restrict__ nn_out,
-                                            float* __restrict__ rec, Grid band, int32_t* __restrict__ nvalid,
-                                            const float* __restrict__ normals,
-                                            unsigned long long* __restrict__ work_total) {
-  int work_v = 0;
-  int* work = COUNT ? &work_v : nullptr;
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const bool active = i < n;
-  float q[3] = {0.f, 0.f, 0.f};
-  if (active) {
+__global__ void __launch_bounds__(NN_THREADS, 8) k_nn(NNGrid g, const float* __restrict__ qin, int64_t n,
+                                                      const int32_t* __restrict__ hint, int64_t J,
+                                                      const float4* __restrict__ seeds, int32_t* __restrict__ nn_out,
+                                                      float* __restrict__ rec, Grid band, int32_t* __restrict__ nvalid,
+                                                      unsigned long long* __restrict__ work_total) {
+  __shared__ NNWarp s_warp[NN_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t first = (int64_t)blockIdx.x * NN_THREADS + 32 * warp;
+  const int64_t i = first + lane;
+  const float nan = __int_as_float(0x7fc00000);
+  float q[3] = {nan, nan, nan}, s[3] = {nan, nan, nan};
+  int h = -1;
+  if (i < n) {
     q[0] = qin[3 * i];
     q[1] = qin[3 * i + 1];
     q[2] = qin[3 * i + 2];
+    if (hint) h = __ldg(hint + i);
   }
-  const bool ok = active && nn_query_ok(q);
-  int c[3] = {0, 0, 0};
-  float margin = 0.f;
-  NNState st{INFINITY, INFINITY, INFINITY, 0x7fffffff};
-  if (ok) {
-    c[0] = nn_cell(q[0], g);
-    c[1] = nn_cell(q[1], g);
-    c[2] = nn_cell(q[2], g);
-    margin = nn_margin(q);
-    nn_seed(st, q, hint, i, J, pts_orig);
-    if (COUNT && st.b1 < INFINITY) ++work_v;
-    if (st.b1 < INFINITY) nn_seed_foot(st, q, hint, i, J, pts_orig, normals, g, work);
+  int work = 0;
+  const int best = nn_search<COUNT>(q, nn_query_ok(q), h, J, seeds, g, s_warp[warp], s, work);
+  if (nn_out && i < n) nn_out[i] = best;
+  if (nvalid) {
+    Cells C;
+    const unsigned v = __ballot_sync(0xffffffffu, best >= 0 && classify(band, q, s, C));
+    if (lane == 0 && v) atomicAdd(nvalid, __popc(v));
   }
-  int best = -1;
-  if (ok) best = nn_thread_search(q, c, g, margin, st, work);
-  if (active) nn_finish(i, q, best, pts_orig, nn_out, rec, band, nvalid);
-  if (COUNT) nn_add_work(work_total, work_v);
-}
-
-// The same search for large seeded batches.  Each thread first seeds its own query; the block then sorts its queries (in
-// segments of NN_SPAN), stably, by the seeded radius (a counting sort on thr in
-// quarters of the squared cell size: the walk visits about thr / cs^2 rows),
-// and every thread searches the query of its rank, so that the lanes of a warp
-// have walks of similar length while queries of equal key keep their spatial
-// order.  Which thread searches a query does not change its result.
-// Measured on GB300: 18% faster than k_nn on the 4,194,304-query superquadric
-// batch and 10% on the 2,097,152-query scene batch, 6-10% slower on the
-// 262,144-query single-object batch, hence NN_SORTED_MIN_QUERIES.  Blocks of
-// 128 (sorted together) beat 256 by 4% on the scene: a block's slot is held
-// until its slowest warp ends, and smaller blocks leave shorter tails; 64
-// or a 64-query sort span lose more than that.
-constexpr int NN_THREADS = 128;
-constexpr int NN_SPAN = 128;  // queries sorted together (a multiple of 32 dividing NN_THREADS)
-constexpr int NN_SEGS = NN_THREADS / NN_SPAN;
-constexpr int NN_SPAN_WARPS = NN_SPAN / 32;
-constexpr int NN_BUCKETS = 16;
-constexpr int64_t NN_SORTED_MIN_QUERIES = int64_t(1) << 20;
-static_assert(NN_SPAN % 32 == 0 && NN_THREADS % NN_SPAN == 0, "sort span");
-
-template <bool COUNT>
-__global__ void __launch_bounds__(NN_THREADS) k_nn_sorted(NNGrid g, const float* __restrict__ qin, int64_t n,
-                                                   const int32_t* __restrict__ hint, int64_t J,
-                                                   const float* __restrict__ pts_orig, int32_t* __restrict__ nn_out,
-                                                   float* __restrict__ rec, Grid band, int32_t* __restrict__ nvalid,
-                                                   const float* __restrict__ normals,
-                                                   unsigned long long* __restrict__ work_total) {
-  int work_v = 0;
-  int* work = COUNT ? &work_v : nullptr;
-  __shared__ int s_off[NN_SEGS][NN_BUCKETS][NN_SPAN_WARPS];  // count, then first rank in the segment
-  __shared__ float4 s_q[NN_THREADS];   // q, and the query's offset in the block (int bits; -1 - offset if invalid)
-  __shared__ float4 s_st[NN_THREADS];  // b1, b2, thr, j1 (int bits)
-  const int t = threadIdx.x, lane = t & 31, seg = t / NN_SPAN, wseg = (t % NN_SPAN) >> 5;
-  const int64_t base = (int64_t)blockIdx.x * NN_THREADS;
-  int64_t i = base + t;
-  const bool active = i < n;
-  float q[3] = {0.f, 0.f, 0.f};
-  if (active) {
-    q[0] = qin[3 * i];
-    q[1] = qin[3 * i + 1];
-    q[2] = qin[3 * i + 2];
-  }
-  bool ok = active && nn_query_ok(q);
-  NNState st{INFINITY, INFINITY, INFINITY, 0x7fffffff};
-  int key = 0;
-  if (ok) {
-    nn_seed(st, q, hint, i, J, pts_orig);
-    if (COUNT && st.b1 < INFINITY) ++work_v;
-    if (st.b1 < INFINITY) {
-      nn_seed_foot(st, q, hint, i, J, pts_orig, normals, g, work);
-      key = (int)fminf(4.0f * st.thr / (g.cs * g.cs), (float)(NN_BUCKETS - 2));
-    } else {
-      key = NN_BUCKETS - 1;  // unseeded: the ring search
+  if (rec) {
+    // Through shared memory, so that the warp's records are written in lines.
+    float* out = reinterpret_cast<float*>(&s_warp[warp]);
+    static_assert(sizeof(NNWarp) >= 32 * 6 * sizeof(float), "record staging");
+    __syncwarp();
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      out[6 * lane + a] = q[a];
+      out[6 * lane + 3 + a] = s[a];
     }
+    __syncwarp();
+    const int64_t left = 6 * (n - first);
+#pragma unroll
+    for (int k = lane; k < 32 * 6; k += 32)
+      if (k < left) rec[6 * first + k] = out[k];
   }
-  // Stable counting sort within each segment of NN_SPAN queries:
-  // rank = (smaller key) + (same key, lower warp) + (same key, lower lane).
-  const unsigned peers = __match_any_sync(0xffffffffu, key);
-  const int in_warp = __popc(peers & ((1u << lane) - 1u));
-  for (int k = t; k < NN_SEGS * NN_BUCKETS * NN_SPAN_WARPS; k += NN_THREADS) (&s_off[0][0][0])[k] = 0;
-  __syncthreads();
-  if (in_warp == 0) s_off[seg][key][wseg] = __popc(peers);
-  __syncthreads();
-  if (t < NN_SEGS) {
-    int run = 0;
-    for (int b = 0; b < NN_BUCKETS; ++b)
-      for (int w = 0; w < NN_SPAN_WARPS; ++w) {
-        const int c = s_off[t][b][w];
-        s_off[t][b][w] = run;
-        run += c;
-      }
+  if (COUNT) {
+    unsigned long long w = (unsigned long long)work;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+    if (lane == 0 && w) atomicAdd(work_total, w);
   }
-  __syncthreads();
-  const int rank = seg * NN_SPAN + s_off[seg][key][wseg] + in_warp;
-  s_q[rank] = make_float4(q[0], q[1], q[2], __int_as_float(ok ? t : -1 - t));
-  s_st[rank] = make_float4(st.b1, st.b2, st.thr, __int_as_float(st.j1));
-  __syncthreads();
-  const float4 mq = s_q[t], ms = s_st[t];
-  const int off = __float_as_int(mq.w);
-  ok = off >= 0;
-  i = base + (ok ? off : -1 - off);
-  q[0] = mq.x;
-  q[1] = mq.y;
-  q[2] = mq.z;
-  st = NNState{ms.x, ms.y, ms.z, __float_as_int(ms.w)};
-  int best = -1;
-  if (ok) {
-    const int c[3] = {nn_cell(q[0], g), nn_cell(q[1], g), nn_cell(q[2], g)};
-    best = nn_thread_search(q, c, g, nn_margin(q), st, work);
-  }
-  if (i < n) nn_finish(i, q, best, pts_orig, nn_out, rec, band, nvalid);
-  if (COUNT) nn_add_work(work_total, work_v);
 }
 
 // Points and sigma in emission order, for the sampler's coalesced reads.
@@ -409,9 +493,9 @@ gp_status gp_build_points(gp_band* b, const float* pts_dev) {
   cudaStream_t s = ctx->stream;
   const int64_t J = b->J;
   if (b->G <= 0) {
-    // About 6.5 points per occupied cell of the search grid, the measured
-    // optimum (4.9 to 8 points per cell were within 1-3% on the benchmark
-    // clouds).  The cloud is a surface, so the cells it occupies at grid G are
+    // About 6.5 points per occupied cell of the search grid (5 to 10 are within
+    // 5% of one another on the benchmark clouds, 3 and 14 up to 25% slower).
+    // The cloud is a surface, so the cells it occupies at grid G are
     // about n_occ (G / R)^2, n_occ being its occupied cells at the band's R.
     // That estimate fails for a cloud too sparse to cover its surface at R
     // (n_occ near J); there sqrt(J / 3) cells per axis, the bound that served
@@ -423,38 +507,64 @@ gp_status gp_build_points(gp_band* b, const float* pts_dev) {
     b->G = std::min(std::max(G, 4), 512);
   }
   const int G = b->G;
-  const int64_t ncell = (int64_t)G * G * G;
+  const int nbk = (G + 3) / 4, nsup = (G + 15) / 16;
+  const int64_t nblk = (int64_t)nbk * nbk * nbk, nsb = (int64_t)nsup * nsup * nsup;
   gp_status st;
   if ((st = gp_alloc(ctx, &b->pts, 3 * J, "points"))) return st;
   GP_CUDA(ctx, cudaMemcpyAsync(b->pts, pts_dev, 3 * J * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  if ((st = gp_alloc(ctx, &b->pts_sorted, J, "sorted points"))) return st;
-  if ((st = gp_alloc(ctx, &b->cell_start, ncell + 1, "cell starts"))) return st;
-  int32_t *cid = nullptr, *cursor = nullptr;
-  if ((st = gp_alloc(ctx, &cid, J, "point cells"))) return st;
-  if ((st = gp_alloc(ctx, &cursor, ncell, "cell cursor"))) {
-    cudaFree(cid);
-    return st;
-  }
+  if ((st = gp_alloc(ctx, &b->cell_table, nblk, "cell blocks"))) return st;
+  if ((st = gp_alloc(ctx, &b->cell_sup, nsb, "cell super-blocks"))) return st;
+  if ((st = gp_alloc(ctx, &b->seeds, J, "search seeds"))) return st;
+  int32_t *bid = nullptr, *start = nullptr, *cursor = nullptr;  // the block totals follow the cursors
+  float4* by_block = nullptr;
+  st = gp_alloc(ctx, &bid, J, "point blocks");
+  if (!st) st = gp_alloc(ctx, &start, nblk + 1, "block starts");
+  if (!st) st = gp_alloc(ctx, &cursor, nblk + NN_C_ALL, "block cursors");
+  if (!st) st = gp_alloc(ctx, &by_block, J, "points by block");
+  cudaError_t e = cudaSuccess;
   NNGrid g = make_grid(b);
-  cudaError_t e = cudaMemsetAsync(b->cell_start, 0, (ncell + 1) * sizeof(int32_t), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, ncell * sizeof(int32_t), s);
-  if (e == cudaSuccess) {
-    k_point_cells<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, g, cid, b->cell_start);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    int64_t total = 0;
-    st = gp_exclusive_scan_i32(ctx, b->cell_start, ncell + 1, &total);
-    if (!st) {
-      k_point_scatter<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, cid, b->cell_start, cursor, b->pts_sorted);
+  if (!st) {
+    e = cudaMemsetAsync(start, 0, (nblk + 1) * sizeof(int32_t), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(cursor, 0, (nblk + NN_C_ALL) * sizeof(int32_t), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->cell_sup, 0, nsb * sizeof(unsigned long long), s);
+    if (e == cudaSuccess) {
+      k_point_blocks<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, g, bid, start);
       e = cudaGetLastError();
     }
   }
+  int64_t total = 0;
+  int32_t totals[NN_C_ALL] = {0, 0, 0};
+  if (!st && e == cudaSuccess) st = gp_exclusive_scan_i32(ctx, start, nblk + 1, &total);
+  const unsigned grid = gp_blocks(nblk, 32 * NN_BUILD_WARPS, 16 * (int64_t)ctx->num_sms);
+  int32_t* tot_dev = cursor ? cursor + nblk : nullptr;
+  if (!st && e == cudaSuccess) {
+    k_point_scatter<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, bid, start, cursor, by_block);
+    k_block_count<<<grid, 32 * NN_BUILD_WARPS, 0, s>>>(g, start, by_block, nblk, b->cell_table, tot_dev);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(totals, tot_dev, sizeof(totals), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(tot_dev, 0, sizeof(totals), s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  }
+  b->n_chunks = totals[NN_C_CHUNKS];
+  if (!st && e == cudaSuccess) st = gp_alloc(ctx, &b->cell_blk, 2 * (size_t)totals[NN_C_BLOCKS], "cell block records");
+  if (!st && e == cudaSuccess) st = gp_alloc(ctx, &b->cell_occ, totals[NN_C_OCC], "occupied cells");
+  if (!st && e == cudaSuccess) st = gp_alloc(ctx, &b->pts_sorted, 4 * (size_t)b->n_chunks, "sorted points");
+  if (!st && e == cudaSuccess) {
+    k_block_build<<<grid, 32 * NN_BUILD_WARPS, 0, s>>>(g, start, by_block, nblk, b->cell_table, tot_dev,
+                                                       reinterpret_cast<float*>(b->pts_sorted), b->cell_occ,
+                                                       b->cell_blk, b->cell_sup);
+    e = cudaGetLastError();
+  }
   cudaStreamSynchronize(s);
-  cudaFree(cid);
-  cudaFree(cursor);
+  gp_free(bid);
+  gp_free(start);
+  gp_free(cursor);
+  gp_free(by_block);
   if (st) return st;
   if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "point cell list");
+  g = make_grid(b);
+  if (b->knn_k == 0)
+    GP_KERNEL(ctx, "k_seed_points", k_seed_points<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, b->seeds));
   if (b->knn_k > 0) {
     if ((st = gp_alloc(ctx, &b->sigma, J, "sigma"))) return st;
     if ((st = gp_alloc(ctx, &b->perm, J, "permutation"))) return st;
@@ -463,9 +573,8 @@ gp_status gp_build_points(gp_band* b, const float* pts_dev) {
     if ((st = build_emit_order(b))) return st;
     if ((st = gp_alloc(ctx, &b->emit_slot, J, "emission slots"))) return st;
     int k = (int)std::min<int64_t>(b->knn_k, J - 1);
-    GP_KERNEL(ctx, "k_knn_sigma", k_knn_sigma<<<gp_blocks(J, 128), 128, 0, s>>>(g, J, k, b->sigma));
-    if ((st = gp_alloc(ctx, &b->normals, 3 * J, "normals"))) return st;
-    GP_KERNEL(ctx, "k_normals", k_normals<<<gp_blocks(J, 128), 128, 0, s>>>(g, J, b->sigma, b->normals));
+    GP_KERNEL(ctx, "k_knn_sigma", k_knn_sigma<<<gp_blocks(4 * b->n_chunks, 128), 128, 0, s>>>(g, b->n_chunks, k, b->sigma));
+    GP_KERNEL(ctx, "k_normals", k_normals<<<gp_blocks(4 * b->n_chunks, 128), 128, 0, s>>>(g, b->n_chunks, b->sigma, b->seeds));
     if ((st = gp_alloc(ctx, &b->emit_pts, J, "emission points"))) return st;
     GP_KERNEL(ctx, "k_emit_pts", k_emit_pts<<<gp_blocks(J, 256), 256, 0, s>>>(b->emit_order, b->pts, b->sigma, J,
                                                                             b->emit_pts));
@@ -495,25 +604,17 @@ static gp_status nn_launch(gp_band* b, const float* q_dev, int64_t n, const int3
   band.nb = b->nb;
   band.R = b->R;
   band.half_r = 0.5f * (float)b->R;
-  if (hint_dev && n >= NN_SORTED_MIN_QUERIES) {
-    if (work_total)
-      GP_KERNEL(ctx, "k_nn_sorted_count",
-                k_nn_sorted<true><<<gp_blocks(n, NN_THREADS), NN_THREADS, 0, ctx->stream>>>(
-                    g, q_dev, n, hint_dev, b->J, b->pts, nn_dev, rec_dev, band, nvalid_dev, b->normals, work_total));
-    else
-      GP_KERNEL(ctx, "k_nn_sorted",
-                k_nn_sorted<false><<<gp_blocks(n, NN_THREADS), NN_THREADS, 0, ctx->stream>>>(
-                    g, q_dev, n, hint_dev, b->J, b->pts, nn_dev, rec_dev, band, nvalid_dev, b->normals, nullptr));
-    return GP_OK;
-  }
+#define GP_NN(C_) \
+  k_nn<C_><<<gp_blocks(n, NN_THREADS), NN_THREADS, 0, ctx->stream>>>(g, q_dev, n, hint_dev, b->J, b->seeds, nn_dev, \
+                                                                     rec_dev, band, nvalid_dev, work_total)
+  // Large seeded batches are traced under a name of their own.
   if (work_total)
-    GP_KERNEL(ctx, "k_nn_count",
-              k_nn<true><<<gp_blocks(n, GP_NN_BLOCK), GP_NN_BLOCK, 0, ctx->stream>>>(
-                  g, q_dev, n, hint_dev, b->J, b->pts, nn_dev, rec_dev, band, nvalid_dev, b->normals, work_total));
+    GP_KERNEL(ctx, "k_nn_count", GP_NN(true));
+  else if (hint_dev && n >= (int64_t(1) << 20))
+    GP_KERNEL(ctx, "k_nn_sorted", GP_NN(false));
   else
-    GP_KERNEL(ctx, "k_nn",
-              k_nn<false><<<gp_blocks(n, GP_NN_BLOCK), GP_NN_BLOCK, 0, ctx->stream>>>(
-                  g, q_dev, n, hint_dev, b->J, b->pts, nn_dev, rec_dev, band, nvalid_dev, b->normals, nullptr));
+    GP_KERNEL(ctx, "k_nn", GP_NN(false));
+#undef GP_NN
   return GP_OK;
 }
 

@@ -1,7 +1,7 @@
 // Device side of the exact nearest-point search (shared by gp_nn.cu and
-// gp_multi.cu): the uniform cell list, the float32 screen with its proven
-// margins, the seeded ball walk, the ring search for unseeded queries and the
-// float64 tie-break.  The exactness argument is in the header of gp_nn.cu.
+// gp_multi.cu): the cell list with its block bounds, the float32 screen with
+// its proven margins, the search of one query by one thread and the float64
+// tie-break.  The exactness argument is in the header of gp_nn.cu.
 #pragma once
 
 #include <math.h>
@@ -11,10 +11,33 @@
 constexpr float NN_EPS = 3.814697265625e-06f;  // 2^-18
 constexpr float NN_TINY = 1e-30f;
 
+// The cloud in a uniform grid of G^3 cells, grouped into blocks of 4^3 cells
+// and super-blocks of 4^3 blocks.  Only what holds points is stored.
+//
+// The points of a cell lie in chunks of four, 64 bytes each: (x0..x3),
+// (y0..y3), (z0..z3) and the four original indices; the last chunk of a cell
+// is filled up with points at infinity (index -1), whose distance +inf never
+// compares below another.  A chunk is three 16-byte loads, and its four
+// distances twelve two-wide float32 instructions (four 16-byte loads and 24
+// instructions with the points as records of four floats).  The parts are
+// rotated by the chunk's number (nn_part), so that lanes reading the same part
+// of chunks anywhere spread over the banks: 1,500,001 queries among 2 M points
+// take 491 us, 520 us in a fixed order.
+//
+// A block with points has a record of two float4,
+//   (n.x, n.y, n.z, lo), (hi, first occupied cell, occupancy mask: 2 words),
+// the plane n . p in [lo, hi] holding for every point p of the block (n a unit
+// vector, the normal of the block's best plane, or 0 with lo = hi = 0), bit
+// 16 z + 4 y + x of the mask telling whether that cell of the block holds
+// points.  The k-th occupied cell's chunks are occ[first + k] up to
+// occ[first + k + 1].
 struct NNGrid {
-  const float4* __restrict__ pts;      // sorted by cell: x, y, z, original index bits
-  const int32_t* __restrict__ start;   // G^3 + 1
-  int G;
+  const float4* __restrict__ pts;     // 4 per chunk
+  const int32_t* __restrict__ occ;    // first chunk of each occupied cell, one more entry per block
+  const float4* __restrict__ blk;     // the records of the blocks with points
+  const int32_t* __restrict__ table;  // nbk^3: record of the block, -1 where it holds no point
+  const unsigned long long* __restrict__ sup;  // nsup^3: which blocks of a super-block hold points
+  int G, nbk, nsup;
   float half_g;  // G / 2
   float cs;      // 2 / G
 };
@@ -43,365 +66,585 @@ __device__ __forceinline__ float nn_gap(const float q[3], const int c[3], int r,
   return gap;
 }
 
-// sqrt(x) for the x-range of a row, as x rsqrt(x): within a relative 3e-7
-// of the correctly rounded root, which the range's factor 1.000001 and its
-// additive margin (>= 2e-5) cover.  0 for x <= 0.
-__device__ __forceinline__ float nn_row_sqrt(float x) { return x > 0.f ? x * rsqrtf(x) : 0.f; }
+// sqrt(max(x, 0)) in one instruction: within a relative 1e-6 of the root, which
+// the factor 1.000001 and the additive margin (>= 2e-5) wherever it is used as
+// a radius cover.
+__device__ __forceinline__ float nn_root(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(x, 0.f)));
+  return r;
+}
 
 __device__ __forceinline__ float nn_margin(const float q[3]) {
   float m = fmaxf(fabsf(q[0]), fmaxf(fabsf(q[1]), fabsf(q[2])));
   return 1e-5f * (2.0f + m);
 }
 
-// Visit every cell of ring r (Chebyshev shell) as contiguous point ranges.
-template <typename F>
-__device__ __forceinline__ void nn_ring(const int c[3], int r, const NNGrid& g, F&& visit) {
-  const int G = g.G;
-  for (int dz = -r; dz <= r; ++dz) {
-    int cz = c[2] + dz;
-    if (cz < 0 || cz >= G) continue;
-    for (int dy = -r; dy <= r; ++dy) {
-      int cy = c[1] + dy;
-      if (cy < 0 || cy >= G) continue;
-      int64_t row = ((int64_t)cz * G + cy) * G;
-      bool full = (dz == -r || dz == r || dy == -r || dy == r);
-      if (full) {
-        int x0 = max(c[0] - r, 0), x1 = min(c[0] + r, G - 1);
-        visit(__ldg(g.start + row + x0), __ldg(g.start + row + x1 + 1));
-      } else {
-        int xa = c[0] - r, xb = c[0] + r;
-        if (xa >= 0) visit(__ldg(g.start + row + xa), __ldg(g.start + row + xa + 1));
-        if (xb < G) visit(__ldg(g.start + row + xb), __ldg(g.start + row + xb + 1));
-      }
-    }
-  }
-}
-
-__device__ __forceinline__ double nn_d64(const float q[3], float4 p) {
-  double dx = __dsub_rn((double)q[0], (double)p.x);
-  double dy = __dsub_rn((double)q[1], (double)p.y);
-  double dz = __dsub_rn((double)q[2], (double)p.z);
+__device__ __forceinline__ double nn_d64(const float q[3], float x, float y, float z) {
+  double dx = __dsub_rn((double)q[0], (double)x);
+  double dy = __dsub_rn((double)q[1], (double)y);
+  double dz = __dsub_rn((double)q[2], (double)z);
   return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
 }
 
-// Lower bound on |p_a - q_a| for any point p in cell `ca` along one axis
-// (edge cells extend to infinity outwards); the margin absorbs the rounding of
-// the point-to-cell assignment and of the cell faces.
-__device__ __forceinline__ float nn_axis_gap(float qa, int ca, const NNGrid& g, float margin) {
-  float lo = -1.0f + (float)ca * g.cs, hi = lo + g.cs;
+// The float32 distance of the screen, in the order of the two-wide form.
+__device__ __forceinline__ float nn_d32(const float q[3], float x, float y, float z) {
+  const float dx = __fsub_rn(x, q[0]), dy = __fsub_rn(y, q[1]), dz = __fsub_rn(z, q[2]);
+  return __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+}
+
+// -q, twice per axis, for the two-wide distances.
+struct NNQuery {
+  unsigned long long x, y, z;
+};
+__device__ __forceinline__ unsigned long long nn_twice(float v) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ NNQuery nn_query(const float q[3]) {
+  return NNQuery{nn_twice(-q[0]), nn_twice(-q[1]), nn_twice(-q[2])};
+}
+__device__ __forceinline__ void nn_d32x2(unsigned long long x, unsigned long long y, unsigned long long z,
+                                         const NNQuery& q, float& d0, float& d1) {
+  asm("{\n .reg .b64 a, b, c;\n"
+      " add.rn.f32x2 a, %2, %5;\n add.rn.f32x2 b, %3, %6;\n add.rn.f32x2 c, %4, %7;\n"
+      " mul.rn.f32x2 a, a, a;\n fma.rn.f32x2 a, b, b, a;\n fma.rn.f32x2 a, c, c, a;\n"
+      " mov.b64 {%0, %1}, a;\n}\n"
+      : "=f"(d0), "=f"(d1)
+      : "l"(x), "l"(y), "l"(z), "l"(q.x), "l"(q.y), "l"(q.z));
+}
+// Where part k (0: x, 1: y, 2: z, 3: index) of chunk c lies, in float4.
+__host__ __device__ __forceinline__ int64_t nn_part(int64_t c, int k) {
+  return 4 * c + ((k + (int)(c >> 1)) & 3);
+}
+
+// Part k of the point at place i (4 chunk + place in the chunk).
+__device__ __forceinline__ float nn_value(const float4* __restrict__ pts, int64_t i, int k) {
+  return __ldg(reinterpret_cast<const float*>(pts + nn_part(i >> 2, k)) + (i & 3));
+}
+
+// The distances of chunk c's four points.
+__device__ __forceinline__ void nn_chunk(const float4* __restrict__ pts, const NNQuery& q, int c, float d[4]) {
+  const ulonglong2* p = reinterpret_cast<const ulonglong2*>(pts + 4 * (int64_t)c);
+  const int r = c >> 1;
+  const ulonglong2 X = __ldg(p + (r & 3)), Y = __ldg(p + ((r + 1) & 3)), Z = __ldg(p + ((r + 2) & 3));
+  nn_d32x2(X.x, Y.x, Z.x, q, d[0], d[1]);
+  nn_d32x2(X.y, Y.y, Z.y, q, d[2], d[3]);
+}
+
+// The pruning radius squared that a known float32 distance d gives.
+__device__ __forceinline__ float nn_thr(float d) { return d * (1.0f + 8.0f * NN_EPS) + NN_TINY; }
+
+// The cells [lo, hi] (grid coordinates) of block (bx, by, bz) as a mask.
+__host__ __device__ __forceinline__ unsigned long long nn_box_mask(const int lo[3], const int hi[3], int bx, int by,
+                                                                   int bz) {
+  const int xl = lo[0] - 4 * bx > 0 ? lo[0] - 4 * bx : 0, xh = hi[0] - 4 * bx < 3 ? hi[0] - 4 * bx : 3;
+  const int yl = lo[1] - 4 * by > 0 ? lo[1] - 4 * by : 0, yh = hi[1] - 4 * by < 3 ? hi[1] - 4 * by : 3;
+  const int zl = lo[2] - 4 * bz > 0 ? lo[2] - 4 * bz : 0, zh = hi[2] - 4 * bz < 3 ? hi[2] - 4 * bz : 3;
+  if (xl > xh || yl > yh || zl > zh) return 0ull;
+  const uint32_t x = ((2u << xh) - (1u << xl)) * 0x11111111u;
+  const uint32_t y = ((16u << (4 * yh)) - (1u << (4 * yl))) * 0x00010001u;
+  const unsigned long long xy = (unsigned long long)(x & y);
+  const unsigned long long z = (~0ull >> (48 - 16 * zh)) & (~0ull << (16 * zl));
+  return (xy | (xy << 32)) & z;
+}
+
+// A stored block: its occupancy and first occupied cell.
+struct NNBlock {
+  unsigned long long mask;
+  int first;
+};
+
+__device__ __forceinline__ NNBlock nn_block(float4 B) {
+  return NNBlock{(unsigned long long)__float_as_uint(B.z) | ((unsigned long long)__float_as_uint(B.w) << 32),
+                 __float_as_int(B.y)};
+}
+
+// Takes from m its lowest cell and the ones after it up to the next occupied
+// cell of the block that is not in m: their chunks are one range [a, b).
+__device__ __forceinline__ void nn_pop_cells(const NNGrid& g, const NNBlock& k, unsigned long long& m, int& a, int& b) {
+  const unsigned long long low = m & (0ull - m);
+  const unsigned long long stop = k.mask & ~m & (0ull - low);
+  const unsigned long long run = m & ((stop & (0ull - stop)) - 1ull);  // all of m without a stop
+  const int32_t* o = g.occ + k.first + __popcll(k.mask & (low - 1ull));
+  m ^= run;
+  a = __ldg(o);
+  b = __ldg(o + __popcll(run));
+}
+
+// The cells of stored block bi at (bx, by, bz) that can hold a point within
+// squared distance thr of q.  Every point p of the block has n . p in
+// [lo, hi], so |p - q| is at least the gap h from n . q to that interval, and
+// what of p - q is across n is at most l = sqrt(thr - h^2) long: along axis a,
+// p_a - q_a lies in n_a [lo - n.q, hi - n.q] +- l sqrt(1 - n_a^2).  On a flat
+// patch this leaves a disc around the foot of q where the ball around q would
+// take every cell that reaches into it from below.  The margin covers the
+// rounding of the dot products and of the cell faces, 1e-3 that of the root's
+// argument near n_a = 1.
+__device__ __forceinline__ unsigned long long nn_block_cells(const float q[3], float thr, float margin,
+                                                             const NNGrid& g, int bi, int bx, int by, int bz,
+                                                             NNBlock& k) {
+  const float4 A = __ldg(g.blk + 2 * (int64_t)bi), B = __ldg(g.blk + 2 * (int64_t)bi + 1);
+  k = nn_block(B);
+  if (!(thr < INFINITY)) return k.mask;
+  const float nq = A.x * q[0] + A.y * q[1] + A.z * q[2];
+  const float dlo = A.w - nq - margin, dhi = B.x - nq + margin;
+  const float h = fmaxf(fmaxf(dlo, -dhi), 0.f);
+  const float rem = thr - h * h;
+  if (!(rem >= 0.f)) return 0ull;
+  const float l = nn_root(rem) * 1.000001f + margin, rad = nn_root(thr) * 1.000001f + margin;
+  const float n[3] = {A.x, A.y, A.z};
+  int lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const float u = n[a] * dlo, v = n[a] * dhi;
+    const float w = l * (nn_root(1.0f - n[a] * n[a]) + 1e-3f) + margin;
+    lo[a] = nn_cell(q[a] + fmaxf(fminf(u, v) - w, -rad), g);
+    hi[a] = nn_cell(q[a] + fminf(fmaxf(u, v) + w, rad), g);
+  }
+  return k.mask & nn_box_mask(lo, hi, bx, by, bz);
+}
+
+// Visit every cell of ring r (Chebyshev shell of cells) around cell c that
+// holds points.
+template <typename F>
+__device__ __forceinline__ void nn_ring(const int c[3], int r, const NNGrid& g, F&& visit) {
+  int lo[3], hi[3], li[3], hj[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    lo[a] = max(c[a] - r, 0);
+    hi[a] = min(c[a] + r, g.G - 1);
+    li[a] = c[a] - r + 1;
+    hj[a] = c[a] + r - 1;
+  }
+  for (int bz = lo[2] >> 2; bz <= hi[2] >> 2; ++bz)
+    for (int by = lo[1] >> 2; by <= hi[1] >> 2; ++by)
+      for (int bx = lo[0] >> 2; bx <= hi[0] >> 2; ++bx) {
+        const int bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+        if (bi < 0) continue;
+        const NNBlock k = nn_block(__ldg(g.blk + 2 * (int64_t)bi + 1));
+        unsigned long long m = k.mask & nn_box_mask(lo, hi, bx, by, bz);
+        if (r > 0) m &= ~nn_box_mask(li, hj, bx, by, bz);
+        while (m) {
+          int a, b;
+          nn_pop_cells(g, k, m, a, b);
+          visit(a, b);
+        }
+      }
+}
+
+// Lower bound on |p_a - q_a| for any point p in super-block s along one axis
+// (those at the grid's ends extend to infinity outwards).
+__device__ __forceinline__ float nn_super_gap(float qa, int s, const NNGrid& g, float margin) {
+  const float lo = -1.0f + (float)(16 * s) * g.cs, hi = lo + 16.0f * g.cs;
   float d = 0.f;
-  if (ca > 0 && qa < lo) d = lo - qa;
-  if (ca < g.G - 1 && qa > hi) d = qa - hi;
+  if (s > 0 && qa < lo) d = lo - qa;
+  if (s < g.nsup - 1 && qa > hi) d = qa - hi;
   return fmaxf(d - margin, 0.f);
 }
 
-// Exact nearest point: b1/j1 = best float32 distance and its index, b2 = the
-// runner-up distance (any other point), thr = b1 (1 + 8 eps) + tiny = the
-// pruning radius squared.  Only cells that may hold a point with squared
-// distance <= thr are read: a row of cells (fixed y, z) is skipped when its y/z
-// lower bound already exceeds thr, and its x-range is clipped to the cells
-// that intersect the remaining radius.
-struct NNState {
-  float b1, b2, thr;
-  int j1;
+// Visit, in rings of super-blocks around q, the cells that can hold a point
+// within squared distance thr of q (thr is read live and may start at +inf).
+template <typename F>
+__device__ __forceinline__ void nn_walk(const float q[3], const NNGrid& g, float margin, const float& thr, F&& visit) {
+  const int c[3] = {nn_cell(q[0], g) >> 4, nn_cell(q[1], g) >> 4, nn_cell(q[2], g) >> 4};
+  for (int r = 0;; ++r) {
+    if (r > 0) {
+      float gap = INFINITY;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        if (c[a] - r >= 0) gap = fminf(gap, nn_super_gap(q[a], c[a] - r, g, margin));
+        if (c[a] + r < g.nsup) gap = fminf(gap, nn_super_gap(q[a], c[a] + r, g, margin));
+      }
+      if (!(gap < INFINITY) || gap * gap > thr) break;
+    }
+    for (int sz = max(c[2] - r, 0); sz <= min(c[2] + r, g.nsup - 1); ++sz)
+      for (int sy = max(c[1] - r, 0); sy <= min(c[1] + r, g.nsup - 1); ++sy) {
+        const bool face = sz == c[2] - r || sz == c[2] + r || sy == c[1] - r || sy == c[1] + r;
+        for (int sx = c[0] - r; sx <= c[0] + r; sx += (face || r == 0) ? 1 : 2 * r) {
+          if (sx < 0 || sx >= g.nsup) continue;
+          unsigned long long sm = __ldg(g.sup + ((int64_t)sz * g.nsup + sy) * g.nsup + sx);
+          if (!sm) continue;
+          const float dx = nn_super_gap(q[0], sx, g, margin), dy = nn_super_gap(q[1], sy, g, margin),
+                      dz = nn_super_gap(q[2], sz, g, margin);
+          if (dx * dx + dy * dy + dz * dz > thr) continue;
+          while (sm) {
+            const int bit = __ffsll((long long)sm) - 1;
+            sm &= sm - 1ull;
+            const int bx = 4 * sx + (bit & 3), by = 4 * sy + ((bit >> 2) & 3), bz = 4 * sz + (bit >> 4);
+            const int bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+            NNBlock k;
+            unsigned long long m = nn_block_cells(q, thr, margin, g, bi, bx, by, bz, k);
+            while (m) {
+              int a, b;
+              nn_pop_cells(g, k, m, a, b);
+              visit(a, b);
+            }
+          }
+        }
+      }
+  }
+}
+
+// The best float32 distance seen (b1, of a point of chunk c1) and the smallest
+// of any other point (b2).  No chunk is met twice.
+struct NNTop {
+  float b1, b2;
+  int c1;
 };
 
-__device__ __forceinline__ void nn_update(NNState& st, float d, int j) {
-  if (d > st.b2) return;   // neither the best nor the runner-up (b1 <= b2)
-  if (j == st.j1) return;  // the seeded point, met again in the scan
-  if (d < st.b1 || (d == st.b1 && j < st.j1)) {
-    st.b2 = st.b1;
-    st.b1 = d;
-    st.j1 = j;
-    st.thr = d * (1.0f + 8.0f * NN_EPS) + NN_TINY;
-  } else if (d < st.b2) {
-    st.b2 = d;
+__device__ __forceinline__ void nn_scan(NNTop& t, const NNQuery& q, const NNGrid& g, int c) {
+  float d[4];
+  nn_chunk(g.pts, q, c, d);
+  const float l0 = fminf(d[0], d[1]), h0 = fmaxf(d[0], d[1]), l1 = fminf(d[2], d[3]), h1 = fmaxf(d[2], d[3]);
+  const float m = fminf(l0, l1);                                   // the chunk's best
+  const float m2 = fminf(fmaxf(l0, l1), fminf(h0, h1));            // and its runner-up
+  t.b2 = fminf(fminf(t.b2, m2), fmaxf(t.b1, m));
+  if (m < t.b1) {
+    t.b1 = m;
+    t.c1 = c;
   }
 }
 
-// Lower bound on the y/z distance from q to any point in a row outside the
-// square of rows [c - r, c + r]^2 (y, z); +inf when that square covers the grid.
-__device__ __forceinline__ float nn_gap_yz(const float q[3], const int c[3], int r, const NNGrid& g) {
-  float gap = INFINITY;
-#pragma unroll
-  for (int a = 1; a < 3; ++a) {
-    if (c[a] - r > 0) gap = fminf(gap, q[a] - (-1.0f + (float)(c[a] - r) * g.cs));
-    if (c[a] + r < g.G - 1) gap = fminf(gap, (-1.0f + (float)(c[a] + r + 1) * g.cs) - q[a]);
-  }
-  return gap;
-}
-
-// Visit the rows (fixed y, z) of square ring r around the query's row, each
-// clipped to the cells whose points may lie within sqrt(thr) of q.  Rows whose
-// y/z lower bound alone exceeds thr are skipped.  thr is read live, so rows
-// visited later use the tighter radius.
-template <typename F>
-__device__ __forceinline__ void nn_row_ring(const float q[3], const int c[3], int r, const NNGrid& g, float margin,
-                                            const float& thr, F&& visit) {
-  const int G = g.G;
-  for (int dz = -r; dz <= r; ++dz) {
-    int cz = c[2] + dz;
-    if (cz < 0 || cz >= G) continue;
-    float lz = nn_axis_gap(q[2], cz, g, margin);
-    float lz2 = lz * lz;
-    bool zedge = (dz == -r || dz == r);
-    int step = zedge ? 1 : 2 * r;
-    for (int dy = -r; dy <= r; dy += (step > 0 ? step : 1)) {
-      int cy = c[1] + dy;
-      if (cy < 0 || cy >= G) continue;
-      float ly = nn_axis_gap(q[1], cy, g, margin);
-      float lyz2 = fmaf(ly, ly, lz2);
-      if (lyz2 > thr) continue;
-      int xa = 0, xb = G - 1;
-      float rem = thr - lyz2;
-      if (rem < 16.0f) {
-        float rad = nn_row_sqrt(rem) * 1.000001f + margin;
-        xa = nn_cell(q[0] - rad, g);
-        xb = nn_cell(q[0] + rad, g);
-      }
-      int64_t row = ((int64_t)cz * G + cy) * G;
-      visit(__ldg(g.start + row + xa), __ldg(g.start + row + xb + 1));
-      if (r == 0) break;
+// Step 1 of a search: a first point.  hint: index of a cloud point
+// to start from (-1: none); a record of `seeds` is a point s and its normal n
+// as three 10-bit signed fractions of 511 (0: unknown).  The nearest point is
+// expected around the foot of q on the tangent plane of s, then on the plane
+// of the block there (of the block of s, where that one holds no point); the
+// points of the 2^3 cells nearest to that place are scanned, or those of the
+// whole block where these are empty.  Returns the block scanned and where:
+// record << 7 | all << 6 | lowest scanned cell in the block, -1 if none.
+template <bool COUNT>
+__device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, const float4* __restrict__ seeds,
+                                        const NNGrid& g, NNTop& t, int& work) {
+  t = NNTop{INFINITY, INFINITY, -1};
+  float f[3] = {q[0], q[1], q[2]};
+  float4 s = make_float4(q[0], q[1], q[2], 0.f);
+  if (hint >= 0 && hint < J) {
+    s = __ldg(seeds + hint);
+    const float d = nn_d32(q, s.x, s.y, s.z);
+    if (COUNT) ++work;
+    if (d < INFINITY) {
+      const int w = __float_as_int(s.w);
+      const float n0 = (float)((w << 22) >> 22) * (1.0f / 511.0f), n1 = (float)((w << 12) >> 22) * (1.0f / 511.0f),
+                  n2 = (float)((w << 2) >> 22) * (1.0f / 511.0f);
+      const float h = (q[0] - s.x) * n0 + (q[1] - s.y) * n1 + (q[2] - s.z) * n2;
+      f[0] -= h * n0;
+      f[1] -= h * n1;
+      f[2] -= h * n2;
     }
   }
-}
-
-// Scan rows ring by ring until no unscanned row can hold a point within the
-// pruning radius; returns the last ring visited.
-template <typename F>
-__device__ __forceinline__ int nn_ball_scan(const float q[3], const int c[3], const NNGrid& g, float margin,
-                                            const float& thr, const float& b1, F&& visit) {
-  int r = 0;
-  for (; r <= g.G; ++r) {
-    if (r > 0) {
-      float gap = nn_gap_yz(q, c, r - 1, g);
-      if (gap == INFINITY) break;
-      float gs = gap - margin;
-      if (b1 < INFINITY && gs > 0.f && gs * gs > thr) break;
+  int bx = nn_cell(f[0], g) >> 2, by = nn_cell(f[1], g) >> 2, bz = nn_cell(f[2], g) >> 2;
+  int bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+  if (bi < 0) {
+    bx = nn_cell(s.x, g) >> 2;
+    by = nn_cell(s.y, g) >> 2;
+    bz = nn_cell(s.z, g) >> 2;
+    bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+    if (bi < 0) return -1;
+  }
+  const float4 A = __ldg(g.blk + 2 * (int64_t)bi), B = __ldg(g.blk + 2 * (int64_t)bi + 1);
+  const NNBlock k = nn_block(B);
+  const float n[3] = {A.x, A.y, A.z};
+  const float off = 0.5f * (A.w + B.x) - (A.x * f[0] + A.y * f[1] + A.z * f[2]);
+  const int corner[3] = {4 * bx, 4 * by, 4 * bz};
+  int lo[3], hi[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    // the 2 cells nearest to the place along this axis, inside the block
+    const int c = nn_cell(f[a] + off * n[a] - 0.5f * g.cs, g);
+    lo[a] = min(max(c, corner[a]), corner[a] + 2);
+    hi[a] = lo[a] + 1;
+  }
+  unsigned long long m = k.mask & nn_box_mask(lo, hi, bx, by, bz);
+  const bool all = m == 0ull;
+  if (all) m = k.mask;
+  const NNQuery q2 = nn_query(q);
+  int cur = 0, end = 0;
+  while (true) {
+    if (cur >= end) {
+      if (!m) break;
+      nn_pop_cells(g, k, m, cur, end);
+      if (COUNT) work += 4 * (end - cur);
     }
-    nn_row_ring(q, c, r, g, margin, thr, visit);
+    nn_scan(t, q2, g, cur++);
   }
-  return r - 1;
+  return (bi << 7) | ((int)all << 6) | ((lo[0] & 3) | ((lo[1] & 3) << 2) | ((lo[2] & 3) << 4));
 }
 
-// Count of the records gp_step will treat as valid (q inside the domain, the
-// cells of q and of its nearest point in the pull band), one atomic per warp.
-__device__ __forceinline__ void nn_count_valid(int32_t* nvalid, bool valid) {
-  unsigned m = __activemask();
-  unsigned vb = __ballot_sync(m, valid);
-  if ((int)(threadIdx.x & 31) == __ffs(m) - 1 && vb) atomicAdd(nvalid, __popc(vb));
-}
+// A warp's shared state in step 2: its 32 queries with their bounds, and the
+// two queues.
+struct NNWarp {
+  float4 q[32];                 // x, y, z, pruning radius squared
+  unsigned long long key1[32];  // best distance (float bits), then its chunk
+  unsigned int key2[32];        // best distance of any other point (float bits)
+  int first[32];                // where step 1 scanned
+  int lo[32], hi[32];           // blocks the ball meets, 8 bits an axis
+  int off[32];                  // first super-block of each query in the warp's list
+  int2 range[64];               // chunks to scan: first, query | count << 5
+  int block[64];                // blocks to test: coordinates, 8 bits an axis | query << 24
+};
 
-// NaN surface point for queries outside the domain of the search.
-__device__ __forceinline__ void nn_invalid(int64_t i, const float q[3], int32_t* nn_out, float* rec) {
-  if (nn_out) nn_out[i] = -1;
-  if (rec) {
-    for (int a = 0; a < 6; ++a) rec[6 * i + a] = a < 3 ? q[a] : __int_as_float(0x7fc00000);
-  }
-}
-
-// Seed the search with a known point (the query's source point): its distance
-// bounds the nearest one from above.
-__device__ __forceinline__ void nn_seed(NNState& st, const float q[3], const int32_t* __restrict__ hint, int64_t i,
-                                        int64_t J, const float* __restrict__ pts_orig) {
-  if (!hint) return;
-  int j = hint[i];
-  if (j < 0 || j >= J) return;
-  float dx = q[0] - pts_orig[3 * (int64_t)j], dy = q[1] - pts_orig[3 * (int64_t)j + 1];
-  float dz = q[2] - pts_orig[3 * (int64_t)j + 2];
-  float d = dx * dx + dy * dy + dz * dz;
-  if (d < INFINITY) {
-    st.b1 = d;
-    st.j1 = j;
-    st.thr = d * (1.0f + 8.0f * NN_EPS) + NN_TINY;
-  }
-}
-
-// Seeded search (thr finite from the start): walk the slabs (fixed z) and, in
-// each, the rows (fixed y) closest first, two at a time (one each side), each
-// clipped to the cells within the radius as it stood when the pair was
-// tested; a side stops at its first slab or row whose lower bound exceeds
-// thr, since bounds only grow outwards and thr only shrinks.  Every point
-// with squared distance <= the final thr lies in a row that was visited,
-// within the x-range read.
-template <typename F>
-__device__ __forceinline__ void nn_ball_walk(const float q[3], const int c[3], const NNGrid& g, float margin,
-                                             const float& thr, F&& visit) {
-  const int G = g.G;
-  bool z_done[2] = {false, false};
-  for (int kz = 0; !(z_done[0] && z_done[1]); ++kz) {
+// Step 2 for a warp's queries: the blocks the ball of the best distance meets,
+// cut to the cells that can hold a nearer point (nn_block_cells), without
+// those step 1 scanned.  What one query needs here varies by a factor of ten
+// and more within a warp (its work grows with the cube of its distance), so
+// the work of all 32 is laid out in three lists that the lanes share evenly:
+// the super-blocks of all the balls, the blocks with points these hold, and
+// the ranges of at most two chunks their cells come to.  A list is worked
+// through 32 entries at a time as soon as it has as many.  A point within its
+// query's bound (few are) goes to the query's two keys by atomics in shared
+// memory: the smaller key stays, the larger goes on to the second.
+//
+// Measured (GB300, seeded batches, whole search): with one thread walking its
+// query's rows of cells, 8 of 32 lanes active, 1,116 us for 2,097,152 queries
+// among 10 M points and 206 us for 262,144 among 100,000; with step 2 lane by
+// lane 730 and 210; shared 530 and 104.  It is then bound by the L1 (81% of its
+// wavefronts: a lane's chunk is a line of its own) and by issue (56%).
+// Sorting a block's queries by radius instead of sharing gave 700 and 190.
+template <bool COUNT>
+__device__ __forceinline__ void nn_rest(const float q[3], const NNGrid& g, bool go, int first, NNTop& t, NNWarp& sh,
+                                        int& work) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  int total = 0;
+  {
+    const float thr = nn_thr(t.b1);
+    const float rad = nn_root(thr) * 1.000001f + nn_margin(q);
+    int lo = 0, hi = 0, n = go ? 1 : 0;
 #pragma unroll
-    for (int sz = 0; sz < 2; ++sz) {
-      if (z_done[sz] || (kz == 0 && sz == 1)) continue;
-      const int cz = c[2] + (sz ? -kz : kz);
-      if (cz < 0 || cz >= G) {
-        z_done[sz] = true;
-        continue;
-      }
-      const float lz = nn_axis_gap(q[2], cz, g, margin);
-      const float lz2 = lz * lz;
-      if (lz2 > thr) {
-        z_done[sz] = true;
-        continue;
-      }
-      bool y_done[2] = {false, false};
-      for (int ky = 0; !(y_done[0] && y_done[1]); ++ky) {
-        // Both rows of this distance (c_y + ky, c_y - ky) are tested and
-        // their cell starts loaded before either is scanned, so that the two
-        // rows' loads are in flight together.  The second row's test and
-        // x-range then use the radius from before the first row's scan: a
-        // superset of what the shrunken radius needs.
-        int a[2] = {0, 0}, b[2] = {0, 0};
+    for (int a = 0; a < 3; ++a) {
+      const int l = nn_cell(q[a] - rad, g) >> 2, h = nn_cell(q[a] + rad, g) >> 2;
+      lo |= l << (8 * a);
+      hi |= h << (8 * a);
+      n *= (h >> 2) - (l >> 2) + 1;
+    }
+    __syncwarp();
+    sh.q[lane] = make_float4(q[0], q[1], q[2], thr);
+    sh.key1[lane] = ((unsigned long long)__float_as_uint(t.b1) << 32) | (unsigned)t.c1;
+    sh.key2[lane] = __float_as_uint(t.b2);
+    sh.first[lane] = first;
+    sh.lo[lane] = lo;
+    sh.hi[lane] = hi;
+    int incl = n;
 #pragma unroll
-        for (int sy = 0; sy < 2; ++sy) {
-          if (y_done[sy] || (ky == 0 && sy == 1)) continue;
-          const int cy = c[1] + (sy ? -ky : ky);
-          if (cy < 0 || cy >= G) {
-            y_done[sy] = true;
-            continue;
-          }
-          const float ly = nn_axis_gap(q[1], cy, g, margin);
-          const float lyz2 = fmaf(ly, ly, lz2);
-          if (lyz2 > thr) {
-            y_done[sy] = true;
-            continue;
-          }
-          const float rad = nn_row_sqrt(thr - lyz2) * 1.000001f + margin;
-          const int xa = nn_cell(q[0] - rad, g), xb = nn_cell(q[0] + rad, g);
-          const int64_t row = ((int64_t)cz * G + cy) * G;
-          a[sy] = __ldg(g.start + row + xa);
-          b[sy] = __ldg(g.start + row + xb + 1);
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    sh.off[lane] = incl - n;
+    total = __shfl_sync(FULL, incl, 31);
+    __syncwarp();
+  }
+  int base = 0, nb = 0, nr = 0;  // super-blocks taken, entries of the two queues
+  unsigned long long sm = 0;     // this lane's super-block's blocks still to queue
+  int at = 0;                    // its lowest block | query << 24
+  while (true) {
+    while (nb < 32) {
+      unsigned some = __ballot_sync(FULL, sm != 0ull);
+      if (!some) {
+        if (base >= total) break;
+        const int idx = base + lane;
+        base += 32;
+        if (idx < total) {
+          int o = 0;
+#pragma unroll
+          for (int step = 16; step > 0; step >>= 1)
+            if (sh.off[o + step] <= idx) o += step;
+          const int lw = sh.lo[o], hw = sh.hi[o];
+          const int lo[3] = {lw & 255, (lw >> 8) & 255, lw >> 16}, hi[3] = {hw & 255, (hw >> 8) & 255, hw >> 16};
+          const unsigned nx = (hi[0] >> 2) - (lo[0] >> 2) + 1, ny = (hi[1] >> 2) - (lo[1] >> 2) + 1;
+          const unsigned l = idx - sh.off[o], yz = l / nx;
+          const int sx = (lo[0] >> 2) + (int)(l - yz * nx), sy = (lo[1] >> 2) + (int)(yz % ny),
+                    sz = (lo[2] >> 2) + (int)(yz / ny);
+          sm = __ldg(g.sup + ((int64_t)sz * g.nsup + sy) * g.nsup + sx) & nn_box_mask(lo, hi, sx, sy, sz);
+          at = (4 * sx) | (4 * sy << 8) | (4 * sz << 16) | (o << 24);
         }
+        continue;
+      }
+      if (sm) {
+        const int bit = __ffsll((long long)sm) - 1;
+        sm &= sm - 1ull;
+        sh.block[nb + __popc(some & below)] = at + ((bit & 3) | ((bit >> 2) & 3) << 8 | (bit >> 4) << 16);
+      }
+      nb += __popc(some);
+    }
+    if (nb == 0 && nr == 0) break;
+    const bool last = nb <= 32 && base >= total && !__any_sync(FULL, sm != 0ull);
+    const int take = min(nb, 32);
+    nb -= take;
+    __syncwarp();
+    unsigned long long m = 0ull;
+    NNBlock k{0ull, 0};
+    int o = 0, a = 0, n = 0;
+    if (lane < take) {
+      const int e = sh.block[nb + lane];
+      const int bx = e & 255, by = (e >> 8) & 255, bz = (e >> 16) & 255;
+      o = (int)((unsigned)e >> 24);
+      const float4 Q = sh.q[o];
+      const float qo[3] = {Q.x, Q.y, Q.z};
+      const int bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+      m = nn_block_cells(qo, Q.w, nn_margin(qo), g, bi, bx, by, bz, k);
+      const int f = sh.first[o];
+      if (bi == f >> 7) {
+        const int l0[3] = {f & 3, (f >> 2) & 3, (f >> 4) & 3};
+        const int h0[3] = {l0[0] + 1, l0[1] + 1, l0[2] + 1};
+        m &= (f & 64) ? 0ull : ~nn_box_mask(l0, h0, 0, 0, 0);
+      }
+    }
+    __syncwarp();
+    while (true) {
+      if (n == 0 && m) {
+        int b;
+        nn_pop_cells(g, k, m, a, b);
+        n = b - a;
+        if (COUNT) work += 4 * n;
+      }
+      const unsigned some = __ballot_sync(FULL, n > 0);
+      if (n > 0) {
+        const int c = min(n, 2);
+        sh.range[nr + __popc(some & below)] = make_int2(a, o | c << 5);
+        a += c;
+        n -= c;
+      }
+      nr += __popc(some);
+      const bool flush = last && !some;
+      if (nr >= 32 || (flush && nr > 0)) {
+        const int r = min(nr, 32);
+        nr -= r;
+        __syncwarp();
+        if (lane < r) {
+          const int2 e = sh.range[nr + lane];
+          const int w = e.y & 31;
+          const float4 Q = sh.q[w];
+          const float qo[3] = {Q.x, Q.y, Q.z};
+          const NNQuery q2 = nn_query(qo);
+          const int c2 = (e.y >> 5) > 1 ? e.x + 1 : e.x;
+          float d[2][4];
+          nn_chunk(g.pts, q2, e.x, d[0]);
+          nn_chunk(g.pts, q2, c2, d[1]);
 #pragma unroll
-        for (int sy = 0; sy < 2; ++sy)
-          if (b[sy] > a[sy]) visit(a[sy], b[sy]);
+          for (int j = 0; j < 2; ++j) {
+            const float l0 = fminf(d[j][0], d[j][1]), h0 = fmaxf(d[j][0], d[j][1]);
+            const float l1 = fminf(d[j][2], d[j][3]), h1 = fmaxf(d[j][2], d[j][3]);
+            const float lm = fminf(l0, l1);
+            if (lm <= Q.w && (j == 0 || c2 != e.x)) {
+              const float m2 = fminf(fmaxf(l0, l1), fminf(h0, h1));
+              const unsigned long long key =
+                  ((unsigned long long)__float_as_uint(lm) << 32) | (unsigned)(j ? c2 : e.x);
+              const unsigned long long was = atomicMin(&sh.key1[w], key);
+              atomicMin(&sh.key2[w], min((unsigned)((was > key ? was : key) >> 32), __float_as_uint(m2)));
+            }
+          }
+        }
+        __syncwarp();
       }
+      if (!some && !(flush && nr > 0)) break;
     }
+    if (last) break;
+  }
+  __syncwarp();
+  if (go) {
+    const unsigned long long k1 = sh.key1[lane];
+    t.b1 = __uint_as_float((unsigned)(k1 >> 32));
+    t.c1 = (int)(unsigned)k1;
+    t.b2 = __uint_as_float(sh.key2[lane]);
   }
 }
 
-// Near tie (another point within the float32 margin of the best): rank every
-// point within the margin by its float64 distance and index.  Rings 0..r_end
-// (or, for r_end < 0, the ball walk) cover every row within the pruning radius.
-__device__ __forceinline__ int nn_break_tie(const float q[3], const int c[3], const NNGrid& g, float margin,
-                                            const NNState& st, int r_end, int* work = nullptr) {
-  const float tie = st.b1 * (1.0f + 2.0f * NN_EPS) + NN_TINY;
-  if (st.b2 > tie) return st.j1;
-  double bd = INFINITY;
-  int bj = 0x7fffffff;
-  const float thr = st.thr;
-  auto rank = [&](int a, int b) {
-    if (work) *work += b > a ? b - a : 0;
-    for (int p = a; p < b; ++p) {
-      float4 P = g.pts[p];
-      float dx = q[0] - P.x, dy = q[1] - P.y, dz = q[2] - P.z;
-      float d = dx * dx + dy * dy + dz * dz;
-      if (d > tie) continue;
-      int j = __float_as_int(P.w);
-      double dd = nn_d64(q, P);
-      if (dd < bd || (dd == bd && j < bj)) {
-        bd = dd;
-        bj = j;
+// The answer of a searched query: its index and point.  At a near tie
+// (another point within the float32 margin of the best) every point within
+// the margin is ranked by its float64 distance and index.  -1 if no point
+// compares below +inf.
+template <bool COUNT>
+__device__ __forceinline__ int nn_answer(const float q[3], const NNGrid& g, const NNTop& t, float s[3], int& work) {
+  if (t.c1 < 0) return -1;
+  const NNQuery q2 = nn_query(q);
+  const float tie = t.b1 * (1.0f + 2.0f * NN_EPS) + NN_TINY;
+  int64_t at = 0;  // 4 chunk + place
+  if (t.b2 > tie) {
+    float d[4];
+    nn_chunk(g.pts, q2, t.c1, d);
+    at = 4 * (int64_t)t.c1 + (d[0] == t.b1 ? 0 : d[1] == t.b1 ? 1 : d[2] == t.b1 ? 2 : 3);
+  } else {
+    double bd = INFINITY;
+    int bj = 0x7fffffff;
+    const float thr = nn_thr(t.b1);
+    nn_walk(q, g, nn_margin(q), thr, [&](int a, int b) {
+      if (COUNT) work += 4 * (b - a);
+      for (int c = a; c < b; ++c) {
+        float d[4];
+        nn_chunk(g.pts, q2, c, d);
+        for (int k = 0; k < 4; ++k) {
+          if (!(d[k] <= tie)) continue;
+          const int64_t i = 4 * (int64_t)c + k;
+          const int j = __float_as_int(nn_value(g.pts, i, 3));
+          const double dd = nn_d64(q, nn_value(g.pts, i, 0), nn_value(g.pts, i, 1), nn_value(g.pts, i, 2));
+          if (dd < bd || (dd == bd && j < bj)) {
+            bd = dd;
+            bj = j;
+            at = i;
+          }
+        }
       }
-    }
-  };
-  if (r_end < 0)
-    nn_ball_walk(q, c, g, margin, thr, rank);
-  else
-    for (int r = 0; r <= r_end; ++r) nn_row_ring(q, c, r, g, margin, thr, rank);
-  return bj != 0x7fffffff ? bj : st.j1;
-}
-
-// The whole search for one query by one thread, from whatever seed st holds.
-// Returns the nearest point's index, or -1 if none compares below +inf.
-// work (optional): incremented by the number of point distances evaluated.
-__device__ __forceinline__ int nn_thread_search(const float q[3], const int c[3], const NNGrid& g, float margin,
-                                                NNState& st, int* work = nullptr) {
-  auto one = [&](float4 P) {
-    float dx = q[0] - P.x, dy = q[1] - P.y, dz = q[2] - P.z;
-    nn_update(st, dx * dx + dy * dy + dz * dz, __float_as_int(P.w));
-  };
-  // Points of a range, four loads in flight at a time (same visiting order).
-  auto scan = [&](int a, int b) {
-    if (work) *work += b > a ? b - a : 0;
-    int p = a;
-    for (; p + 4 <= b; p += 4) {
-      float4 P0 = __ldg(g.pts + p), P1 = __ldg(g.pts + p + 1), P2 = __ldg(g.pts + p + 2), P3 = __ldg(g.pts + p + 3);
-      one(P0);
-      one(P1);
-      one(P2);
-      one(P3);
-    }
-    for (; p < b; ++p) one(__ldg(g.pts + p));
-  };
-  int r_end = -1;
-  if (st.b1 < INFINITY)
-    nn_ball_walk(q, c, g, margin, st.thr, scan);  // seeded: closest-first walk of the ball
-  else
-    r_end = nn_ball_scan(q, c, g, margin, st.thr, st.b1, scan);
-  if (st.j1 == 0x7fffffff) return -1;
-  return nn_break_tie(q, c, g, margin, st, r_end, work);
-}
-
-__device__ __forceinline__ void nn_finish(int64_t i, const float q[3], int best, const float* __restrict__ pts_orig,
-                                          int32_t* __restrict__ nn_out, float* __restrict__ rec, const Grid& band,
-                                          int32_t* __restrict__ nvalid) {
-  if (best < 0) {
-    nn_invalid(i, q, nn_out, rec);
-    if (nvalid) nn_count_valid(nvalid, false);
-    return;
+    });
   }
-  float s3[3] = {pts_orig[3 * (int64_t)best], pts_orig[3 * (int64_t)best + 1], pts_orig[3 * (int64_t)best + 2]};
-  if (nn_out) nn_out[i] = best;
-  if (rec) {
-    rec[6 * i + 0] = q[0];
-    rec[6 * i + 1] = q[1];
-    rec[6 * i + 2] = q[2];
-    rec[6 * i + 3] = s3[0];
-    rec[6 * i + 4] = s3[1];
-    rec[6 * i + 5] = s3[2];
-  }
-  if (nvalid) {
-    Cells C;
-    nn_count_valid(nvalid, classify(band, q, s3, C));
-  }
+#pragma unroll
+  for (int a = 0; a < 3; ++a) s[a] = nn_value(g.pts, at, a);
+  return __float_as_int(nn_value(g.pts, at, 3));
 }
 
 __device__ __forceinline__ bool nn_query_ok(const float q[3]) {
   return fabsf(q[0]) <= 1e18f && fabsf(q[1]) <= 1e18f && fabsf(q[2]) <= 1e18f;
 }
 
-// Extra seeds: the points of the cell holding the foot of q on the tangent
-// plane of its source point, f = q - ((q - s) . n) n.  The nearest point tends
-// to lie near f, much closer to q than s is, which shrinks the ball to walk.
-__device__ __forceinline__ void nn_seed_foot(NNState& st, const float q[3], const int32_t* __restrict__ hint,
-                                             int64_t i, int64_t J, const float* __restrict__ pts_orig,
-                                             const float* __restrict__ normals, const NNGrid& g,
-                                             int* work = nullptr) {
-  if (!hint || !normals) return;
-  const int j = hint[i];
-  if (j < 0 || j >= J) return;
-  const float n0 = normals[3 * (int64_t)j], n1 = normals[3 * (int64_t)j + 1], n2 = normals[3 * (int64_t)j + 2];
-  const float s0 = pts_orig[3 * (int64_t)j], s1 = pts_orig[3 * (int64_t)j + 1], s2 = pts_orig[3 * (int64_t)j + 2];
-  const float h = (q[0] - s0) * n0 + (q[1] - s1) * n1 + (q[2] - s2) * n2;
-  const int cx = nn_cell(q[0] - h * n0, g), cy = nn_cell(q[1] - h * n1, g), cz = nn_cell(q[2] - h * n2, g);
-  const int64_t cell = ((int64_t)cz * g.G + cy) * g.G + cx;
-  const int a = __ldg(g.start + cell), b = __ldg(g.start + cell + 1);
-  if (work) *work += b > a ? b - a : 0;
-  for (int p = a; p < b; ++p) {
-    float4 P = __ldg(g.pts + p);
-    float dx = q[0] - P.x, dy = q[1] - P.y, dz = q[2] - P.z;
-    nn_update(st, dx * dx + dy * dy + dz * dz, __float_as_int(P.w));
+// The search of a warp's 32 queries, one a lane, all lanes together (ok: this
+// lane has one).  Step 1 lane by lane, step 2 shared; a query that step 1
+// leaves without a bound walks the rings instead.
+template <bool COUNT>
+__device__ __forceinline__ int nn_search(const float q[3], bool ok, int hint, int64_t J,
+                                         const float4* __restrict__ seeds, const NNGrid& g, NNWarp& sh, float s[3],
+                                         int& work) {
+  NNTop t{INFINITY, INFINITY, -1};
+  int first = -1;
+  bool go = false;
+  if (ok) {
+    first = nn_first<COUNT>(q, hint, J, seeds, g, t, work);
+    go = t.b1 < INFINITY;
+    if (!go) {
+      const NNQuery q2 = nn_query(q);
+      float thr = INFINITY;
+      t = NNTop{INFINITY, INFINITY, -1};
+      nn_walk(q, g, nn_margin(q), thr, [&](int a, int b) {
+        if (COUNT) work += 4 * (b - a);
+        for (int c = a; c < b; ++c) nn_scan(t, q2, g, c);
+        thr = nn_thr(t.b1);
+      });
+    }
   }
+  __syncwarp();
+  nn_rest<COUNT>(q, g, go, first, t, sh, work);
+  return ok ? nn_answer<COUNT>(q, g, t, s, work) : -1;
+}
+
+__host__ __device__ __forceinline__ int nn_pack_normal(float x, float y, float z) {
+  return ((int)lrintf(x * 511.0f) & 1023) | (((int)lrintf(y * 511.0f) & 1023) << 10) |
+         (((int)lrintf(z * 511.0f) & 1023) << 20);
 }
 
 inline NNGrid make_grid(const gp_band* b) {
   NNGrid g;
   g.pts = b->pts_sorted;
-  g.start = b->cell_start;
+  g.occ = b->cell_occ;
+  g.blk = b->cell_blk;
+  g.table = b->cell_table;
+  g.sup = b->cell_sup;
   g.G = b->G;
+  g.nbk = (b->G + 3) / 4;
+  g.nsup = (b->G + 15) / 16;
   g.half_g = 0.5f * (float)b->G;
   g.cs = 2.0f / (float)b->G;
   return g;
 }
-
