@@ -56,7 +56,9 @@ __global__ void k_na_clear(double* __restrict__ scratch) {
   }
 }
 
-__global__ void k_na_zero(float* __restrict__ g, int64_t n) {
+// The gradient and the counters in one launch.
+__global__ void k_na_zero(float* __restrict__ g, int64_t n, double* __restrict__ scratch) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) *na_counters(scratch) = NACounters{0, 0};
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     g[i] = 0.f;
 }
@@ -234,12 +236,26 @@ __global__ void __launch_bounds__(NA_THREADS) k_na_query(int R, const float* __r
   __syncthreads();
   if (!am_last) return;
   __threadfence();
+  // The block sums, summed by the whole block in a fixed order.  One thread
+  // alone took 45 of the kernel's 70 us at 99,999 records: three dependent
+  // L2 reads for each of 391 rows.
+  __shared__ double tot[3][NA_THREADS / 32];
+  double t[3] = {0, 0, 0};
+  for (unsigned k = threadIdx.x; k < gridDim.x; k += NA_THREADS)
+#pragma unroll
+    for (int a = 0; a < 3; ++a) t[a] += __ldcg(scratch + (int64_t)k * 4 + a);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    t[a] = gp_warp_sum_d(t[a]);
+    if ((threadIdx.x & 31) == 0) tot[a][threadIdx.x >> 5] = t[a];
+  }
+  __syncthreads();
   if (threadIdx.x == 0) {
     double t0 = 0, t1 = 0, t2 = 0;
-    for (unsigned k = 0; k < gridDim.x; ++k) {
-      t0 += __ldcg(scratch + (int64_t)k * 4 + 0);
-      t1 += __ldcg(scratch + (int64_t)k * 4 + 1);
-      t2 += __ldcg(scratch + (int64_t)k * 4 + 2);
+    for (int k = 0; k < NA_THREADS / 32; ++k) {
+      t0 += tot[0][k];
+      t1 += tot[1][k];
+      t2 += tot[2][k];
     }
     double lp = bv > 0 ? t0 / bv : 0.0, lg = bv > 0 ? t1 / bv : 0.0, ls = bv > 0 ? t2 / bv : 0.0;
     loss[GP_LOSS_TOTAL] = (float)(lp + beta * ls + gamma * lg);
@@ -308,8 +324,10 @@ extern "C" gp_status gp_step_dense_noalloc(gp_ctx* ctx, int32_t R, const float* 
   if (st) return st;
   cudaStream_t s = ctx->stream;
   const int64_t nv = (int64_t)(R + 1) * (R + 1) * (R + 1);
-  GP_KERNEL(ctx, "k_na_clear", k_na_clear<<<1, 32, 0, s>>>(scratch));
-  if (grad_dev) GP_KERNEL(ctx, "k_na_zero", k_na_zero<<<gp_blocks(nv, 256, 4096), 256, 0, s>>>(grad_dev, nv));
+  if (grad_dev)
+    GP_KERNEL(ctx, "k_na_zero", k_na_zero<<<gp_blocks(nv, 256, 4096), 256, 0, s>>>(grad_dev, nv, scratch));
+  else
+    GP_KERNEL(ctx, "k_na_clear", k_na_clear<<<1, 32, 0, s>>>(scratch));
   const unsigned blocks = gp_blocks(B, NA_THREADS, NA_MAX_BLOCKS);
   if (B > 0) GP_KERNEL(ctx, "k_na_count", k_na_count<<<blocks, NA_THREADS, 0, s>>>(R, rec_dev, B, scratch));
   GP_KERNEL(ctx, "k_na_query", k_na_query<<<blocks, NA_THREADS, 0, s>>>(R, d_dev, rec_dev, B, w->beta, w->gamma,
