@@ -10,109 +10,157 @@ gp_status gp_build_points(gp_band* band, const float* pts_dev);  // gp_nn.cu
 
 namespace {
 
-// Cell map bits.
-constexpr uint8_t C_OCC = 1, C_M1 = 2, C_M2 = 4, C_MX = 8;
-// Vertex map bits (match the export flags).
-constexpr uint8_t V_T = 1, V_TRAIN = 2, V_PULL = 8;
+// The cell and vertex sets are bit rows along x: 32 cells (or vertices) a
+// word, row (y, z) starting at word (z n + y) W.  A byte per element took 16
+// times the bytes in the dilation, and a thread per element: the kernels that
+// make an object band on a 256^3 grid took 864 us, and the whole build is
+// 0.8 ms shorter this way (7.96 -> 7.16 ms).
+struct CellRows {
+  int R, W;  // cells per axis, words per row
+};
+struct VertRows {
+  int n, W;  // vertices per axis, words per row
+};
 
-__global__ void k_mark_occupied(const float* __restrict__ pts, int64_t J, int R, uint8_t* __restrict__ cells) {
+__device__ __forceinline__ uint32_t row_tail(int n, int w) {  // the bits of word w that exist in a row of n
+  const int left = n - 32 * w;
+  return left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+}
+
+__global__ void k_mark_occupied(const float* __restrict__ pts, int64_t J, CellRows g, uint32_t* __restrict__ occ) {
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= J) return;
-  float half_r = 0.5f * (float)R;
+  const float half_r = 0.5f * (float)g.R;
   int c[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    gp_cell1 g = gp_cell_exact(pts[3 * j + a], half_r);
-    c[a] = min(max(g.c, 0), R - 1);
+    gp_cell1 p = gp_cell_exact(pts[3 * j + a], half_r);
+    c[a] = min(max(p.c, 0), g.R - 1);
   }
-  cells[((int64_t)c[2] * R + c[1]) * R + c[0]] = C_OCC;
+  uint32_t* word = occ + ((int64_t)c[2] * g.R + c[1]) * g.W + (c[0] >> 5);
+  const uint32_t bit = 1u << (c[0] & 31);
+  if (!(*word & bit)) atomicOr(word, bit);  // a stale read only costs the atomic
 }
 
-// One axis of the separable Chebyshev dilation.  Pass 0 dilates the occupied
-// bit into the three band bits; later passes dilate each band bit by its own
-// radius.  Bit C_OCC is carried through.
-__global__ void k_dilate_axis(const uint8_t* __restrict__ in, uint8_t* __restrict__ out, int R, int axis,
-                              int M1, int M2, int MX, int first) {
-  int64_t n = (int64_t)R * R * R;
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= n) return;
-  int x = (int)(idx % R), y = (int)((idx / R) % R), z = (int)(idx / ((int64_t)R * R));
-  int pos = axis == 0 ? x : (axis == 1 ? y : z);
-  int64_t stride = axis == 0 ? 1 : (axis == 1 ? R : (int64_t)R * R);
-  int mm = max(M1, max(M2, MX));
-  uint8_t acc = in[idx] & C_OCC;
-  for (int d = -mm; d <= mm; ++d) {
-    int p = pos + d;
-    if (p < 0 || p >= R) continue;
-    uint8_t v = in[idx + d * stride];
-    int ad = d < 0 ? -d : d;
-    uint8_t s1 = first ? (v & C_OCC) : (v & C_M1);
-    uint8_t s2 = first ? (v & C_OCC) : (v & C_M2);
-    uint8_t s3 = first ? (v & C_OCC) : (v & C_MX);
-    if (s1 && ad <= M1) acc |= C_M1;
-    if (s2 && ad <= M2) acc |= C_M2;
-    if (s3 && ad <= MX) acc |= C_MX;
+// Sum of v over the block, added to *total by one thread.
+__device__ __forceinline__ void add_count(int v, unsigned long long* total) {
+  v = gp_warp_sum_i(v);
+  if ((threadIdx.x & 31) == 0 && v) atomicAdd(total, (unsigned long long)v);
+}
+
+// v with every set bit spread s places up (0 <= s <= 31).
+__device__ __forceinline__ unsigned long long spread_up(unsigned long long v, int s) {
+  for (int done = 0; done < s;) {
+    const int step = min(done + 1, s - done);
+    v |= v << step;
+    done += step;
   }
-  out[idx] = acc;
+  return v;
 }
-
-__global__ void k_set_all_bits(uint8_t* __restrict__ cells, int64_t n, uint8_t bits) {
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx < n) cells[idx] |= bits;
-}
-
-__global__ void k_count_cells(const uint8_t* __restrict__ cells, int64_t n, unsigned long long* counts) {
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  uint8_t v = idx < n ? cells[idx] : 0;
-  int occ = __syncthreads_count(v & C_OCC);
-  int pull = __syncthreads_count(v & C_M1);
-  if (threadIdx.x == 0) {
-    if (occ) atomicAdd(counts + 0, (unsigned long long)occ);
-    if (pull) atomicAdd(counts + 1, (unsigned long long)pull);
+__device__ __forceinline__ unsigned long long spread_down(unsigned long long v, int s) {
+  for (int done = 0; done < s;) {
+    const int step = min(done + 1, s - done);
+    v |= v >> step;
+    done += step;
   }
+  return v;
 }
 
-// Vertex flags: T = corner of an M2 cell, trainable = corner of an MX cell,
-// pull = lowest corner of an M1 cell.
-__global__ void k_vertex_flags(const uint8_t* __restrict__ cells, uint8_t* __restrict__ verts, int R) {
-  int n1 = R + 1;
-  int64_t nv = (int64_t)n1 * n1 * n1;
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nv) return;
-  int i = (int)(idx % n1), j = (int)((idx / n1) % n1), k = (int)(idx / ((int64_t)n1 * n1));
-  uint8_t any = 0;
-  for (int dz = 0; dz < 2; ++dz)
-    for (int dy = 0; dy < 2; ++dy)
-      for (int dx = 0; dx < 2; ++dx) {
-        int ci = i - dx, cj = j - dy, ck = k - dz;
-        if (ci < 0 || cj < 0 || ck < 0 || ci >= R || cj >= R || ck >= R) continue;
-        any |= cells[((int64_t)ck * R + cj) * R + ci];
-      }
-  uint8_t f = 0;
-  if (any & C_M2) f |= V_T;
-  if (any & C_MX) f |= V_TRAIN;
-  if (i < R && j < R && k < R && (cells[((int64_t)k * R + j) * R + i] & C_M1)) f |= V_PULL;
-  verts[idx] = f;
-}
-
-// Required vertices (T, trainable and the axis neighbours of T) mark their brick.
-__global__ void k_required(uint8_t* __restrict__ verts, int R, int nb, uint8_t* __restrict__ need) {
-  int n1 = R + 1;
-  int64_t nv = (int64_t)n1 * n1 * n1;
-  int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= nv) return;
-  int i = (int)(idx % n1), j = (int)((idx / n1) % n1), k = (int)(idx / ((int64_t)n1 * n1));
-  uint8_t f = verts[idx];
-  bool req = (f & (V_T | V_TRAIN)) != 0;
-  if (!req) {
-    const int di[6] = {-1, 1, 0, 0, 0, 0}, dj[6] = {0, 0, -1, 1, 0, 0}, dk[6] = {0, 0, 0, 0, -1, 1};
-    for (int t = 0; t < 6 && !req; ++t) {
-      int a = i + di[t], b = j + dj[t], c = k + dk[t];
-      if (a < 0 || b < 0 || c < 0 || a > R || b > R || c > R) continue;
-      if (verts[((int64_t)c * n1 + b) * n1 + a] & V_T) req = true;
-    }
+// Dilation along x by m <= 31 cells (wider ones are several passes; Chebyshev
+// dilations add up).  count (optional): the set bits of the input.
+__global__ void k_dilate_x(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, CellRows g, int m,
+                           unsigned long long* count) {
+  const int64_t n = (int64_t)g.R * g.R * g.W;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int bits = 0;
+  if (i < n) {
+    const int w = (int)(i % g.W);
+    const uint32_t cur = in[i];
+    const uint32_t lo = w > 0 ? in[i - 1] : 0u, hi = w + 1 < g.W ? in[i + 1] : 0u;
+    const uint32_t up = (uint32_t)(spread_up(((unsigned long long)cur << 32) | lo, m) >> 32);
+    const uint32_t down = (uint32_t)spread_down(((unsigned long long)hi << 32) | cur, m);
+    out[i] = (up | down) & row_tail(g.R, w);
+    bits = __popc(cur);
   }
-  if (req) need[((int64_t)(k >> 3) * nb + (j >> 3)) * nb + (i >> 3)] = 1;
+  if (count) add_count(bits, count);
+}
+
+// Dilation along y (axis 1) or z (axis 2) by m.  count: the set bits of the
+// output.
+__global__ void k_dilate_rows(const uint32_t* __restrict__ in, uint32_t* __restrict__ out, CellRows g, int axis, int m,
+                              unsigned long long* count) {
+  const int64_t n = (int64_t)g.R * g.R * g.W;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  int bits = 0;
+  if (i < n) {
+    const int64_t row = i / g.W;
+    const int pos = axis == 1 ? (int)(row % g.R) : (int)(row / g.R);
+    const int64_t stride = axis == 1 ? g.W : (int64_t)g.R * g.W;
+    uint32_t v = 0u;
+    for (int p = max(pos - m, 0); p <= min(pos + m, g.R - 1); ++p) v |= in[i + (p - pos) * stride];
+    out[i] = v;
+    bits = __popc(v);
+  }
+  if (count) add_count(bits, count);
+}
+
+__global__ void k_fill_rows(uint32_t* __restrict__ out, CellRows g) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < (int64_t)g.R * g.R * g.W) out[i] = row_tail(g.R, (int)(i % g.W));
+}
+
+// The corners of a set of cells: vertex (i, j, k) is one if any of the cells
+// (i - dx, j - dy, k - dz), dx, dy, dz in {0, 1}, is in the set.
+__global__ void k_corner_rows(const uint32_t* __restrict__ cells, CellRows g, VertRows v, uint32_t* __restrict__ out) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)v.n * v.n * v.W) return;
+  const int w = (int)(i % v.W);
+  const int64_t row = i / v.W;
+  const int j = (int)(row % v.n), k = (int)(row / v.n);
+  uint32_t bits = 0u;
+#pragma unroll
+  for (int d = 0; d < 4; ++d) {
+    const int cj = j - (d & 1), ck = k - (d >> 1);
+    if (cj < 0 || ck < 0 || cj >= g.R || ck >= g.R) continue;
+    const uint32_t* r = cells + ((int64_t)ck * g.R + cj) * g.W;
+    const uint32_t c = w < g.W ? r[w] : 0u;
+    bits |= c | (c << 1) | (w > 0 ? r[w - 1] >> 31 : 0u);
+  }
+  out[i] = bits;
+}
+
+// The 8 bits of a vertex (or cell) row from position 8 b on.
+__device__ __forceinline__ uint32_t row_byte(const uint32_t* __restrict__ row, int b) {
+  return (row[b >> 2] >> (8 * (b & 3))) & 255u;
+}
+
+// Bricks that hold a required vertex: one of T, a trainable one or an axis
+// neighbour of one of T.  A thread takes one z layer of a brick, its rows'
+// neighbours in x and y, and the layers below and above for the outer two.
+__global__ void k_brick_need(const uint32_t* __restrict__ tv, const uint32_t* __restrict__ train, VertRows v, int nb,
+                             uint8_t* __restrict__ need) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (int64_t)nb * nb * nb * 8) return;
+  const int64_t b = i >> 3;
+  const int bx = (int)(b % nb), by = (int)((b / nb) % nb), bz = (int)(b / ((int64_t)nb * nb));
+  const int k = 8 * bz + (int)(i & 7);
+  if (k >= v.n) return;
+  const int R = v.n - 1;
+  uint32_t any = 0u;
+  auto row = [&](const uint32_t* s, int j, int kk) { return s + ((int64_t)kk * v.n + j) * v.W; };
+  const int j1 = min(8 * by + 7, R);
+#pragma unroll 4
+  for (int j = 8 * by; j <= j1; ++j) {
+    const uint32_t* t = row(tv, j, k);
+    any |= row_byte(t, bx) | row_byte(row(train, j, k), bx);
+    if (bx > 0) any |= row_byte(t, bx - 1) >> 7;
+    if (8 * bx + 8 <= R) any |= row_byte(t, bx + 1) & 1u;
+    if ((i & 7) == 0 && k > 0) any |= row_byte(row(tv, j, k - 1), bx);
+    if ((i & 7) == 7 && k < R) any |= row_byte(row(tv, j, k + 1), bx);
+  }
+  if (by > 0) any |= row_byte(row(tv, 8 * by - 1, k), bx);
+  if (8 * by + 8 <= R) any |= row_byte(row(tv, 8 * by + 8, k), bx);
+  if (any) need[b] = 1;
 }
 
 __device__ __forceinline__ uint32_t compact3(uint32_t x) {  // every third bit -> contiguous
@@ -164,32 +212,38 @@ __global__ void k_brick_nbr(const int32_t* __restrict__ table, const int32_t* __
   nbr[a] = v;
 }
 
-// One block of 512 threads per brick: masks by warp ballots, counts, active flag.
-__global__ void k_brick_masks(const uint8_t* __restrict__ verts, int R, const int32_t* __restrict__ coord,
-                              uint32_t* __restrict__ masks, int32_t* __restrict__ active_flag,
-                              unsigned long long* counts) {
-  int slot = blockIdx.x;
-  int l = threadIdx.x;
-  int i = coord[3 * slot] * 8 + (l & 7);
-  int j = coord[3 * slot + 1] * 8 + ((l >> 3) & 7);
-  int k = coord[3 * slot + 2] * 8 + (l >> 6);
-  int n1 = R + 1;
-  uint8_t f = 0;
-  if (i <= R && j <= R && k <= R) f = verts[((int64_t)k * n1 + j) * n1 + i];
-  uint32_t bt = __ballot_sync(0xffffffffu, f & V_T);
-  uint32_t br = __ballot_sync(0xffffffffu, f & V_TRAIN);
-  uint32_t bp = __ballot_sync(0xffffffffu, f & V_PULL);
-  int w = l >> 5;
-  if ((l & 31) == 0) {
-    uint32_t* mk = masks + (int64_t)slot * 48;
-    mk[w] = bt;
-    mk[16 + w] = br;
-    mk[32 + w] = bp;
-    if (bt) atomicAdd(counts + 2, (unsigned long long)__popc(bt));
-    if (br) atomicAdd(counts + 3, (unsigned long long)__popc(br));
+// A brick's masks, one thread per word (four rows of 8), 16 words a set.
+__global__ void __launch_bounds__(256) k_brick_masks(const uint32_t* __restrict__ tv,
+                                                     const uint32_t* __restrict__ train,
+                                                     const uint32_t* __restrict__ pull, CellRows g, VertRows v,
+                                                     const int32_t* __restrict__ coord, int64_t n_bricks,
+                                                     uint32_t* __restrict__ masks, int32_t* __restrict__ active_flag,
+                                                     unsigned long long* counts) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t slot = i >> 4;
+  const int w = (int)(i & 15);
+  uint32_t t = 0u, r = 0u, p = 0u;
+  if (slot < n_bricks) {
+    const int bx = coord[3 * slot], k = 8 * coord[3 * slot + 2] + (w >> 1);
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const int j = 8 * coord[3 * slot + 1] + 4 * (w & 1) + y;
+      if (j >= v.n || k >= v.n) continue;
+      const int64_t at = ((int64_t)k * v.n + j) * v.W;
+      t |= row_byte(tv + at, bx) << (8 * y);
+      r |= row_byte(train + at, bx) << (8 * y);
+      if (j < g.R && k < g.R && 8 * bx < g.R)
+        p |= row_byte(pull + ((int64_t)k * g.R + j) * g.W, bx) << (8 * y);
+    }
+    uint32_t* mk = masks + slot * 48;
+    mk[w] = t;
+    mk[16 + w] = r;
+    mk[32 + w] = p;
   }
-  int any = __syncthreads_or(f & V_TRAIN);
-  if (l == 0) active_flag[slot] = any ? 1 : 0;
+  const unsigned any = __ballot_sync(0xffffffffu, r != 0u);
+  if (slot < n_bricks && w == 0) active_flag[slot] = (any >> (threadIdx.x & 16)) & 0xffffu ? 1 : 0;
+  add_count(__popc(t), counts + 2);
+  add_count(__popc(r), counts + 3);
 }
 
 __global__ void k_compact_active(const int32_t* __restrict__ flags, const int32_t* __restrict__ offs, int64_t n,
@@ -296,44 +350,65 @@ gp_status build_band_sets(gp_band* b, const float* pts_dev) {
   gp_ctx* ctx = b->ctx;
   cudaStream_t s = ctx->stream;
   const int R = b->R;
-  const int64_t ncell = (int64_t)R * R * R;
-  const int64_t nvert = (int64_t)(R + 1) * (R + 1) * (R + 1);
   const int nb = b->nb;
   const int64_t nbr = (int64_t)nb * nb * nb;
   TempBufs tmp;
-  uint8_t *cA = nullptr, *cB = nullptr, *verts = nullptr, *need = nullptr;
+  const CellRows cr{R, (R + 31) / 32};
+  const VertRows vr{R + 1, (R + 32) / 32};
+  const int64_t nc = (int64_t)R * R * cr.W, nv = (int64_t)vr.n * vr.n * vr.W;
+  uint32_t *occ = nullptr, *ping = nullptr, *pong = nullptr, *s1 = nullptr, *s2 = nullptr, *sx = nullptr;
+  uint32_t *tv = nullptr, *train = nullptr;
+  uint8_t* need = nullptr;
   unsigned long long* counts = nullptr;
   gp_status st;
-  if ((st = tmp.alloc(ctx, &cA, ncell, "cell map"))) return st;
-  if ((st = tmp.alloc(ctx, &cB, ncell, "cell map"))) return st;
+  // Negative widths mean "every cell".
+  const bool all1 = b->M1 < 0, all2 = b->M2 < 0;
+  const int m1 = std::min(b->M1, R), m2 = std::min(b->M2, R);
+  if ((st = tmp.alloc(ctx, &occ, nc, "occupied cells"))) return st;
+  if ((st = tmp.alloc(ctx, &ping, nc, "cell rows"))) return st;
+  if ((st = tmp.alloc(ctx, &pong, nc, "cell rows"))) return st;
+  if ((st = tmp.alloc(ctx, &s1, nc, "pull cells"))) return st;
   if ((st = tmp.alloc(ctx, &counts, 8, "band counts"))) return st;
-  GP_CUDA(ctx, cudaMemsetAsync(cA, 0, ncell, s));
+  GP_CUDA(ctx, cudaMemsetAsync(occ, 0, nc * sizeof(uint32_t), s));
   GP_CUDA(ctx, cudaMemsetAsync(counts, 0, 8 * sizeof(unsigned long long), s));
-  GP_KERNEL(ctx, "k_mark_occupied", k_mark_occupied<<<gp_blocks(b->J, 256), 256, 0, s>>>(pts_dev, b->J, R, cA));
+  GP_KERNEL(ctx, "k_mark_occupied", k_mark_occupied<<<gp_blocks(b->J, 256), 256, 0, s>>>(pts_dev, b->J, cr, occ));
 
-  // Negative widths mean "every cell": dilate by 0 and set the bit afterwards.
-  int m1 = b->M1 < 0 ? 0 : std::min(b->M1, R);
-  int m2 = b->M2 < 0 ? 0 : std::min(b->M2, R);
-  bool all1 = b->M1 < 0, all2 = b->M2 < 0;
-  bool allx = all1 || all2;
-  int mx = allx ? 0 : std::max(m1, m2);
-  uint8_t* in = cA;
-  uint8_t* out = cB;
-  for (int axis = 0; axis < 3; ++axis) {
-    GP_KERNEL(ctx, "k_dilate_axis", k_dilate_axis<<<gp_blocks(ncell, 256), 256, 0, s>>>(in, out, R, axis, m1, m2, mx, axis == 0));
-    std::swap(in, out);
+  // The Chebyshev dilation of the occupied cells by m, one axis after another.
+  auto dilate = [&](int m, uint32_t* out, unsigned long long* n_in, unsigned long long* n_out) -> gp_status {
+    const uint32_t* in = occ;
+    for (int left = m, first = 1; first || left > 0; first = 0) {
+      const int step = std::min(left, 31);
+      GP_KERNEL(ctx, "k_dilate_x", k_dilate_x<<<gp_blocks(nc, 256), 256, 0, s>>>(in, ping, cr, step, first ? n_in : nullptr));
+      left -= step;
+      std::swap(ping, pong);
+      in = pong;
+    }
+    GP_KERNEL(ctx, "k_dilate_rows", k_dilate_rows<<<gp_blocks(nc, 256), 256, 0, s>>>(pong, ping, cr, 1, m, nullptr));
+    GP_KERNEL(ctx, "k_dilate_rows", k_dilate_rows<<<gp_blocks(nc, 256), 256, 0, s>>>(ping, out, cr, 2, m, n_out));
+    return GP_OK;
+  };
+  if ((st = dilate(all1 ? 0 : m1, s1, counts + 0, counts + 1))) return st;
+  if (all1) GP_KERNEL(ctx, "k_fill_rows", k_fill_rows<<<gp_blocks(nc, 256), 256, 0, s>>>(s1, cr));
+  s2 = s1;
+  if (all2 != all1 || (!all1 && m2 != m1)) {
+    if ((st = tmp.alloc(ctx, &s2, nc, "TV cells"))) return st;
+    if (all2)
+      GP_KERNEL(ctx, "k_fill_rows", k_fill_rows<<<gp_blocks(nc, 256), 256, 0, s>>>(s2, cr));
+    else if ((st = dilate(m2, s2, nullptr, nullptr)))
+      return st;
   }
-  uint8_t all_bits = (all1 ? C_M1 : 0) | (all2 ? C_M2 : 0) | (allx ? C_MX : 0);
-  if (all_bits) {
-    GP_KERNEL(ctx, "k_set_all_bits", k_set_all_bits<<<gp_blocks(ncell, 256), 256, 0, s>>>(in, ncell, all_bits));
+  // The trainable cells are the wider of the two sets.
+  sx = all1 || (!all2 && m1 > m2) ? s1 : s2;
+  if ((st = tmp.alloc(ctx, &tv, nv, "TV vertices"))) return st;
+  GP_KERNEL(ctx, "k_corner_rows", k_corner_rows<<<gp_blocks(nv, 256), 256, 0, s>>>(s2, cr, vr, tv));
+  train = tv;
+  if (sx != s2) {
+    if ((st = tmp.alloc(ctx, &train, nv, "trainable vertices"))) return st;
+    GP_KERNEL(ctx, "k_corner_rows", k_corner_rows<<<gp_blocks(nv, 256), 256, 0, s>>>(sx, cr, vr, train));
   }
-  GP_KERNEL(ctx, "k_count_cells", k_count_cells<<<gp_blocks(ncell, 256), 256, 0, s>>>(in, ncell, counts));
-
-  if ((st = tmp.alloc(ctx, &verts, nvert, "vertex map"))) return st;
-  GP_KERNEL(ctx, "k_vertex_flags", k_vertex_flags<<<gp_blocks(nvert, 256), 256, 0, s>>>(in, verts, R));
   if ((st = tmp.alloc(ctx, &need, nbr, "brick flags"))) return st;
   GP_CUDA(ctx, cudaMemsetAsync(need, 0, nbr, s));
-  GP_KERNEL(ctx, "k_required", k_required<<<gp_blocks(nvert, 256), 256, 0, s>>>(verts, R, nb, need));
+  GP_KERNEL(ctx, "k_brick_need", k_brick_need<<<gp_blocks(8 * nbr, 256), 256, 0, s>>>(tv, train, vr, nb, need));
 
   // Slots in Morton order of the brick coordinates.
   int nbm = 1;
@@ -358,7 +433,7 @@ gp_status build_band_sets(gp_band* b, const float* pts_dev) {
   if ((st = tmp.alloc(ctx, &aflag, n_bricks, "active flags"))) return st;
   if ((st = tmp.alloc(ctx, &aoffs, n_bricks, "active offsets"))) return st;
   if (n_bricks > 0) {
-    GP_KERNEL(ctx, "k_brick_masks", k_brick_masks<<<(unsigned)n_bricks, 512, 0, s>>>(verts, R, b->brick_coord, b->masks, aflag, counts));
+    GP_KERNEL(ctx, "k_brick_masks", k_brick_masks<<<gp_blocks(16 * n_bricks, 256), 256, 0, s>>>(tv, train, s1, cr, vr, b->brick_coord, n_bricks, b->masks, aflag, counts));
     GP_CUDA(ctx, cudaMemcpyAsync(aoffs, aflag, n_bricks * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
   }
   int64_t n_active = 0;
@@ -372,7 +447,7 @@ gp_status build_band_sets(gp_band* b, const float* pts_dev) {
   GP_CUDA(ctx, cudaMemcpyAsync(hc, counts, sizeof(hc), cudaMemcpyDeviceToHost, s));
   GP_CUDA(ctx, cudaStreamSynchronize(s));
   b->n_occ = (int64_t)hc[0];
-  b->n_pull = (int64_t)hc[1];
+  b->n_pull = all1 ? (int64_t)R * R * R : (int64_t)hc[1];
   b->V_tv = (int64_t)hc[2];
   b->V_trainable = (int64_t)hc[3];
   return GP_OK;
