@@ -21,7 +21,6 @@
 // (nn_block_cells), each taken with a rounding margin of 1e-5 (2 + |q|_inf).
 #include <algorithm>
 #include <cmath>
-#include <vector>
 
 #include "gp_internal.cuh"
 #include "gp_nn_device.cuh"
@@ -432,6 +431,94 @@ __global__ void __launch_bounds__(NN_THREADS, 8) k_nn(NNGrid g, const float* __r
   }
 }
 
+// Emission order of the spatial batches: point indices sorted by the Morton
+// code of their cell-list cell (ties by index), so that consecutive points, and
+// the queries drawn around them, stay close in all three directions.  A radix
+// sort of (code, index), 8 bits a pass from the lowest, each pass stable: the
+// digits of a tile are counted, the counts scanned over digits and tiles, and
+// the tile's pairs written in order.  (On the host, with a comparison sort of
+// 64-bit keys, the order took 4 of the 8 ms that a band of 100,000 points took
+// to build.)
+constexpr int RS_THREADS = 256, RS_WARPS = RS_THREADS / 32;
+constexpr int RS_ROUNDS = 16;                     // 32 pairs a warp and round
+constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;
+
+__device__ __forceinline__ uint32_t nn_spread3(uint32_t x) {  // bit k to bit 3 k (10 bits)
+  x = (x | x << 16) & 0x030000FFu;
+  x = (x | x << 8) & 0x0300F00Fu;
+  x = (x | x << 4) & 0x030C30C3u;
+  return (x | x << 2) & 0x09249249u;
+}
+
+__global__ void k_emit_keys(const float* __restrict__ pts, int64_t J, NNGrid g, uint32_t* __restrict__ key,
+                            int32_t* __restrict__ order) {
+  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= J) return;
+  key[j] = nn_spread3(nn_cell(pts[3 * j], g)) | nn_spread3(nn_cell(pts[3 * j + 1], g)) << 1 |
+           nn_spread3(nn_cell(pts[3 * j + 2], g)) << 2;
+  order[j] = (int32_t)j;
+}
+
+__global__ void __launch_bounds__(RS_THREADS) k_radix_count(const uint32_t* __restrict__ key, int64_t n, int shift,
+                                                            int64_t ntiles, int32_t* __restrict__ counts) {
+  __shared__ int hist[256];
+  hist[threadIdx.x] = 0;
+  __syncthreads();
+  const int64_t base = (int64_t)blockIdx.x * RS_TILE;
+  for (int k = 0; k < RS_ROUNDS; ++k) {
+    const int64_t i = base + k * RS_THREADS + threadIdx.x;
+    if (i < n) atomicAdd(hist + ((key[i] >> shift) & 255u), 1);
+  }
+  __syncthreads();
+  counts[(int64_t)threadIdx.x * ntiles + blockIdx.x] = hist[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(GP_ORDER_THREADS) k_radix_scan(int32_t* __restrict__ counts, int64_t n) {
+  gp_block_scan_inplace(counts, n);
+}
+
+__global__ void __launch_bounds__(RS_THREADS) k_radix_scatter(const uint32_t* __restrict__ key,
+                                                              const int32_t* __restrict__ val, int64_t n, int shift,
+                                                              int64_t ntiles, const int32_t* __restrict__ offs,
+                                                              uint32_t* __restrict__ key_out,
+                                                              int32_t* __restrict__ val_out) {
+  __shared__ int at[RS_WARPS][256];  // pairs of each digit per warp, then the next place of each
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int k = lane; k < 256; k += 32) at[w][k] = 0;
+  __syncwarp();
+  const int64_t base = (int64_t)blockIdx.x * RS_TILE + (int64_t)w * (32 * RS_ROUNDS) + lane;
+  for (int r = 0; r < RS_ROUNDS; ++r) {
+    const int64_t i = base + 32 * r;
+    if (i < n) atomicAdd(&at[w][(key[i] >> shift) & 255u], 1);
+  }
+  __syncthreads();
+  {
+    int run = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    for (int k = 0; k < RS_WARPS; ++k) {
+      const int c = at[k][threadIdx.x];
+      at[k][threadIdx.x] = run;
+      run += c;
+    }
+  }
+  __syncthreads();
+  for (int r = 0; r < RS_ROUNDS; ++r) {
+    const int64_t i = base + 32 * r;
+    const bool mine = i < n;
+    const uint32_t k = mine ? key[i] : 0u;
+    const int d = mine ? (int)((k >> shift) & 255u) : 256;  // lanes past the end share a digit of their own
+    const unsigned peers = __match_any_sync(0xffffffffu, d);
+    const int before = __popc(peers & ((1u << lane) - 1u));
+    const int pos = mine ? at[w][d] + before : 0;
+    __syncwarp();
+    if (mine) {
+      if (before == 0) at[w][d] = pos + __popc(peers);
+      key_out[pos] = k;
+      val_out[pos] = val[i];
+    }
+    __syncwarp();
+  }
+}
+
 // Points and sigma in emission order, for the sampler's coalesced reads.
 __global__ void k_emit_pts(const int32_t* __restrict__ order, const float* __restrict__ pts,
                            const float* __restrict__ sigma, int64_t J, float4* __restrict__ out) {
@@ -443,45 +530,41 @@ __global__ void k_emit_pts(const int32_t* __restrict__ order, const float* __res
 
 }  // namespace
 
-// Emission order of the spatial batches: point indices sorted by the Morton
-// code of their cell-list cell (ties by index), so that consecutive points, and
-// the queries drawn around them, stay close in all three directions.  Set-up
-// only: the sort runs once per cloud on the host.
-static uint64_t spread3(uint64_t x) {
-  x &= 0x1fffff;
-  x = (x | x << 32) & 0x1f00000000ffffull;
-  x = (x | x << 16) & 0x1f0000ff0000ffull;
-  x = (x | x << 8) & 0x100f00f00f00f00full;
-  x = (x | x << 4) & 0x10c30c30c30c30c3ull;
-  x = (x | x << 2) & 0x1249249249249249ull;
-  return x;
-}
-
 static gp_status build_emit_order(gp_band* b) {
   gp_ctx* ctx = b->ctx;
-  const int64_t J = b->J;
-  std::vector<float> pts((size_t)(3 * J));
-  GP_CUDA(ctx, cudaMemcpyAsync(pts.data(), b->pts, 3 * J * sizeof(float), cudaMemcpyDeviceToHost, ctx->stream));
-  GP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  const float half_g = 0.5f * (float)b->G;
-  std::vector<uint64_t> key((size_t)J);
-  for (int64_t j = 0; j < J; ++j) {
-    uint64_t c[3];
-    for (int a = 0; a < 3; ++a) {
-      float t = (pts[3 * j + a] + 1.0f) * half_g;
-      int ci = (t < 0.f) ? 0 : (int)std::floor(std::fmin(t, 1.0e6f));
-      c[a] = (uint64_t)std::min(std::max(ci, 0), b->G - 1);
+  cudaStream_t s = ctx->stream;
+  const int64_t J = b->J, ntiles = (J + RS_TILE - 1) / RS_TILE;
+  int bits = 0;  // per axis
+  while ((1 << bits) < b->G) ++bits;
+  uint32_t* key[2] = {nullptr, nullptr};
+  int32_t *val[2] = {nullptr, nullptr}, *counts = nullptr;
+  gp_status st = gp_alloc(ctx, &val[0], J, "emission order");
+  if (!st) st = gp_alloc(ctx, &val[1], J, "emission order");
+  if (!st) st = gp_alloc(ctx, &key[0], J, "emission keys");
+  if (!st) st = gp_alloc(ctx, &key[1], J, "emission keys");
+  if (!st) st = gp_alloc(ctx, &counts, 256 * ntiles, "emission digit counts");
+  cudaError_t e = cudaSuccess;
+  int cur = 0;
+  if (!st) {
+    k_emit_keys<<<gp_blocks(J, 256), 256, 0, s>>>(b->pts, J, make_grid(b), key[0], val[0]);
+    for (int shift = 0; shift < 3 * bits; shift += 8, cur ^= 1) {
+      k_radix_count<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(key[cur], J, shift, ntiles, counts);
+      k_radix_scan<<<1, GP_ORDER_THREADS, 0, s>>>(counts, 256 * ntiles);
+      k_radix_scatter<<<(unsigned)ntiles, RS_THREADS, 0, s>>>(key[cur], val[cur], J, shift, ntiles, counts,
+                                                             key[cur ^ 1], val[cur ^ 1]);
     }
-    uint64_t m = spread3(c[0]) | (spread3(c[1]) << 1) | (spread3(c[2]) << 2);
-    key[(size_t)j] = (m << 31) | (uint64_t)j;  // Morton code (<= 30 bits), then index
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  std::sort(key.begin(), key.end());
-  std::vector<int32_t> order((size_t)J);
-  for (int64_t t = 0; t < J; ++t) order[(size_t)t] = (int32_t)(key[(size_t)t] & 0x7fffffffull);
-  gp_status st = gp_alloc(ctx, &b->emit_order, J, "emission order");
-  if (st) return st;
-  GP_CUDA(ctx, cudaMemcpyAsync(b->emit_order, order.data(), J * sizeof(int32_t), cudaMemcpyHostToDevice, ctx->stream));
-  GP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+  gp_free(key[0]);
+  gp_free(key[1]);
+  gp_free(counts);
+  gp_free(val[cur ^ 1]);
+  if (st || e != cudaSuccess) {
+    gp_free(val[cur]);
+    return st ? st : gp_cuda_fail(ctx, e, "emission order");
+  }
+  b->emit_order = val[cur];
   return GP_OK;
 }
 
