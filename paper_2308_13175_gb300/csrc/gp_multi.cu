@@ -312,10 +312,9 @@ struct MultiTvSrc {
   }
 };
 
-// L_TV sweep: one brick per tile (TV_SWEEP_THREADS threads, pipelined across
-// the block's tiles); the gradient is overwritten at every slot of every
-// brick; the TV sums go to each cloud's slot 3, one atomic per run of tiles of
-// the same cloud.
+// L_TV sweep: one brick per tile, the tiles dealt to the warps (tv_sweep); the
+// gradient is overwritten at every slot of every brick; the TV sums go to each
+// cloud's slot 3, one atomic per warp and run of tiles of the same cloud.
 // DET: the query pass ran first into the fixed-point sums (its contributions
 // already scaled by 1/B_v of the cloud), which are folded in here and
 // cleared; the TV sums go to the integer loss sums.
@@ -325,76 +324,62 @@ __global__ void __launch_bounds__(TV_SWEEP_THREADS, TV_BLOCKS_PER_SM) k_m_tv(con
                                                            float alpha, double* __restrict__ sums,
                                                            long long* __restrict__ isums) {
   __shared__ TvShared sh;
-  __shared__ float red[32];
   int cur = -1;
   float acc = 0.f;
   auto flush = [&]() {
-    const float bs = block_sum(acc, red);
-    if (threadIdx.x == 0 && bs != 0.f) {
+    const float ws = gp_warp_sum(acc);
+    if ((threadIdx.x & 31) == 0 && ws != 0.f) {
       if (DET)
-        atomicAdd((unsigned long long*)(isums + 4 * cur + 3), (unsigned long long)loss_fixed(bs));
+        atomicAdd((unsigned long long*)(isums + 4 * cur + 3), (unsigned long long)loss_fixed(ws));
       else
-        atomicAdd(sums + 4 * cur + 3, (double)bs);
+        atomicAdd(sums + 4 * cur + 3, (double)ws);
     }
     acc = 0.f;
   };
-  // DET: this thread's two vertices of each brick (those tv_gather hands
-  // it) have their fixed-point sums loaded at the top of the brick's
-  // iteration, under its halo copies; only trainable vertices can hold any.
-  const int tt = threadIdx.x;
-  const int lv0 = (tt & 7) + 16 * ((tt >> 3) & 3) + 64 * (tt >> 5);
-  long long phi[2] = {0, 0}, plo[2] = {0, 0};
-  bool ptr[2] = {false, false};
-  auto out = [&](int64_t ti, int l0, float g0, int l1, float g1, float ts) {
-        const MTile tl = tiles[ti];
-        const MShape& S = shapes[tl.shape];
-        if (tl.shape != cur) {
-          if (cur >= 0) flush();
-          cur = tl.shape;
-        }
-        acc += ts;
-        const float tv_scale = S.V_tv > 0 ? alpha / (float)S.V_tv : 0.f;
-        float* gp = S.grad + (int64_t)tl.first * 512;
-        if (DET) {
-          unsigned long long* ap = S.acc + 2 * (int64_t)tl.first * 512;
-          const int ls[2] = {l0, l1};
-          const float gs[2] = {g0, g1};
+  // DET: only trainable vertices can hold fixed-point sums.
+  struct Quad {
+    uint32_t bits;
+    longlong2 f[4];
+  };
+  auto fetch = [&](int64_t ti, int q) {
+    Quad o;
+    if (DET) {
+      const MTile tl = tiles[ti];
+      const MShape& S = shapes[tl.shape];
+      o.bits = (__ldg(S.G.masks + (int64_t)tl.first * 48 + 16 + (q >> 3)) >> ((4 * q) & 31)) & 15u;
+      const unsigned long long* ap = S.acc + 2 * ((int64_t)tl.first * 512 + 4 * q);
+      if (o.bits) {
 #pragma unroll
-          for (int k = 0; k < 2; ++k) {
-            float g = tv_scale * gs[k];
-            if (ptr[k]) {
-              ap[2 * ls[k]] = 0ull;
-              ap[2 * ls[k] + 1] = 0ull;
-              const float qv = __fmaf_rn(__ll2float_rn(phi[k]), 9.5367431640625e-07f,
-                                         __ll2float_rn(plo[k]) * 8.673617379884035e-19f);
-              g = __fadd_rn(qv, g);
-            }
-            gp[ls[k]] = g;
-          }
-        } else {
-          gp[l0] = tv_scale * g0;
-          gp[l1] = tv_scale * g1;
-        }
-      };
-  auto pre = [&](int64_t ti) {
-        const MTile tl = tiles[ti];
-        const MShape& S = shapes[tl.shape];
-        const unsigned long long* ap = S.acc + 2 * (int64_t)tl.first * 512;
+        for (int k = 0; k < 4; ++k) o.f[k] = reinterpret_cast<const longlong2*>(ap)[k];
+      }
+    }
+    return o;
+  };
+  auto out = [&](int64_t ti, int q, float4, float4 g, const Quad& o) {
+    const MTile tl = tiles[ti];
+    const MShape& S = shapes[tl.shape];
+    const float sc = S.V_tv > 0 ? alpha / (float)S.V_tv : 0.f;
+    const int64_t at = (int64_t)tl.first * 512 + 4 * q;
+    float v[4] = {sc * g.x, sc * g.y, sc * g.z, sc * g.w};
+    if (DET && o.bits) {
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-          const int l = lv0 + 8 * k;
-          const uint32_t word = __ldg(S.G.masks + (int64_t)tl.first * 48 + 16 + (l >> 5));
-          ptr[k] = (word >> (l & 31)) & 1u;
-          if (ptr[k]) {
-            phi[k] = (long long)ap[2 * l];
-            plo[k] = (long long)ap[2 * l + 1];
-          }
-        }
-      };
-  if constexpr (DET)
-    tv_sweep(MultiTvSrc{shapes, tiles}, blockIdx.x, gridDim.x, ntiles, sh, out, pre);
-  else
-    tv_sweep(MultiTvSrc{shapes, tiles}, blockIdx.x, gridDim.x, ntiles, sh, out);
+      for (int k = 0; k < 4; ++k) {
+        if (!((o.bits >> k) & 1u)) continue;
+        reinterpret_cast<longlong2*>(S.acc + 2 * at)[k] = longlong2{0, 0};
+        v[k] = __fadd_rn(__fmaf_rn(__ll2float_rn(o.f[k].x), 9.5367431640625e-07f,
+                                   __ll2float_rn(o.f[k].y) * 8.673617379884035e-19f), v[k]);
+      }
+    }
+    *reinterpret_cast<float4*>(S.grad + at) = make_float4(v[0], v[1], v[2], v[3]);
+  };
+  tv_sweep<true>(MultiTvSrc{shapes, tiles}, ntiles, sh, fetch, out, [&](int64_t ti, float ts) {
+    const int shape = tiles[ti].shape;
+    if (shape != cur) {
+      if (cur >= 0) flush();
+      cur = shape;
+    }
+    acc += ts;
+  });
   if (cur >= 0) flush();
 }
 
@@ -581,7 +566,7 @@ gp_status launch_nn(gp_multi* m) {
 
 gp_status launch_tv(gp_multi* m, const gp_loss_w* w) {
   gp_ctx* ctx = m->ctx;
-  const unsigned grid = persistent_grid(m, m->bpsm[ST_TV], m->n_brick_tiles);
+  const unsigned grid = persistent_grid(m, m->bpsm[ST_TV], (m->n_brick_tiles + TV_SWEEP_WARPS - 1) / TV_SWEEP_WARPS);
   if (m->acc)
     GP_KERNEL(ctx, "k_m_tv",
               k_m_tv<true><<<grid, TV_SWEEP_THREADS, 0, ctx->stream>>>(m->shapes, m->brick_tiles, m->n_brick_tiles,

@@ -22,7 +22,6 @@
 #include "gp_internal.cuh"
 #include "gp_step_device.cuh"
 #include "gp_query_win.cuh"
-#include "gp_tv2.cuh"
 
 namespace {
 
@@ -344,12 +343,6 @@ cudaError_t launch_query_tuned(const gp_band* b, int64_t B, cudaStream_t s, Grid
   return launch_query_ilp<DET, LAST, 1, 3>(ctx, B, s, G, rec, bv, beta, gamma, grad, acc, partials, err, fa);
 }
 
-// The L_TV sweep over the band's bricks (tv_sweep: one brick at a time per
-// block of TV_THREADS, one persistent wave of blocks, the next brick's halo
-// copied while the current one is computed).  Writes the gradient of every
-// stored slot: alpha/|T| * dTV/dd_i (+ the fixed-point query sums in
-// deterministic mode, which are cleared for the next step).  Each TV_i enters
-// the loss sum once, from the brick that stores i.
 struct BandTvSrc {
   Grid G;
   const int32_t* coord;
@@ -360,201 +353,85 @@ struct BandTvSrc {
   }
 };
 
+// The fixed-point sums of a quad (4 vertices, two words each): loaded, turned
+// into float32, cleared.
+struct FixQuad {
+  longlong2 v[4];
+};
+__device__ __forceinline__ FixQuad fix_load(const unsigned long long* __restrict__ acc, int64_t vertex) {
+  FixQuad f;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) f.v[k] = *reinterpret_cast<const longlong2*>(acc + 2 * (vertex + k));
+  return f;
+}
+// hi 2^-20 + lo 2^-60 in float32 (the scales are exact powers of two): the
+// same operations on the same integers, so bit-reproducible.  The query pass
+// added its contributions already scaled by 1/B_v.
+__device__ __forceinline__ float fix_value(longlong2 v) {
+  return __fmaf_rn(__ll2float_rn(v.x), 9.5367431640625e-07f, __ll2float_rn(v.y) * 8.673617379884035e-19f);
+}
+__device__ __forceinline__ void fix_clear(unsigned long long* __restrict__ acc, int64_t vertex) {
+  *reinterpret_cast<longlong2*>(acc + 2 * vertex) = longlong2{0, 0};
+}
+
+// The block's sum of TV_i into partials[block * 8 + 3].
+__device__ __forceinline__ void store_tv_sum(double* __restrict__ partials, float tsum) {
+  __shared__ float red[TV_SWEEP_WARPS];
+  const float w = gp_warp_sum(tsum);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double sum = 0;
+    for (int k = 0; k < TV_SWEEP_WARPS; ++k) sum += red[k];
+    partials[(int64_t)blockIdx.x * 8 + 3] = sum;
+  }
+}
+
+// L_TV over the band's bricks (tv_sweep, one persistent wave of blocks).
+// GRAD: writes the gradient of every stored slot, alpha/|T| dTV/dd (0 without
+// TV), DET plus the fixed-point query sums, which are cleared for the next
+// step.  Each TV_i enters the loss sum once, from the brick that stores i.
+// LAST: this kernel writes the loss slots.
+//
+// Measured (GB300), against two passes that stored 1/TV per slot (20 bytes a
+// slot and 13 shared words a vertex, a thread per vertex): 127,169 bricks (a
+// 10 M-point scene) 430 -> 351 us, 4,661 bricks 19.5 -> 16.9.
 template <bool DET, bool GRAD, bool TV, bool LAST>
 __global__ void __launch_bounds__(TV_THREADS, TV_BLOCKS_PER_SM) k_tv(Grid G, const int32_t* __restrict__ coord,
                                                    const int32_t* __restrict__ nbrs, int64_t n_bricks,
                                                    float tv_scale, float* __restrict__ grad,
                                                    unsigned long long* __restrict__ acc,
-                                                   double* __restrict__ partials, int32_t* __restrict__ err,
-                                                   FinalArgs fa) {
-  __shared__ TvShared sh;
+                                                   double* __restrict__ partials, FinalArgs fa) {
   float tsum = 0.f;
-  const int l = threadIdx.x;
-  auto emit = [&](int64_t addr, float gv) {
-    if (!GRAD) return;
+  auto fetch = [&](int64_t slot, int q) {
+    FixQuad f;
+    if (DET) f = fix_load(acc, slot * 512 + 4 * q);
+    return f;
+  };
+  auto emit = [&](int64_t slot, int q, float4 g, const FixQuad& f) {
+    const int64_t at = slot * 512 + 4 * q;
+    float v[4] = {tv_scale * g.x, tv_scale * g.y, tv_scale * g.z, tv_scale * g.w};
     if (DET) {
-      long long hi = (long long)acc[2 * addr], lo = (long long)acc[2 * addr + 1];
-      acc[2 * addr] = 0ull;
-      acc[2 * addr + 1] = 0ull;
-      // hi 2^-20 + lo 2^-60 in float32 (the scales are exact powers of two):
-      // the same operations on the same integers, so still bit-reproducible.
-      // The query pass added its contributions already scaled by 1/B_v.
-      const float qv = __fmaf_rn(__ll2float_rn(hi), 9.5367431640625e-07f, __ll2float_rn(lo) * 8.673617379884035e-19f);
-      gv = __fadd_rn(qv, gv);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        v[k] = __fadd_rn(fix_value(f.v[k]), v[k]);
+        fix_clear(acc, at + k);
+      }
     }
-    grad[addr] = gv;
+    *reinterpret_cast<float4*>(grad + at) = make_float4(v[0], v[1], v[2], v[3]);
   };
   if (TV) {
-    tv_sweep(BandTvSrc{G, coord, nbrs}, blockIdx.x, gridDim.x, n_bricks, sh,
-             [&](int64_t slot, int l0, float g0, int l1, float g1, float ts) {
-               tsum += ts;
-               emit(slot * 512 + l0, tv_scale * g0);
-               emit(slot * 512 + l1, tv_scale * g1);
-             });
-  } else {
-    for (int64_t slot = blockIdx.x; slot < n_bricks; slot += gridDim.x) {
-      emit(slot * 512 + l, 0.f);
-      emit(slot * 512 + l + 256, 0.f);
-    }
+    __shared__ TvShared sh;
+    tv_sweep<GRAD>(
+        BandTvSrc{G, coord, nbrs}, n_bricks, sh, fetch,
+        [&](int64_t slot, int q, float4, float4 g, const FixQuad& f) { emit(slot, q, g, f); },
+        [&](int64_t, float ts) { tsum += ts; });
+  } else if (GRAD) {
+    const int64_t n = n_bricks * 128;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+      emit(i >> 7, (int)(i & 127), make_float4(0.f, 0.f, 0.f, 0.f), fetch(i >> 7, (int)(i & 127)));
   }
-  // block reduction of the TV sum into partials[block*8 + 3]
-  __shared__ float red[TV_THREADS / 32];
-  float w = gp_warp_sum(tsum);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = w;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sum = 0;
-    for (int k = 0; k < TV_THREADS / 32; ++k) sum += red[k];
-    partials[(int64_t)blockIdx.x * 8 + 3] = sum;
-  }
-  if (LAST) finish_if_last(partials, fa);
-  (void)err;
-}
-
-// The two-pass L_TV of gp_step (gp_tv2.cuh).  Each block walks bricks
-// blockIdx.x, + gridDim.x, ...: the next brick's copies are issued into the
-// other of two stage buffers (cp.async) before the current one is computed,
-// and the brick after that has its neighbour slots read meanwhile.
-//
-// Pass 1: 1/TV_i of every T vertex into inv (0 at every other slot), the
-// block's sum of TV_i into partials[block*8 + 3].  The 6 squared differences
-// are summed in the order of the single-sweep form (-x, +x, -y, +y, -z, +z),
-// so inv is the same.
-constexpr int TV2_INV_BLOCKS_PER_SM = 16;
-constexpr int TV2_GRAD_BLOCKS_PER_SM = 12;
-__global__ void __launch_bounds__(TV2_THREADS, TV2_INV_BLOCKS_PER_SM)
-    k_tv_inv(Grid G, const int32_t* __restrict__ coord, const int32_t* __restrict__ nbrs, int64_t n_bricks,
-             float* __restrict__ inv, double* __restrict__ partials) {
-  __shared__ Tv2Stage s[2];
-  __shared__ __align__(16) uint32_t Tw[2][16];
-  const int t = threadIdx.x, x = t & 7, y = t >> 3;
-  float tsum = 0.f;
-  const int64_t first = blockIdx.x, stride = gridDim.x;
-  auto issue = [&](int p, const Tv2Brick& k) {
-    tv2_issue(s[p], G.D, k);
-    if (t < 4) cp_async_cg16(&Tw[p][4 * t], G.masks + k.slot * 48 + 4 * t, 16);
-  };
-  Tv2Brick cur, nxt;
-  if (first < n_bricks) {
-    cur = tv2_brick(coord, nbrs, first);
-    issue(0, cur);
-  }
-  cp_async_commit();
-  if (first + stride < n_bricks) nxt = tv2_brick(coord, nbrs, first + stride);
-  int p = 0;
-  for (int64_t b = first; b < n_bricks; b += stride) {
-    if (b + stride < n_bricks) issue(p ^ 1, nxt);
-    cp_async_commit();
-    Tv2Brick after;
-    if (b + 2 * stride < n_bricks) after = tv2_brick(coord, nbrs, b + 2 * stride);
-    cp_async_wait1();  // this thread's copies of brick b have landed
-    __syncthreads();   // ... and everyone's
-    const Tv2Stage& S = s[p];
-#pragma unroll 2
-    for (int z = 0; z < 8; ++z) {
-      const int l = (z * 8 + y) * 8 + x;
-      float iv = 0.f;
-      if ((Tw[p][z * 2 + (y >> 2)] >> ((y & 3) * 8 + x)) & 1u) {
-        float n[6];
-        bool ok[6];
-        tv2_nbrs(S, x, y, z, n);
-        tv2_ingrid(cur.ox + x, cur.oy + y, cur.oz + z, G.R, ok);
-        const float d = S.c[l];
-        float s2 = 0.f;
-#pragma unroll
-        for (int j = 0; j < 6; ++j) {
-          const float e = d - n[j];
-          if (ok[j]) s2 = fmaf(e, e, s2);
-        }
-        iv = s2 > 0.f ? rsqrtf(s2) : 0.f;
-        tsum += s2 * iv;
-      }
-      inv[b * 512 + l] = iv;
-    }
-    __syncthreads();  // buffer p is free for the copies of brick b + 2 stride
-    cur = nxt;
-    nxt = after;
-    p ^= 1;
-  }
-  cp_async_wait0();
-  __shared__ float red[TV2_THREADS / 32];
-  const float w = gp_warp_sum(tsum);
-  if ((t & 31) == 0) red[t >> 5] = w;
-  __syncthreads();
-  if (t == 0) {
-    double sum = 0;
-    for (int k = 0; k < TV2_THREADS / 32; ++k) sum += red[k];
-    partials[(int64_t)blockIdx.x * 8 + 3] = sum;
-  }
-}
-
-// Pass 2: the gradient of every stored slot, alpha/|T| dTV/dd (0 outside the
-// grid), plus, DET, the fixed-point query sums (folded and cleared), in the
-// single-sweep form's order of terms.  LAST: this kernel writes the loss slots.
-template <bool DET, bool LAST>
-__global__ void __launch_bounds__(TV2_THREADS, TV2_GRAD_BLOCKS_PER_SM)
-    k_tv_grad(Grid G, const int32_t* __restrict__ coord, const int32_t* __restrict__ nbrs, int64_t n_bricks,
-              const float* __restrict__ inv, float tv_scale, float* __restrict__ grad,
-              unsigned long long* __restrict__ acc, double* __restrict__ partials, FinalArgs fa) {
-  __shared__ Tv2Stage sd[2], si[2];
-  const int t = threadIdx.x, x = t & 7, y = t >> 3;
-  const int64_t first = blockIdx.x, stride = gridDim.x;
-  auto issue = [&](int p, const Tv2Brick& k) {
-    tv2_issue(sd[p], G.D, k);
-    tv2_issue(si[p], inv, k);
-  };
-  Tv2Brick cur, nxt;
-  if (first < n_bricks) {
-    cur = tv2_brick(coord, nbrs, first);
-    issue(0, cur);
-  }
-  cp_async_commit();
-  if (first + stride < n_bricks) nxt = tv2_brick(coord, nbrs, first + stride);
-  int p = 0;
-  for (int64_t b = first; b < n_bricks; b += stride) {
-    if (b + stride < n_bricks) issue(p ^ 1, nxt);
-    cp_async_commit();
-    Tv2Brick after;
-    if (b + 2 * stride < n_bricks) after = tv2_brick(coord, nbrs, b + 2 * stride);
-    cp_async_wait1();
-    __syncthreads();
-    const Tv2Stage& SD = sd[p];
-    const Tv2Stage& SI = si[p];
-#pragma unroll 2
-    for (int z = 0; z < 8; ++z) {
-      const int l = (z * 8 + y) * 8 + x;
-      const int X = cur.ox + x, Y = cur.oy + y, Z = cur.oz + z;
-      float nd[6], ni[6];
-      bool ok[6];
-      tv2_nbrs(SD, x, y, z, nd);
-      tv2_nbrs(SI, x, y, z, ni);
-      tv2_ingrid(X, Y, Z, G.R, ok);
-      const float d = SD.c[l], own = SI.c[l];
-      float g = 0.f;
-#pragma unroll
-      for (int j = 0; j < 6; ++j) {
-        // own != 0 only for T vertices, whose in-grid neighbours are all
-        // stored; ni[j] != 0 only for neighbours in T.
-        if (ok[j]) g = fmaf(d - nd[j], own + ni[j], g);
-      }
-      float gv = (X <= G.R && Y <= G.R && Z <= G.R) ? tv_scale * g : 0.f;
-      const int64_t addr = b * 512 + l;
-      if (DET) {
-        const long long hi = (long long)acc[2 * addr], lo = (long long)acc[2 * addr + 1];
-        acc[2 * addr] = 0ull;
-        acc[2 * addr + 1] = 0ull;
-        const float qv =
-            __fmaf_rn(__ll2float_rn(hi), 9.5367431640625e-07f, __ll2float_rn(lo) * 8.673617379884035e-19f);
-        gv = __fadd_rn(qv, gv);
-      }
-      grad[addr] = gv;
-    }
-    __syncthreads();
-    cur = nxt;
-    nxt = after;
-    p ^= 1;
-  }
-  cp_async_wait0();
+  store_tv_sum(partials, tsum);
   if (LAST) finish_if_last(partials, fa);
 }
 
@@ -574,85 +451,61 @@ struct AdamArgs {
 template <bool DET, bool TV>
 __global__ void __launch_bounds__(TV_THREADS, TV_BLOCKS_PER_SM) k_tv_adam(
     Grid G, const int32_t* __restrict__ coord, const int32_t* __restrict__ nbrs, int64_t n_bricks, float tv_scale,
-    float* __restrict__ qgrad, unsigned long long* __restrict__ acc, float* __restrict__ Dnext, float* __restrict__ m, float* __restrict__ v, AdamArgs ad,
-    double* __restrict__ partials, int32_t* __restrict__ err, FinalArgs fa) {
-  __shared__ TvShared sh;
-  float tsum = 0.f;
-  // This thread's two vertices of every brick (those tv_gather hands it), and
-  // their Adam operands, loaded at the top of the brick's iteration.
-  const int tt = threadIdx.x;
-  const int lv[2] = {(tt & 7) + 16 * ((tt >> 3) & 3) + 64 * (tt >> 5), (tt & 7) + 16 * ((tt >> 3) & 3) + 64 * (tt >> 5) + 8};
-  float pd[2], pm[2], pv[2], pq[2];
-  uint32_t pw[2];
-  auto load = [&](int64_t slot, int k, int l) {
-    const int64_t addr = slot * 512 + l;
-    pd[k] = __ldg(G.D + addr);
-    pw[k] = __ldg(G.masks + slot * 48 + 16 + (l >> 5));
-    if ((pw[k] >> (l & 31)) & 1u) {
-      pm[k] = m[addr];
-      pv[k] = v[addr];
-      if (DET) {
-        const long long hi = (long long)acc[2 * addr], lo = (long long)acc[2 * addr + 1];
-        const float qv =
-            __fmaf_rn(__ll2float_rn(hi), 9.5367431640625e-07f, __ll2float_rn(lo) * 8.673617379884035e-19f);
-        pq[k] = qv;  // already scaled by 1/B_v by the query pass
-      } else {
-        pq[k] = qgrad[addr];
-      }
-    }
+    float* __restrict__ qgrad, unsigned long long* __restrict__ acc, float* __restrict__ Dnext, float* __restrict__ m,
+    float* __restrict__ v, AdamArgs ad, double* __restrict__ partials, FinalArgs fa) {
+  struct Quad {
+    uint32_t bits;  // trainable vertices
+    float4 m, v, q;
+    FixQuad f;
   };
-  auto update = [&](int64_t slot, int k, int l, float g_tv) {
-    const int64_t addr = slot * 512 + l;
-    if (!((pw[k] >> (l & 31)) & 1u)) {
-      Dnext[addr] = pd[k];
-      return;
+  float tsum = 0.f;
+  auto fetch = [&](int64_t slot, int q) {
+    const int64_t at = slot * 512 + 4 * q;
+    Quad o;
+    o.bits = (__ldg(G.masks + slot * 48 + 16 + (q >> 3)) >> ((4 * q) & 31)) & 15u;
+    if (o.bits) {
+      o.m = *reinterpret_cast<const float4*>(m + at);
+      o.v = *reinterpret_cast<const float4*>(v + at);
+      if (DET)
+        o.f = fix_load(acc, at);
+      else
+        o.q = *reinterpret_cast<const float4*>(qgrad + at);
     }
-    float g;
-    if (DET) {
-      acc[2 * addr] = 0ull;
-      acc[2 * addr + 1] = 0ull;
-      g = __fadd_rn(pq[k], tv_scale * g_tv);
-    } else {
-      qgrad[addr] = 0.f;
-      g = tv_scale * g_tv + pq[k];
+    return o;
+  };
+  auto update = [&](int64_t slot, int q, float4 d, float4 g, Quad& o) {
+    const int64_t at = slot * 512 + 4 * q;
+    if (o.bits) {
+      float* mp = reinterpret_cast<float*>(&o.m);
+      float* vp = reinterpret_cast<float*>(&o.v);
+      float* dp = reinterpret_cast<float*>(&d);
+      const float gt[4] = {tv_scale * g.x, tv_scale * g.y, tv_scale * g.z, tv_scale * g.w};
+      const float qv[4] = {o.q.x, o.q.y, o.q.z, o.q.w};
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (!((o.bits >> k) & 1u)) continue;
+        const float gk = DET ? __fadd_rn(fix_value(o.f.v[k]), gt[k]) : gt[k] + qv[k];
+        if (DET) fix_clear(acc, at + k);
+        dp[k] = adam_elem(gk, mp[k], vp[k], dp[k], ad.lr, ad.b1, ad.b2, ad.eps, ad.ibc1, ad.ibc2);
+      }
+      *reinterpret_cast<float4*>(m + at) = o.m;
+      *reinterpret_cast<float4*>(v + at) = o.v;
+      if (!DET) *reinterpret_cast<float4*>(qgrad + at) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    float mm = pm[k], vv = pv[k];
-    const float dn = adam_elem(g, mm, vv, pd[k], ad.lr, ad.b1, ad.b2, ad.eps, ad.ibc1, ad.ibc2);
-    m[addr] = mm;
-    v[addr] = vv;
-    Dnext[addr] = dn;
+    *reinterpret_cast<float4*>(Dnext + at) = d;
   };
   if (TV) {
-    tv_sweep(
-        BandTvSrc{G, coord, nbrs}, blockIdx.x, gridDim.x, n_bricks, sh,
-        [&](int64_t slot, int l0, float g0, int l1, float g1, float ts) {
-          tsum += ts;
-          update(slot, 0, l0, g0);
-          update(slot, 1, l1, g1);
-        },
-        [&](int64_t slot) {
-          load(slot, 0, lv[0]);
-          load(slot, 1, lv[1]);
-        });
+    __shared__ TvShared sh;
+    tv_sweep<true>(BandTvSrc{G, coord, nbrs}, n_bricks, sh, fetch, update, [&](int64_t, float ts) { tsum += ts; });
   } else {
-    for (int64_t slot = blockIdx.x; slot < n_bricks; slot += gridDim.x) {
-      load(slot, 0, threadIdx.x);
-      load(slot, 1, threadIdx.x + 256);
-      update(slot, 0, threadIdx.x, 0.f);
-      update(slot, 1, threadIdx.x + 256, 0.f);
+    const int64_t n = n_bricks * 128;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+      Quad o = fetch(i >> 7, (int)(i & 127));
+      update(i >> 7, (int)(i & 127), __ldg(reinterpret_cast<const float4*>(G.D) + i), make_float4(0.f, 0.f, 0.f, 0.f), o);
     }
   }
-  __shared__ float red[TV_THREADS / 32];
-  const float wsum = gp_warp_sum(tsum);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = wsum;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double sum = 0;
-    for (int k = 0; k < TV_THREADS / 32; ++k) sum += red[k];
-    partials[(int64_t)blockIdx.x * 8 + 3] = sum;
-  }
+  store_tv_sum(partials, tsum);
   finish_if_last(partials, fa);
-  (void)err;
 }
 
 // One thread per 4 consecutive vertices of an active brick (128 per brick).
@@ -673,16 +526,10 @@ unsigned q_grid(const gp_ctx* ctx, int64_t B) {
   return gp_blocks(B, Q_THREADS, cap);
 }
 
-unsigned tv2_grid(const gp_ctx* ctx, int64_t n_bricks, int per_sm) {
-  int64_t cap = (int64_t)ctx->num_sms * per_sm;
-  if (cap > GP_MAX_PARTIAL_BLOCKS) cap = GP_MAX_PARTIAL_BLOCKS;
-  return gp_blocks(n_bricks, 1, cap);
-}
-
 unsigned tv_grid(const gp_ctx* ctx, int64_t n_bricks) {
   int64_t cap = (int64_t)ctx->num_sms * TV_BLOCKS_PER_SM;  // persistent: one wave
   if (cap > GP_MAX_PARTIAL_BLOCKS) cap = GP_MAX_PARTIAL_BLOCKS;
-  return gp_blocks(n_bricks, 1, cap);
+  return gp_blocks(n_bricks, TV_SWEEP_WARPS, cap);
 }
 
 }  // namespace
@@ -729,7 +576,7 @@ extern "C" gp_status gp_step(gp_band* b, const float* rec_dev, int64_t B, const 
   FinalArgs fa;
   fa.done = b->dev_ints + GP_DI_DONE;
   fa.q_blocks = (int)qb;
-  fa.tv_blocks = (int)tb;
+  fa.tv_blocks = !tv_on && !grad_on ? 1 : (int)tb;
   fa.bv = bv;
   fa.n_tv = b->V_tv;
   fa.alpha = w->alpha;
@@ -741,44 +588,27 @@ extern "C" gp_status gp_step(gp_band* b, const float* rec_dev, int64_t B, const 
   // it; in deterministic mode the query pass fills the fixed-point sums first
   // and the sweep folds them in.  Whichever runs second writes the loss.
   const bool tv_last = det && grad_on;
-  const unsigned tb2 = b->n_bricks ? tv2_grid(ctx, b->n_bricks, TV2_INV_BLOCKS_PER_SM) : 1;
-  const unsigned tg2 = b->n_bricks ? tv2_grid(ctx, b->n_bricks, TV2_GRAD_BLOCKS_PER_SM) : 1;
-  if (tv_on) fa.tv_blocks = (int)tb2;
   auto launch_tv = [&]() -> gp_status {
     if (b->n_bricks == 0) {
       GP_CUDA(ctx, cudaMemsetAsync(b->partials + 3, 0, sizeof(double), s));
       return GP_OK;
     }
-    if (tv_on) {
-      // Two passes: 1/TV of the T vertices, then the gradient of every slot.
-      GP_KERNEL(ctx, "k_tv_inv",
-                k_tv_inv<<<tb2, TV2_THREADS, 0, s>>>(G, b->brick_coord, b->brick_nbr, b->n_bricks, b->tv_inv,
-                                                      b->partials));
-      if (!grad_on) return GP_OK;
-#define GP_TV2(D_, L_)                                                                                          \
-  k_tv_grad<D_, L_><<<tg2, TV2_THREADS, 0, s>>>(G, b->brick_coord, b->brick_nbr, b->n_bricks, b->tv_inv, tv_scale, \
-                                                grad_dev, b->acc, b->partials, fa)
-      if (tv_last)
-        GP_KERNEL(ctx, "k_tv_grad", GP_TV2(true, true));
-      else
-        GP_KERNEL(ctx, "k_tv_grad", GP_TV2(false, false));
-#undef GP_TV2
+    if (!tv_on && !grad_on) {  // no sweep: no sums
+      GP_CUDA(ctx, cudaMemsetAsync(b->partials + 3, 0, sizeof(double), s));
       return GP_OK;
     }
 #define GP_TV(D_, G_, T_, L_)                                                                                  \
   k_tv<D_, G_, T_, L_><<<tb, TV_THREADS, 0, s>>>(G, b->brick_coord, b->brick_nbr, b->n_bricks, tv_scale, grad_dev, \
-                                                 b->acc, b->partials, err, fa)
-    gp_prof_pre(ctx);
-    if (tv_last) {
-      if (tv_on) GP_TV(true, true, true, true); else GP_TV(true, true, false, true);
-    } else if (grad_on) {
-      if (tv_on) GP_TV(false, true, true, false); else GP_TV(false, true, false, false);
-    } else {
-      if (tv_on) GP_TV(false, false, true, false); else GP_TV(false, false, false, false);
-    }
+                                                 b->acc, b->partials, fa)
+    // Traced as k_tv_inv (the sums alone), k_tv (with the gradient, or the
+    // gradient cleared without L_TV) and k_tv_grad (the fixed-point sums folded in).
+    if (!grad_on)
+      GP_KERNEL(ctx, "k_tv_inv", GP_TV(false, false, true, false));
+    else if (tv_last)
+      GP_KERNEL(ctx, "k_tv_grad", if (tv_on) GP_TV(true, true, true, true); else GP_TV(true, true, false, true));
+    else
+      GP_KERNEL(ctx, "k_tv", if (tv_on) GP_TV(false, true, true, false); else GP_TV(false, true, false, false));
 #undef GP_TV
-    gp_prof_post(ctx, "k_tv");
-    GP_LAUNCH_CHECK(ctx, "k_tv");
     return GP_OK;
   };
   auto launch_q = [&]() -> gp_status {
@@ -1056,7 +886,7 @@ extern "C" gp_status gp_step_update(gp_band* b, const float* rec_dev, int64_t B,
   gp_prof_pre(ctx);
 #define GP_TVA(D_, T_)                                                                                             \
   k_tv_adam<D_, T_><<<tb, TV_THREADS, 0, s>>>(G, b->brick_coord, b->brick_nbr, b->n_bricks, tv_scale, b->qgrad,  \
-                                              b->acc, b->D_alt, b->m, b->v, ad, b->partials, err, fa)
+                                              b->acc, b->D_alt, b->m, b->v, ad, b->partials, fa)
   if (det) {
     if (tv_on) GP_TVA(true, true); else GP_TVA(true, false);
   } else {

@@ -405,42 +405,33 @@ __device__ __forceinline__ bool query_record(const Grid& G, const float q[3], co
   return query_record_to<GRAD>(G, q, s, w, beta, gamma, sink, err, sp, sg, ss);
 }
 
-constexpr int HS = 12;            // staged edge: brick (8) + 2 on each side
-constexpr int HN = HS * HS * HS;  // 1728
-constexpr int IS = 10;            // TV edge: brick + 1 on each side
-constexpr int IN = IS * IS * IS;  // 1000
-
-__device__ __forceinline__ int hidx(int x, int y, int z) { return ((z + 2) * HS + (y + 2)) * HS + (x + 2); }
-// The inner region's 1/TV array: rows of IS values padded to TV_IROW floats,
-// so that the gather's warps (rows y, y + 2, y + 4, y + 6) meet no bank
-// conflict.
-constexpr int TV_IROW = 12;
-constexpr int TV_IPLANE = IS * TV_IROW;
-__device__ __forceinline__ int iidx(int x, int y, int z) { return ((z + 1) * IS + (y + 1)) * TV_IROW + (x + 1); }
-
-
-// The L_TV sweep, one brick at a time per block of TV_SWEEP_THREADS threads
-// (each owns two vertices of the brick).  For each brick: stage
-// the brick plus a two-vertex halo (12^3 values) and the T masks of its 27
-// neighbour bricks in shared memory, compute 1/TV_n on the brick plus a
-// one-vertex halo (10^3), then gather every vertex's
-//   dTV/dd_i = [i in T] sum_n (d_i - d_n) / TV_i + sum_{n in T} (d_i - d_n) / TV_n
-// over the in-grid axis neighbours n.  Each TV_i enters the sum once, from the
-// brick that stores i.
+// The L_TV sweep, one brick at a time per warp.  With 1/TV of T vertices (0
+// elsewhere) the gradient of a vertex is
+//   dTV/dd_i = sum over its in-grid axis neighbours n of
+//              (d_i - d_n) (1/TV_i + 1/TV_n),
+// so a brick needs 1/TV on its 8^3 vertices and on the six layers that touch
+// it, and these need the values two vertices out along an axis and one along
+// two.  The warp stages those values and the T masks of the brick and its six
+// face neighbours in shared memory (cp.async), computes 1/TV there, then the
+// gradient.  A lane works on four vertices along x at a time and keeps its
+// column of values along z in registers, so a stencil costs about 3.5 shared
+// words a vertex instead of 7 (a thread per vertex was bound by them).
+//
+// Every array moves once: values in, gradient out, 8 bytes a stored slot.
+// Warps share nothing, so a block has no barriers; 20 of them an SM hide each
+// other's copies.
 //
 // The band stores every in-grid axis neighbour of a T vertex, so a value the
-// sums use is always present: absent bricks are staged as zeros and only the
-// grid boundary needs checks (bricks within two vertices of it take a checked
-// path).  Staging copies rows: each halo row (fixed y, z) is four cp.async
-// pieces (x = -2..-1 from the brick below in x, 0..3 and 4..7 from the centre
-// column, 8..9 from the brick above), into rows padded to 16 floats.  The next
-// brick's halo is copied into the other of two buffers while the current one
-// is computed; the neighbour slots of the brick after that are fetched in two
-// steps spread over the current brick's phases.
-constexpr int TV_SWEEP_THREADS = 256;
-constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM at the register cap below (48 per thread)
-constexpr int TV_ROW = 20;        // floats per staged row: x = -2..9 at columns 2..13 (20: fewer bank conflicts)
-constexpr int TV_ROWS = HS * HS;  // 144 rows: y, z = -2..9
+// sums use is always present: absent bricks are staged as zeros.  In bricks at
+// the grid's boundary the vertices just outside take the values of their
+// in-grid neighbours (difference 0), and padding slots get gradient 0.
+constexpr int TV_SWEEP_THREADS = 128;
+constexpr int TV_SWEEP_WARPS = TV_SWEEP_THREADS / 32;
+constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM: 43 KB of shared memory, 102 registers a thread
+constexpr int TV_DENSE = 144 * 8;    // rows (y, z) in [-2, 9]^2, x in [0, 8)
+constexpr int TV_SIDE = 100 * 2;     // rows (y, z) in [-1, 8]^2: x = -2, -1 or x = 8, 9
+constexpr int TV_COPIES = 264 + 192; // 16-byte pieces of rows, 8-byte pieces of the sides
+constexpr int TV_PLAN = (TV_COPIES + 31) / 32;  // per lane
 
 // Brick b as the sweep sees it: values, masks, its row of the 27-neighbour
 // table (3x3x3, x fastest, -1 absent), grid size and origin vertex.
@@ -451,15 +442,16 @@ struct TvBrick {
   int R, ox, oy, oz;
 };
 
-struct TvShared {
-  __align__(16) float D[2][TV_ROWS * TV_ROW];   // staged values (0 in absent bricks)
-  __align__(16) uint32_t T[2][27 * 16];         // T-mask words of the 27 neighbour bricks (0 if absent)
-  float inv[IS * TV_IPLANE];                    // 1/TV of T vertices of the inner region, else 0
-  int slot[2][27];
-  TvBrick bk[2];
+struct TvWarp {
+  __align__(16) float d[TV_DENSE + 2 * TV_SIDE];  // values: rows, then the low and the high side
+  __align__(16) float inv[100 * 8];               // 1/TV: rows (y, z) in [-1, 8]^2
+  float side[2][64];                              // 1/TV at x = -1 and x = 8: index 8 z + y
+  __align__(16) uint32_t T[7 * 16];               // T masks: the brick, -x, +x, -y, +y, -z, +z
 };
-
-__device__ __forceinline__ int tv_hc(int x, int y, int z) { return ((z + 2) * HS + (y + 2)) * TV_ROW + (x + 4); }
+struct TvShared {
+  TvWarp w[TV_SWEEP_WARPS];
+  uint32_t plan[TV_PLAN * 32];  // region | local << 5 | destination << 14 | 16 bytes << 25 | valid << 26
+};
 
 __device__ __forceinline__ void cp_async_ca8(void* smem, const void* gmem, int src_bytes) {
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
@@ -469,228 +461,287 @@ __device__ __forceinline__ void cp_async_cg16(void* smem, const void* gmem, int 
   const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(sa), "l"(gmem), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait1() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// This thread's fixed share of every brick's work, decoded once: its row
-// pieces to copy and its inner-region entries.
-constexpr int TV_TASKS = (TV_ROWS * 4 + TV_SWEEP_THREADS - 1) / TV_SWEEP_THREADS;  // 3
-constexpr int TV_INNER = (IN + TV_SWEEP_THREADS - 1) / TV_SWEEP_THREADS;          // 4
-struct TvPlan {
-  uint32_t task[TV_TASKS];   // region | local << 5 | destination << 14 | 16-byte piece << 26 | valid << 27
-  uint32_t entry[TV_INNER];  // halo index | region << 12 | local << 17 | inner << 26 | valid << 27
-};
-
-__device__ __forceinline__ TvPlan tv_plan() {
-  TvPlan pl;
-#pragma unroll
-  for (int k = 0; k < TV_TASKS; ++k) {
-    const int r = threadIdx.x + k * TV_SWEEP_THREADS;
-    pl.task[k] = 0;
-    if (r >= TV_ROWS * 4) continue;
-    const int row = r >> 2, seg = r & 3;
-    const int hy = row % HS - 2, hz = row / HS - 2;
-    const int dx = seg == 0 ? 0 : (seg == 3 ? 2 : 1);  // brick column: below / centre / above
-    const int lx0 = seg == 0 ? 6 : (seg == 2 ? 4 : 0);
-    const int col = seg == 0 ? 2 : (seg == 1 ? 4 : (seg == 2 ? 8 : 12));
-    const uint32_t reg = ((hz >> 3) + 1) * 9 + ((hy >> 3) + 1) * 3 + dx;
-    const uint32_t loc = ((hz & 7) << 6) | ((hy & 7) << 3) | lx0;
-    const uint32_t dst = row * TV_ROW + col;
-    const uint32_t big = (seg == 1 || seg == 2) ? 1u : 0u;
-    pl.task[k] = reg | (loc << 5) | (dst << 14) | (big << 26) | (1u << 27);
-  }
-#pragma unroll
-  for (int k = 0; k < TV_INNER; ++k) {
-    const int h = threadIdx.x + k * TV_SWEEP_THREADS;
-    pl.entry[k] = 0;
-    if (h >= IN) continue;
-    const int x = h % IS - 1, y = (h / IS) % IS - 1, z = h / (IS * IS) - 1;
-    const uint32_t reg = ((z >> 3) + 1) * 9 + ((y >> 3) + 1) * 3 + ((x >> 3) + 1);
-    const uint32_t loc = ((z & 7) << 6) | ((y & 7) << 3) | (x & 7);
-    const uint32_t inner = (x >= 0 && y >= 0 && z >= 0 && x < 8 && y < 8 && z < 8) ? 1u : 0u;
-    pl.entry[k] = (uint32_t)tv_hc(x, y, z) | (reg << 12) | (loc << 17) | (inner << 26) | (1u << 27);
-  }
-  return pl;
+__device__ __forceinline__ int tv_row(int y, int z) { return ((z + 2) * 12 + (y + 2)) * 8; }   // in TvWarp::d
+__device__ __forceinline__ int tv_side(int s, int y, int z) {                                  // the side's pair
+  return TV_DENSE + s * TV_SIDE + ((z + 1) * 10 + (y + 1)) * 2;
 }
+__device__ __forceinline__ int tv_irow(int y, int z) { return ((z + 1) * 10 + (y + 1)) * 8; }  // in TvWarp::inv
 
-// Issue the copies of brick bk[q]'s halo rows and neighbour T masks into
-// buffer q (zero-filled where the brick is absent).
-__device__ __forceinline__ void tv_issue(TvShared& sh, int q, const TvPlan& pl) {
-  const float* D = sh.bk[q].D;
-#pragma unroll
-  for (int k = 0; k < TV_TASKS; ++k) {
-    const uint32_t t = pl.task[k];
-    if (!(t >> 27)) continue;
-    const int sl = sh.slot[q][t & 31];
-    const float* src = sl >= 0 ? D + (size_t)sl * 512u + ((t >> 5) & 511) : D;
-    float* dst = &sh.D[q][(t >> 14) & 4095];
-    if ((t >> 26) & 1)
-      cp_async_cg16(dst, src, sl >= 0 ? 16 : 0);
-    else
-      cp_async_ca8(dst, src, sl >= 0 ? 8 : 0);
-  }
-  if (threadIdx.x < 27 * 4) {
-    const int w = threadIdx.x;
-    const int sl = sh.slot[q][w >> 2];
-    const uint32_t* masks = sh.bk[q].masks;
-    const uint32_t* src = sl >= 0 ? masks + (size_t)sl * 48u + 4u * (w & 3) : masks;
-    cp_async_cg16(&sh.T[q][4 * w], src, sl >= 0 ? 16 : 0);
-  }
-}
-
-// Is every vertex of the halo inside [0, R]^3?
-__device__ __forceinline__ bool tv_interior(const TvBrick& bk) {
-  return bk.ox >= 2 && bk.oy >= 2 && bk.oz >= 2 && bk.ox + 9 <= bk.R && bk.oy + 9 <= bk.R && bk.oz + 9 <= bk.R;
-}
-
-// 1/TV over the inner region of buffer p; adds this thread's share of the
-// brick's own TV_i to tsum.  CHECK: skip out-of-grid neighbours.
-template <bool CHECK>
-__device__ __forceinline__ void tv_inverse(TvShared& sh, int p, const TvBrick& bk, const TvPlan& pl, float& tsum) {
-  const float* D = sh.D[p];
-  const uint32_t* T = sh.T[p];
-#pragma unroll
-  for (int k = 0; k < TV_INNER; ++k) {
-    const uint32_t e = pl.entry[k];
-    if (!(e >> 27)) continue;
-    const int h = threadIdx.x + k * TV_SWEEP_THREADS;
-    const int c = e & 4095, reg = (e >> 12) & 31, loc = (e >> 17) & 511;
-    float inv = 0.f;
-    if ((T[reg * 16 + (loc >> 5)] >> (loc & 31)) & 1u) {
-      const float dc = D[c];
-      const int nb6[6] = {c - 1, c + 1, c - TV_ROW, c + TV_ROW, c - TV_ROW * HS, c + TV_ROW * HS};
-      bool ok[6] = {true, true, true, true, true, true};
-      if (CHECK) {
-        const int x = h % IS - 1 + bk.ox, y = (h / IS) % IS - 1 + bk.oy, z = h / (IS * IS) - 1 + bk.oz;
-        ok[0] = x > 0;
-        ok[1] = x < bk.R;
-        ok[2] = y > 0;
-        ok[3] = y < bk.R;
-        ok[4] = z > 0;
-        ok[5] = z < bk.R;
-      }
-      float acc2 = 0.f;
-#pragma unroll
-      for (int t = 0; t < 6; ++t) {
-        const float d = dc - D[nb6[t]];
-        if (ok[t]) acc2 = fmaf(d, d, acc2);
-      }
-      inv = acc2 > 0.f ? rsqrtf(acc2) : 0.f;  // 1/TV_n
-      if ((e >> 26) & 1) tsum += acc2 * inv;  // TV_n
+// The copies of a brick, the same for each: entry e of the plan.
+__device__ __forceinline__ uint32_t tv_plan_entry(int e) {
+  if (e >= TV_COPIES) return 0u;
+  int y, z, dx, x, dst;
+  const bool big = e < 264;
+  if (big) {
+    // Rows: 96 with z in [0, 8), y in [-2, 9]; 20 with z = -1, 8, y in
+    // [-1, 8]; 16 with z = -2, 9, y in [0, 8).  Two pieces each.
+    const int r = e >> 1;
+    if (r < 96) {
+      z = r / 12;
+      y = r % 12 - 2;
+    } else if (r < 116) {
+      z = r < 106 ? -1 : 8;
+      y = (r - 96) % 10 - 1;
+    } else {
+      z = r < 124 ? -2 : 9;
+      y = (r - 116) % 8;
     }
-    sh.inv[(h / IS) * TV_IROW + h % IS] = inv;  // iidx of the entry
+    dx = 1;
+    x = 4 * (e & 1);
+    dst = ((z + 2) * 12 + (y + 2)) * 8 + x;
+  } else {
+    // Sides: 80 rows with z in [0, 8), y in [-1, 8]; 16 with z = -1, 8, y in [0, 8).
+    const int k = e - 264, s = k / 96, r = k % 96;
+    if (r < 80) {
+      z = r / 10;
+      y = r % 10 - 1;
+    } else {
+      z = r < 88 ? -1 : 8;
+      y = (r - 80) % 8;
+    }
+    dx = 2 * s;
+    x = s ? 0 : 6;
+    dst = TV_DENSE + s * TV_SIDE + ((z + 1) * 10 + (y + 1)) * 2;
   }
+  const uint32_t reg = ((z >> 3) + 1) * 9 + ((y >> 3) + 1) * 3 + dx;
+  const uint32_t loc = ((z & 7) << 6) | ((y & 7) << 3) | x;
+  return reg | (loc << 5) | ((uint32_t)dst << 14) | ((big ? 1u : 0u) << 25) | (1u << 26);
 }
 
-// dTV/dd of this thread's two vertices of the brick in buffer p: (lx, ly, lz)
-// and (lx, ly + 1, lz) with lx = t & 7, ly = 2 ((t >> 3) & 3), lz = t >> 5,
-// vertex indices l0 = lx + 8 ly + 64 lz and l0 + 8.  A warp's four rows y are
-// two apart, which keeps both the staged values (rows 40 floats apart) and
-// the inverses (24 apart) free of bank conflicts.  0 outside the grid.
-template <bool CHECK>
-__device__ __forceinline__ void tv_gather(const TvShared& sh, int p, const TvBrick& bk, float& g0, float& g1,
-                                          int& l0) {
-  const int t = threadIdx.x;
-  const int lx = t & 7, ly0 = 2 * ((t >> 3) & 3), lz = t >> 5;
-  const float* D = sh.D[p];
-  const float* I = sh.inv;
-  l0 = lx + 8 * ly0 + 64 * lz;
-  float out[2];
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const int ly = ly0 + k;
-    bool ok[6] = {true, true, true, true, true, true};
-    bool inside = true;
-    if (CHECK) {
-      const int x = bk.ox + lx, y = bk.oy + ly, z = bk.oz + lz;
-      inside = x <= bk.R && y <= bk.R && z <= bk.R;
-      ok[0] = x > 0;
-      ok[1] = x < bk.R;
-      ok[2] = y > 0;
-      ok[3] = y < bk.R;
-      ok[4] = z > 0;
-      ok[5] = z < bk.R;
+// Boundary bricks: the vertices one step outside the grid take the value of
+// the in-grid vertex next to them.
+__device__ __forceinline__ void tv_close_grid(float* d, const TvBrick& bk, int lane) {
+  auto copy_y = [&](int to, int from) {  // rows y = from to y = to, all z
+    for (int k = lane; k < 96; k += 32) {
+      const int z = (k >> 3) - 2, x = k & 7;
+      d[tv_row(to, z) + x] = d[tv_row(from, z) + x];
     }
-    const int c = tv_hc(lx, ly, lz), ci = iidx(lx, ly, lz);
-    const float di = D[c], own = I[ci];
-    const int hn[6] = {c - 1, c + 1, c - TV_ROW, c + TV_ROW, c - TV_ROW * HS, c + TV_ROW * HS};
-    const int in6[6] = {ci - 1, ci + 1, ci - TV_IROW, ci + TV_IROW, ci - TV_IPLANE, ci + TV_IPLANE};
-    float gsum = 0.f;
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      // own != 0 only for i in T, whose in-grid neighbours are all stored;
-      // inv[n] != 0 only for n in T (inside the grid and stored).
-      if (ok[j]) gsum = fmaf(di - D[hn[j]], own + I[in6[j]], gsum);
+    if (to >= -1 && to <= 8)
+      for (int k = lane; k < 40; k += 32)
+        d[tv_side(k / 20, to, (k % 20) / 2 - 1) + (k & 1)] = d[tv_side(k / 20, from, (k % 20) / 2 - 1) + (k & 1)];
+    __syncwarp();
+  };
+  auto copy_z = [&](int to, int from) {
+    for (int k = lane; k < 96; k += 32) {
+      const int y = (k >> 3) - 2, x = k & 7;
+      d[tv_row(y, to) + x] = d[tv_row(y, from) + x];
     }
-    out[k] = inside ? gsum : 0.f;
+    if (to >= -1 && to <= 8)
+      for (int k = lane; k < 40; k += 32)
+        d[tv_side(k / 20, (k % 20) / 2 - 1, to) + (k & 1)] = d[tv_side(k / 20, (k % 20) / 2 - 1, from) + (k & 1)];
+    __syncwarp();
+  };
+  const int lx = bk.R - bk.ox, ly = bk.R - bk.oy, lz = bk.R - bk.oz;  // the last in-grid vertex
+  if (bk.ox == 0 || lx <= 8) {
+    for (int k = lane; k < 100; k += 32) {
+      const int y = k % 10 - 1, z = k / 10 - 1;
+      if (bk.ox == 0) d[tv_side(0, y, z) + 1] = d[tv_row(y, z)];
+      if (lx == 0) d[tv_row(y, z) + 1] = d[tv_row(y, z)];
+      if (lx == 8) d[tv_side(1, y, z) + 1] = d[tv_side(1, y, z)];
+    }
+    __syncwarp();
   }
-  g0 = out[0];
-  g1 = out[1];
+  if (bk.oy == 0) copy_y(-1, 0);
+  if (ly <= 8) copy_y(ly + 1, ly);
+  if (bk.oz == 0) copy_z(-1, 0);
+  if (lz <= 8) copy_z(lz + 1, lz);
 }
 
-// The sweep over work items first, first + stride, ... < n of this block.
-// src.brick(i) gives item i's TvBrick.  out(i, l0, g0, l1, g1, tsum) is called
-// by every thread once per item, in order, with the unscaled dTV/dd of the
-// thread's two vertices l0, l1 (tv_gather) and its share of the item's sum of
-// TV_i; it may synchronise the block.
-struct TvNoPre {
-  __device__ __forceinline__ void operator()(int64_t) const {}
-};
+__device__ __forceinline__ float4 tv_ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
 
-// pre(i) (optional) is called by every thread at the top of item i's
-// iteration, while the item's halo copies are still in flight: a place to
-// issue loads whose latency the stencil work then hides.
-template <class Src, class Out, class Pre = TvNoPre>
-__device__ __forceinline__ void tv_sweep(const Src& src, int64_t first, int64_t stride, int64_t n, TvShared& sh,
-                                         Out&& out, Pre&& pre = Pre()) {
-  const int l = threadIdx.x;
-  if (first >= n) return;
-  const TvPlan pl = tv_plan();
-  if (l == 0) sh.bk[0] = src.brick(first);
+// 1/TV of a quad from its values and those of its 6 axis neighbours (the
+// squared differences added in the order -x, +x, -y, +y, -z, +z), 0 where the
+// bit of T is clear; tsum: the sum of TV.
+__device__ __forceinline__ float4 tv_inv4(float4 c, float left, float right, float4 ym, float4 yp, float4 zm,
+                                          float4 zp, uint32_t bits, float& tsum) {
+  const float v[6] = {left, c.x, c.y, c.z, c.w, right};
+  const float a[4][4] = {{ym.x, yp.x, zm.x, zp.x}, {ym.y, yp.y, zm.y, zp.y},
+                         {ym.z, yp.z, zm.z, zp.z}, {ym.w, yp.w, zm.w, zp.w}};
+  float out[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float d = v[k + 1];
+    float e = d - v[k];
+    float s = e * e;
+    e = d - v[k + 2];
+    s = fmaf(e, e, s);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      e = d - a[k][j];
+      s = fmaf(e, e, s);
+    }
+    const bool in = (bits >> k) & 1u;
+    out[k] = in && s > 0.f ? rsqrtf(s) : 0.f;
+    tsum += in ? s * out[k] : 0.f;
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
+}
+
+// The gradient of a quad, unscaled, in the same order of neighbours.
+__device__ __forceinline__ float4 tv_grad4(float4 c, float left, float right, float4 ym, float4 yp, float4 zm,
+                                           float4 zp, float4 ic, float ileft, float iright, float4 iym, float4 iyp,
+                                           float4 izm, float4 izp) {
+  const float v[6] = {left, c.x, c.y, c.z, c.w, right}, w[6] = {ileft, ic.x, ic.y, ic.z, ic.w, iright};
+  const float a[4][4] = {{ym.x, yp.x, zm.x, zp.x}, {ym.y, yp.y, zm.y, zp.y},
+                         {ym.z, yp.z, zm.z, zp.z}, {ym.w, yp.w, zm.w, zp.w}};
+  const float b[4][4] = {{iym.x, iyp.x, izm.x, izp.x}, {iym.y, iyp.y, izm.y, izp.y},
+                         {iym.z, iyp.z, izm.z, izp.z}, {iym.w, iyp.w, izm.w, izp.w}};
+  float out[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float d = v[k + 1], own = w[k + 1];
+    float g = (d - v[k]) * (own + w[k]);
+    g = fmaf(d - v[k + 2], own + w[k + 2], g);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) g = fmaf(d - a[k][j], own + b[k][j], g);
+    out[k] = g;
+  }
+  return make_float4(out[0], out[1], out[2], out[3]);
+}
+
+// The sweep over work items 0 .. n - 1, dealt to the warps of the grid in
+// turn.  src.brick(i) gives item i's TvBrick.  For each of the brick's 128
+// quads q (vertices 4 q .. 4 q + 3) one lane calls fetch(i, q), whose loads the
+// stencil work then hides, and out(i, q, d, g, fetched) with the quad's values
+// and unscaled gradient; done(i, tsum) is called by every lane after each item
+// with its share of the sum of TV_i.  All lanes of the warp call these together.
+// GRAD = false: the sums only (no layers, no fetch, no out).
+template <bool GRAD, class Src, class Fetch, class Out, class Done>
+__device__ __forceinline__ void tv_sweep(const Src& src, int64_t n, TvShared& sh, Fetch&& fetch, Out&& out,
+                                         Done&& done) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  for (int e = threadIdx.x; e < TV_PLAN * 32; e += TV_SWEEP_THREADS) sh.plan[e] = tv_plan_entry(e);
   __syncthreads();
-  if (l < 27) sh.slot[0][l] = __ldg(sh.bk[0].nbr + l);
-  __syncthreads();
-  tv_issue(sh, 0, pl);
-  cp_async_commit();
-  if (first + stride < n) {
-    if (l == 0) sh.bk[1] = src.brick(first + stride);
-    __syncthreads();
-    if (l < 27) sh.slot[1][l] = __ldg(sh.bk[1].nbr + l);
+  TvWarp& s = sh.w[wid];
+  const int xq = lane & 1, y = (lane >> 1) & 7, z0 = 4 * (lane >> 4);
+  const int64_t stride = (int64_t)gridDim.x * TV_SWEEP_WARPS;
+  int64_t i = (int64_t)blockIdx.x * TV_SWEEP_WARPS + wid;
+  if (i >= n) return;
+  TvBrick bk = src.brick(i);
+  int nbr = lane < 27 ? __ldg(bk.nbr + lane) : -1;
+  while (true) {
+    // Copies of item i.
+#pragma unroll 5
+    for (int k = 0; k < TV_PLAN; ++k) {
+      const uint32_t t = sh.plan[lane + 32 * k];
+      const int sl = __shfl_sync(0xffffffffu, nbr, t & 31);
+      if (!(t >> 26)) continue;
+      const float* from = sl >= 0 ? bk.D + (int64_t)sl * 512 + ((t >> 5) & 511) : bk.D;
+      float* to = &s.d[(t >> 14) & 2047];
+      if ((t >> 25) & 1)
+        cp_async_cg16(to, from, sl >= 0 ? 16 : 0);
+      else
+        cp_async_ca8(to, from, sl >= 0 ? 8 : 0);
+    }
+    {
+      const int f = lane >> 2;  // the brick, -x, +x, -y, +y, -z, +z
+      const int reg = f == 0 ? 13 : f == 1 ? 12 : f == 2 ? 14 : f == 3 ? 10 : f == 4 ? 16 : f == 5 ? 4 : 22;
+      const int sl = __shfl_sync(0xffffffffu, nbr, reg);
+      if (lane < 28)
+        cp_async_cg16(&s.T[4 * lane], sl >= 0 ? bk.masks + (int64_t)sl * 48 + 4 * (lane & 3) : bk.masks,
+                      sl >= 0 ? 16 : 0);
+    }
+    // The next item's neighbours are fetched meanwhile.
+    const int64_t next = i + stride;
+    TvBrick nk = bk;
+    int nnbr = -1;
+    if (next < n) {
+      nk = src.brick(next);
+      if (lane < 27) nnbr = __ldg(nk.nbr + lane);
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    const bool edge = bk.ox == 0 || bk.oy == 0 || bk.oz == 0 || bk.ox + 8 >= bk.R || bk.oy + 8 >= bk.R ||
+                      bk.oz + 8 >= bk.R;
+    if (edge) tv_close_grid(s.d, bk, lane);
+
+    // 1/TV of the brick's own quads, up a lane's column z0 .. z0 + 3.
+    float tsum = 0.f, none = 0.f;
+    {
+      float4 zm = tv_ld4(s.d + tv_row(y, z0 - 1) + 4 * xq), c = tv_ld4(s.d + tv_row(y, z0) + 4 * xq);
+#pragma unroll 2
+      for (int z = z0; z < z0 + 4; ++z) {
+        const int r = tv_row(y, z);
+        const float4 zp = tv_ld4(s.d + r + 96 + 4 * xq);
+        const float left = s.d[xq ? r + 3 : tv_side(0, y, z) + 1], right = s.d[xq ? tv_side(1, y, z) : r + 4];
+        const float4 iv = tv_inv4(c, left, right, tv_ld4(s.d + r - 8 + 4 * xq), tv_ld4(s.d + r + 8 + 4 * xq), zm, zp,
+                                  s.T[2 * z + (y >> 2)] >> (8 * (y & 3) + 4 * xq), tsum);
+        if (GRAD) *reinterpret_cast<float4*>(s.inv + tv_irow(y, z) + 4 * xq) = iv;
+        zm = c;
+        c = zp;
+      }
+    }
+    if (GRAD) {
+    // The layers y = -1, 8 and z = -1, 8: 16 quads each.
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int f = (lane >> 4) + 2 * k, t = (lane >> 1) & 7;
+      const int fy = f == 0 ? -1 : f == 1 ? 8 : t, fz = f == 2 ? -1 : f == 3 ? 8 : t;
+      const int r = tv_row(fy, fz);
+      const float left = s.d[xq ? r + 3 : tv_side(0, fy, fz) + 1], right = s.d[xq ? tv_side(1, fy, fz) : r + 4];
+      const uint32_t bits = s.T[16 * (f + 3) + 2 * (fz & 7) + ((fy & 7) >> 2)] >> (8 * (fy & 3) + 4 * xq);
+      *reinterpret_cast<float4*>(s.inv + tv_irow(fy, fz) + 4 * xq) =
+          tv_inv4(tv_ld4(s.d + r + 4 * xq), left, right, tv_ld4(s.d + r - 8 + 4 * xq), tv_ld4(s.d + r + 8 + 4 * xq),
+                  tv_ld4(s.d + r - 96 + 4 * xq), tv_ld4(s.d + r + 96 + 4 * xq), bits, none);
+    }
+    // The layers x = -1 and x = 8: 64 vertices each.
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int sd = k >> 1, v = lane + 32 * (k & 1), fy = v & 7, fz = v >> 3;
+      const int at = tv_side(sd, fy, fz) + (sd ? 0 : 1);  // the layer's value; its outer neighbour beside it
+      const float d = s.d[at];
+      const float xm = sd ? s.d[tv_row(fy, fz) + 7] : s.d[at - 1], xp = sd ? s.d[at + 1] : s.d[tv_row(fy, fz)];
+      float e = d - xm, q = e * e;
+      e = d - xp;
+      q = fmaf(e, e, q);
+      e = d - s.d[at - 2];
+      q = fmaf(e, e, q);
+      e = d - s.d[at + 2];
+      q = fmaf(e, e, q);
+      e = d - s.d[at - 20];
+      q = fmaf(e, e, q);
+      e = d - s.d[at + 20];
+      q = fmaf(e, e, q);
+      const bool in = (s.T[16 * (1 + sd) + 2 * fz + (fy >> 2)] >> (8 * (fy & 3) + (sd ? 0 : 7))) & 1u;
+      s.side[sd][v] = in && q > 0.f ? rsqrtf(q) : 0.f;
+    }
+    __syncwarp();
+    // The gradient.
+    float4 zm = tv_ld4(s.d + tv_row(y, z0 - 1) + 4 * xq), c = tv_ld4(s.d + tv_row(y, z0) + 4 * xq);
+    float4 izm = tv_ld4(s.inv + tv_irow(y, z0 - 1) + 4 * xq), ic = tv_ld4(s.inv + tv_irow(y, z0) + 4 * xq);
+#pragma unroll 2
+    for (int z = z0; z < z0 + 4; ++z) {
+      const int r = tv_row(y, z), ir = tv_irow(y, z), q = (z * 8 + y) * 2 + xq;
+      auto got = fetch(i, q);
+      const float4 zp = tv_ld4(s.d + r + 96 + 4 * xq), izp = tv_ld4(s.inv + ir + 80 + 4 * xq);
+      const float left = s.d[xq ? r + 3 : tv_side(0, y, z) + 1], right = s.d[xq ? tv_side(1, y, z) : r + 4];
+      const float ileft = xq ? s.inv[ir + 3] : s.side[0][8 * z + y], iright = xq ? s.side[1][8 * z + y] : s.inv[ir + 4];
+      float4 g = tv_grad4(c, left, right, tv_ld4(s.d + r - 8 + 4 * xq), tv_ld4(s.d + r + 8 + 4 * xq), zm, zp, ic, ileft,
+                          iright, tv_ld4(s.inv + ir - 8 + 4 * xq), tv_ld4(s.inv + ir + 8 + 4 * xq), izm, izp);
+      if (edge) {
+        const bool row = bk.oy + y <= bk.R && bk.oz + z <= bk.R;
+        const int x = bk.ox + 4 * xq;
+        g.x = row && x <= bk.R ? g.x : 0.f;
+        g.y = row && x + 1 <= bk.R ? g.y : 0.f;
+        g.z = row && x + 2 <= bk.R ? g.z : 0.f;
+        g.w = row && x + 3 <= bk.R ? g.w : 0.f;
+      }
+      out(i, q, c, g, got);
+      zm = c;
+      c = zp;
+      izm = ic;
+      ic = izp;
+    }
+    }
+    done(i, tsum);
+    if (next >= n) break;
+    __syncwarp();  // every lane is done with the staged brick
+    i = next;
+    bk = nk;
+    nbr = nnbr;
   }
-  int p = 0;
-  for (int64_t i = first; i < n; i += stride) {
-    pre(i);
-    __syncthreads();  // the previous item is done with buffer p ^ 1 and inv; bk / slot[p ^ 1] written
-    const int64_t next = i + stride, after = next + stride;
-    if (next < n) tv_issue(sh, p ^ 1, pl);
-    cp_async_commit();
-    TvBrick ab;
-    if (l < 27 && after < n) ab = src.brick(after);  // warp 0: one broadcast load per field
-    const TvBrick bk = sh.bk[p];
-    const bool check = !tv_interior(bk);
-    cp_async_wait1();  // this thread's copies of item i have landed
-    __syncthreads();   // ... and everyone's
-    float tsum = 0.f;
-    if (check)
-      tv_inverse<true>(sh, p, bk, pl, tsum);
-    else
-      tv_inverse<false>(sh, p, bk, pl, tsum);
-    __syncthreads();  // inv ready; bk[p] and slot[p] are free
-    if (l == 0 && after < n) sh.bk[p] = ab;
-    int rs = -1;
-    if (l < 27 && after < n) rs = __ldg(ab.nbr + l);
-    float g0, g1;
-    int l0;
-    if (check)
-      tv_gather<true>(sh, p, bk, g0, g1, l0);
-    else
-      tv_gather<false>(sh, p, bk, g0, g1, l0);
-    if (l < 27 && after < n) sh.slot[p][l] = rs;
-    out(i, l0, g0, l0 + 8, g1, tsum);
-    p ^= 1;
-  }
-  cp_async_wait0();
 }
 
 // One Adam step (Kingma and Ba; Sec. 4 "Details") of one vertex, the bias
