@@ -307,21 +307,55 @@ __device__ __forceinline__ void nn_scan(NNTop& t, const NNQuery& q, const NNGrid
   }
 }
 
+// A block with points near q, where the block q lies in has none: of the first
+// ring of super-blocks around q with any, the one whose centre is nearest.
+static __device__ __noinline__ int nn_near_block(float q0, float q1, float q2, const NNGrid& g) {
+  const int c[3] = {nn_cell(q0, g) >> 4, nn_cell(q1, g) >> 4, nn_cell(q2, g) >> 4};
+  float best = INFINITY;
+  int at = -1;
+  for (int r = 0; r < g.nsup && at < 0; ++r)
+    for (int sz = max(c[2] - r, 0); sz <= min(c[2] + r, g.nsup - 1); ++sz)
+      for (int sy = max(c[1] - r, 0); sy <= min(c[1] + r, g.nsup - 1); ++sy) {
+        const bool face = sz == c[2] - r || sz == c[2] + r || sy == c[1] - r || sy == c[1] + r;
+        for (int sx = c[0] - r; sx <= c[0] + r; sx += (face || r == 0) ? 1 : 2 * r) {
+          if (sx < 0 || sx >= g.nsup) continue;
+          unsigned long long sm = __ldg(g.sup + ((int64_t)sz * g.nsup + sy) * g.nsup + sx);
+          while (sm) {
+            const int bit = __ffsll((long long)sm) - 1;
+            sm &= sm - 1ull;
+            const int bx = 4 * sx + (bit & 3), by = 4 * sy + ((bit >> 2) & 3), bz = 4 * sz + (bit >> 4);
+            const float dx = q0 - (-1.0f + (float)(4 * bx + 2) * g.cs), dy = q1 - (-1.0f + (float)(4 * by + 2) * g.cs),
+                        dz = q2 - (-1.0f + (float)(4 * bz + 2) * g.cs);
+            const float d = dx * dx + dy * dy + dz * dz;
+            if (at < 0 || d < best) {
+              best = d;
+              at = bx | by << 8 | bz << 16;
+            }
+          }
+        }
+      }
+  return at;
+}
+
 // Step 1 of a search: a first point.  hint: index of a cloud point
 // to start from (-1: none); a record of `seeds` is a point s and its normal n
 // as three 10-bit signed fractions of 511 (0: unknown).  The nearest point is
 // expected around the foot of q on the tangent plane of s, then on the plane
 // of the block there (of the block of s, where that one holds no point); the
 // points of the 2^3 cells nearest to that place are scanned, or those of the
-// whole block where these are empty.  Returns the block scanned and where:
-// record << 7 | all << 6 | lowest scanned cell in the block, -1 if none.
+// whole block where these are empty.  A query without a hint tends to lie on
+// the surface (a mesh scored against a cloud); within half a cell of the plane
+// its ball is small and the one cell it is in is scanned.  Returns the block scanned
+// and where: record << 8 | (0: 2^3 cells, 1: all, 2: one cell) << 6 | lowest
+// scanned cell in the block, all bits set if there is no block.
 template <bool COUNT>
 __device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, const float4* __restrict__ seeds,
                                         const NNGrid& g, NNTop& t, int& work) {
   t = NNTop{INFINITY, INFINITY, -1};
   float f[3] = {q[0], q[1], q[2]};
   float4 s = make_float4(q[0], q[1], q[2], 0.f);
-  if (hint >= 0 && hint < J) {
+  const bool hinted = hint >= 0 && hint < J;
+  if (hinted) {
     s = __ldg(seeds + hint);
     const float d = nn_d32(q, s.x, s.y, s.z);
     if (COUNT) ++work;
@@ -342,24 +376,35 @@ __device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, c
     by = nn_cell(s.y, g) >> 2;
     bz = nn_cell(s.z, g) >> 2;
     bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
-    if (bi < 0) return -1;
+    if (bi < 0) {
+      const int at = nn_near_block(q[0], q[1], q[2], g);
+      if (at < 0) return -1;
+      bx = at & 255;
+      by = (at >> 8) & 255;
+      bz = at >> 16;
+      bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
+    }
   }
   const float4 A = __ldg(g.blk + 2 * (int64_t)bi), B = __ldg(g.blk + 2 * (int64_t)bi + 1);
   const NNBlock k = nn_block(B);
   const float n[3] = {A.x, A.y, A.z};
   const float off = 0.5f * (A.w + B.x) - (A.x * f[0] + A.y * f[1] + A.z * f[2]);
   const int corner[3] = {4 * bx, 4 * by, 4 * bz};
+  const float h = n[0] * q[0] + n[1] * q[1] + n[2] * q[2] - 0.5f * (A.w + B.x);
+  int how = !hinted && fabsf(h) < 0.5f * g.cs ? 2 : 0;
   int lo[3], hi[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
-    // the 2 cells nearest to the place along this axis, inside the block
-    const int c = nn_cell(f[a] + off * n[a] - 0.5f * g.cs, g);
-    lo[a] = min(max(c, corner[a]), corner[a] + 2);
-    hi[a] = lo[a] + 1;
+    // the 2 cells nearest to the place along this axis (or its cell), inside the block
+    const int c = nn_cell(f[a] + off * n[a] - (how ? 0.f : 0.5f * g.cs), g);
+    lo[a] = min(max(c, corner[a]), corner[a] + (how ? 3 : 2));
+    hi[a] = lo[a] + (how ? 0 : 1);
   }
   unsigned long long m = k.mask & nn_box_mask(lo, hi, bx, by, bz);
-  const bool all = m == 0ull;
-  if (all) m = k.mask;
+  if (!m) {
+    m = k.mask;
+    how = 1;
+  }
   const NNQuery q2 = nn_query(q);
   int cur = 0, end = 0;
   while (true) {
@@ -370,7 +415,7 @@ __device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, c
     }
     nn_scan(t, q2, g, cur++);
   }
-  return (bi << 7) | ((int)all << 6) | ((lo[0] & 3) | ((lo[1] & 3) << 2) | ((lo[2] & 3) << 4));
+  return (bi << 8) | (how << 6) | ((lo[0] & 3) | ((lo[1] & 3) << 2) | ((lo[2] & 3) << 4));
 }
 
 // A warp's shared state in step 2: its 32 queries with their bounds, and the
@@ -475,6 +520,7 @@ __device__ __forceinline__ void nn_rest(const float q[3], const NNGrid& g, bool 
     const bool last = nb <= 32 && base >= total && !__any_sync(FULL, sm != 0ull);
     const int take = min(nb, 32);
     nb -= take;
+    if (go) sh.q[lane].w = nn_thr(__uint_as_float((unsigned)(sh.key1[lane] >> 32)));  // the bounds reached so far
     __syncwarp();
     unsigned long long m = 0ull;
     NNBlock k{0ull, 0};
@@ -488,9 +534,10 @@ __device__ __forceinline__ void nn_rest(const float q[3], const NNGrid& g, bool 
       const int bi = __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx);
       m = nn_block_cells(qo, Q.w, nn_margin(qo), g, bi, bx, by, bz, k);
       const int f = sh.first[o];
-      if (bi == f >> 7) {
+      if (bi == (int)((unsigned)f >> 8)) {
         const int l0[3] = {f & 3, (f >> 2) & 3, (f >> 4) & 3};
-        const int h0[3] = {l0[0] + 1, l0[1] + 1, l0[2] + 1};
+        const int e = (f & 128) ? 0 : 1;
+        const int h0[3] = {l0[0] + e, l0[1] + e, l0[2] + e};
         m &= (f & 64) ? 0ull : ~nn_box_mask(l0, h0, 0, 0, 0);
       }
     }
@@ -602,7 +649,8 @@ __device__ __forceinline__ bool nn_query_ok(const float q[3]) {
 
 // The search of a warp's 32 queries, one a lane, all lanes together (ok: this
 // lane has one).  Step 1 lane by lane, step 2 shared; a query that step 1
-// leaves without a bound walks the rings instead.
+// leaves without a bound (a block of points no distance to which compares
+// below +inf) walks the rings instead.
 template <bool COUNT>
 __device__ __forceinline__ int nn_search(const float q[3], bool ok, int hint, int64_t J,
                                          const float4* __restrict__ seeds, const NNGrid& g, NNWarp& sh, float s[3],
