@@ -302,44 +302,47 @@ __global__ void k_export(const int32_t* __restrict__ coord, const uint32_t* __re
 
 void band_free(gp_band* b) {
   if (!b) return;
-  gp_free(b->brick_table);
-  gp_free(b->brick_coord);
-  gp_free(b->brick_nbr);
-  gp_free(b->masks);
-  gp_free(b->active);
-  gp_free(b->D);
-  gp_free(b->m);
-  gp_free(b->v);
-  gp_free(b->acc);
-  gp_free(b->D_alt);
-  gp_free(b->qgrad);
-  gp_free(b->pts);
-  gp_free(b->pts_sorted);
-  gp_free(b->cell_table);
-  gp_free(b->cell_sup);
-  gp_free(b->cell_blk);
-  gp_free(b->cell_occ);
-  gp_free(b->sigma);
-  gp_free(b->seeds);
-  gp_free(b->perm);
-  gp_free(b->inv_perm);
-  gp_free(b->order_tiles);
-  gp_free(b->emit_order);
-  gp_free(b->emit_slot);
-  gp_free(b->emit_pts);
-  gp_free(b->partials);
-  gp_free(b->dev_ints);
+  cudaDeviceSynchronize();  // any stream may have worked on the band
+  gp_free_idle(b->brick_table);
+  gp_free_idle(b->brick_coord);
+  gp_free_idle(b->brick_nbr);
+  gp_free_idle(b->masks);
+  gp_free_idle(b->active);
+  gp_free_idle(b->D);
+  gp_free_idle(b->m);
+  gp_free_idle(b->v);
+  gp_free_idle(b->acc);
+  gp_free_idle(b->D_alt);
+  gp_free_idle(b->qgrad);
+  gp_free_idle(b->pts);
+  gp_free_idle(b->pts_sorted);
+  gp_free_idle(b->cell_table);
+  gp_free_idle(b->cell_sup);
+  gp_free_idle(b->cell_blk);
+  gp_free_idle(b->cell_occ);
+  gp_free_idle(b->sigma);
+  gp_free_idle(b->seeds);
+  gp_free_idle(b->perm);
+  gp_free_idle(b->inv_perm);
+  gp_free_idle(b->order_tiles);
+  gp_free_idle(b->emit_order);
+  gp_free_idle(b->emit_slot);
+  gp_free_idle(b->emit_pts);
+  gp_free_idle(b->partials);
+  gp_free_idle(b->dev_ints);
   delete b;
 }
 
 struct TempBufs {
+  gp_ctx* ctx;
   std::vector<void*> ptrs;
+  explicit TempBufs(gp_ctx* c) : ctx(c) {}
   ~TempBufs() {
-    for (void* p : ptrs) cudaFree(p);
+    for (void* p : ptrs) gp_free(ctx, p);
   }
   template <typename T>
-  gp_status alloc(gp_ctx* ctx, T** p, size_t n, const char* what) {
-    gp_status st = gp_alloc(ctx, p, n, what);
+  gp_status alloc(gp_ctx* c, T** p, size_t n, const char* what) {
+    gp_status st = gp_alloc(c, p, n, what);
     if (!st) ptrs.push_back(*p);
     return st;
   }
@@ -351,7 +354,7 @@ gp_status build_band_sets(gp_band* b, const float* pts_dev) {
   const int R = b->R;
   const int nb = b->nb;
   const int64_t nbr = (int64_t)nb * nb * nb;
-  TempBufs tmp;
+  TempBufs tmp(ctx);
   const CellRows cr{R, (R + 31) / 32};
   const VertRows vr{R + 1, (R + 32) / 32};
   const int64_t nc = (int64_t)R * R * cr.W, nv = (int64_t)vr.n * vr.n * vr.W;
@@ -517,9 +520,8 @@ extern "C" void gp_band_destroy(gp_band* band) {
   if (!band) return;
   gp_ctx* ctx = band->ctx;
   cudaSetDevice(ctx->device);
-  cudaStreamSynchronize(ctx->stream);
-  cudaGetLastError();
   band_free(band);
+  cudaGetLastError();
   ctx->live_bands -= 1;
   if (ctx->live_bands == 0 && ctx->destroy_pending) gp_ctx_release(ctx);
 }

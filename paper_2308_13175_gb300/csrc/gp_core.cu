@@ -1,5 +1,7 @@
 // Context, errors and the device-wide scan used by the set-up paths.
 #include <cstdio>
+#include <map>
+#include <mutex>
 #include <string>
 
 #include "gp_internal.cuh"
@@ -15,6 +17,47 @@ gp_status gp_cuda_fail(gp_ctx* ctx, cudaError_t e, const char* what) {
   return gp_fail(ctx, GP_ERR_CUDA, msg);
 }
 
+namespace {
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  int64_t users = 0;
+};
+std::mutex g_pool_mutex;
+std::map<int, DevicePool>& device_pools() {
+  static std::map<int, DevicePool>* pools = new std::map<int, DevicePool>();  // outlives every context
+  return *pools;
+}
+}  // namespace
+
+cudaError_t gp_pool_acquire(int device, cudaMemPool_t* pool) {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = device_pools()[device];
+  if (!d.pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaError_t e = cudaMemPoolCreate(&d.pool, &props);
+    if (e != cudaSuccess) {
+      d.pool = nullptr;
+      return e;
+    }
+    uint64_t keep = GP_POOL_KEEP;
+    e = cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) return e;
+  }
+  d.users += 1;
+  *pool = d.pool;
+  return cudaSuccess;
+}
+
+void gp_pool_release(int device) {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = device_pools()[device];
+  if (d.users > 0) d.users -= 1;
+  if (d.users == 0 && d.pool) cudaMemPoolTrimTo(d.pool, 0);
+}
+
 extern "C" gp_status gp_create(gp_ctx** out, int device, void* stream) {
   if (!out) return GP_ERR_ARG;
   *out = nullptr;
@@ -28,7 +71,8 @@ extern "C" gp_status gp_create(gp_ctx** out, int device, void* stream) {
   ctx->device = device;
   ctx->stream = (cudaStream_t)stream;
   if (cudaSetDevice(device) != cudaSuccess ||
-      cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) {
+      cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      gp_pool_acquire(device, &ctx->pool) != cudaSuccess) {
     cudaGetLastError();
     delete ctx;
     return GP_ERR_CUDA;
@@ -58,6 +102,7 @@ void gp_ctx_release(gp_ctx* ctx) {
     if (r.stop) cudaEventDestroy(r.stop);
   }
   for (auto e : ctx->event_pool) cudaEventDestroy(e);
+  gp_pool_release(ctx->device);
   delete ctx;
 }
 
@@ -198,40 +243,36 @@ __global__ void k_scan_add(int32_t* __restrict__ data, int64_t n, const int32_t*
     if (idx < n) data[idx] += add;
 }
 
-gp_status scan_rec(gp_ctx* ctx, int32_t* data, int64_t n) {
-  int64_t tiles = (n + SCAN_TILE - 1) / SCAN_TILE;
-  int32_t* sums = nullptr;
-  gp_status st = gp_alloc(ctx, &sums, (size_t)tiles, "scan tile sums");
-  if (st) return st;
-  k_scan_tiles<<<(unsigned)tiles, SCAN_THREADS, 0, ctx->stream>>>(data, n, sums);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && tiles > 1) {
-    st = scan_rec(ctx, sums, tiles);
-    if (!st) {
-      k_scan_add<<<(unsigned)tiles, SCAN_THREADS, 0, ctx->stream>>>(data, n, sums);
-      e = cudaGetLastError();
-    }
-  }
-  cudaStreamSynchronize(ctx->stream);
-  cudaFree(sums);
-  if (st) return st;
-  if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "scan kernels");
-  return GP_OK;
-}
 }  // namespace
 
+// Level l + 1 scans the tile sums of level l; the last level is one tile,
+// whose sum is the total.
 gp_status gp_exclusive_scan_i32(gp_ctx* ctx, int32_t* data, int64_t n, int64_t* total_host) {
-  if (n <= 0) {
-    if (total_host) *total_host = 0;
-    return GP_OK;
+  if (total_host) *total_host = 0;
+  if (n <= 0) return GP_OK;
+  constexpr int LEVELS = 4;  // SCAN_TILE^4 > 2^31
+  int32_t* level[LEVELS + 1] = {data};
+  int64_t len[LEVELS + 1] = {n};
+  int depth = 0;
+  gp_status st = GP_OK;
+  cudaError_t e = cudaSuccess;
+  do {
+    const int64_t tiles = (len[depth] + SCAN_TILE - 1) / SCAN_TILE;
+    if ((st = gp_alloc(ctx, &level[depth + 1], (size_t)tiles, "scan tile sums"))) break;
+    k_scan_tiles<<<(unsigned)tiles, SCAN_THREADS, 0, ctx->stream>>>(level[depth], len[depth], level[depth + 1]);
+    e = cudaGetLastError();
+    len[++depth] = tiles;
+  } while (e == cudaSuccess && len[depth] > 1 && depth < LEVELS);
+  for (int l = depth - 2; l >= 0 && !st && e == cudaSuccess; --l) {
+    k_scan_add<<<(unsigned)len[l + 1], SCAN_THREADS, 0, ctx->stream>>>(level[l], len[l], level[l + 1]);
+    e = cudaGetLastError();
   }
-  int32_t last_in = 0, last_out = 0;
-  GP_CUDA(ctx, cudaMemcpyAsync(&last_in, data + n - 1, 4, cudaMemcpyDeviceToHost, ctx->stream));
-  GP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  gp_status st = scan_rec(ctx, data, n);
+  int32_t total = 0;
+  if (!st && e == cudaSuccess) e = cudaMemcpyAsync(&total, level[depth], 4, cudaMemcpyDeviceToHost, ctx->stream);
+  if (!st && e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  for (int l = 1; l <= depth; ++l) gp_free(ctx, level[l]);
   if (st) return st;
-  GP_CUDA(ctx, cudaMemcpyAsync(&last_out, data + n - 1, 4, cudaMemcpyDeviceToHost, ctx->stream));
-  GP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-  if (total_host) *total_host = (int64_t)last_out + last_in;
+  if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "scan kernels");
+  if (total_host) *total_host = total;
   return GP_OK;
 }

@@ -168,7 +168,7 @@ extern "C" gp_status gp_eval_nearest(gp_band* b, const float* q_dev, const float
   gp_status st = gp_alloc(ctx, &nn, (size_t)n, "eval nn");
   if (st) return st;
   if ((st = gp_alloc(ctx, &acc, EV_SUMS + 1, "eval sums"))) {
-    gp_free(nn);
+    gp_free(ctx, nn);
     return st;
   }
   double host[EV_SUMS + 1];
@@ -187,8 +187,8 @@ extern "C" gp_status gp_eval_nearest(gp_band* b, const float* q_dev, const float
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) { st = gp_cuda_fail(ctx, e, "gp_eval_nearest"); break; }
   } while (false);
-  gp_free(nn);
-  gp_free(acc);
+  gp_free(ctx, nn);
+  gp_free(ctx, acc);
   if (st) return st;
   const double W = host[0];
   out_host[0] = W;

@@ -32,7 +32,18 @@ struct gp_ctx {
   // release until the last of them is destroyed.
   int64_t live_bands = 0;
   bool destroy_pending = false;
+  // The device's memory pool, shared by its contexts (gp_pool_acquire).
+  cudaMemPool_t pool = nullptr;
+  bool mesh_table = false;  // the case table is in this device's constant memory
 };
+
+// The library's memory pool of a device: created by the first context on it,
+// keeping at most GP_POOL_KEEP bytes of freed memory between calls and none
+// once the last context is released.  Stream ordered, so safe with several
+// threads and streams.
+constexpr uint64_t GP_POOL_KEEP = uint64_t(256) << 20;
+cudaError_t gp_pool_acquire(int device, cudaMemPool_t* pool);
+void gp_pool_release(int device);
 
 // Release a context's memory (called when no band refers to it any more).
 void gp_ctx_release(gp_ctx* ctx);
@@ -129,22 +140,33 @@ gp_status gp_cuda_fail(gp_ctx* ctx, cudaError_t e, const char* what);
     if (_e != cudaSuccess) return gp_cuda_fail(ctx, _e, what); \
   } while (0)
 
+// Device memory from the context's pool, for work on its stream (or, after a
+// synchronisation of that stream, on any).  cudaMalloc and cudaFree take about
+// 20 us each, and a band 49 of either: 1.7 of the 2.9 ms that a band of 100,000
+// points took to build.
 template <typename T>
 gp_status gp_alloc(gp_ctx* ctx, T** p, size_t count, const char* what) {
   *p = nullptr;
   if (count == 0) count = 1;
-  cudaError_t e = cudaMalloc((void**)p, count * sizeof(T));
+  cudaError_t e = cudaMallocFromPoolAsync((void**)p, count * sizeof(T), ctx->pool, ctx->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
     return gp_fail(ctx, e == cudaErrorMemoryAllocation ? GP_ERR_OOM : GP_ERR_CUDA,
-                   std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
+                   std::string("allocation failed for ") + what + ": " + cudaGetErrorString(e));
   }
   return GP_OK;
 }
 
-inline void gp_free(void* p) {
-  if (p) cudaFree(p);
+// Scratch of a call on the context's stream: freed in stream order.
+inline void gp_free(gp_ctx* ctx, void* p) {
+  if (p) cudaFreeAsync(p, ctx->stream);
+}
+
+// Memory that any stream may have used: freed after the caller has
+// synchronised the device (the context's stream may be gone by then).
+inline void gp_free_idle(void* p) {
+  if (p) cudaFreeAsync(p, nullptr);
 }
 
 inline unsigned gp_blocks(int64_t n, int threads, int64_t cap = 1 << 30) {

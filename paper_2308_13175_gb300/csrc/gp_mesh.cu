@@ -431,7 +431,11 @@ extern "C" gp_status gp_mesh_extract(gp_band* b, float iso, float* tri_dev, int6
   if (b->n_active == 0) return GP_OK;
   const McTable* table = mc_table();
   if (!table) return gp_fail(ctx, GP_ERR_STATE, "gp_mesh_extract: case table failed its own checks");
-  GP_CUDA(ctx, cudaMemcpyToSymbolAsync(c_mc, table, sizeof(McTable), 0, cudaMemcpyHostToDevice, ctx->stream));
+  if (!ctx->mesh_table) {  // once: the table never changes
+    GP_CUDA(ctx, cudaMemcpyToSymbolAsync(c_mc, table, sizeof(McTable), 0, cudaMemcpyHostToDevice, ctx->stream));
+    GP_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    ctx->mesh_table = true;
+  }
 
   MeshArgs a;
   a.active = b->active;
@@ -478,10 +482,9 @@ extern "C" gp_status gp_mesh_extract(gp_band* b, float iso, float* tri_dev, int6
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) { st = gp_cuda_fail(ctx, e, "k_mesh_emit"); break; }
-    // counts is freed below: wait until the emit pass has read it.
     e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) st = gp_cuda_fail(ctx, e, "gp_mesh_extract");
   } while (false);
-  gp_free(counts);
+  gp_free(ctx, counts);
   return st;
 }

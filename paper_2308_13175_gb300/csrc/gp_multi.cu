@@ -520,16 +520,17 @@ namespace {
 
 void multi_free(gp_multi* m) {
   if (!m) return;
+  cudaDeviceSynchronize();  // any stream may have worked on the buffers
   for (void* p : {(void*)m->shapes, (void*)m->rec_tiles, (void*)m->pt_tiles, (void*)m->brick_tiles,
                   (void*)m->active_tiles, (void*)m->q, (void*)m->rec, (void*)m->grad, (void*)m->src,
                   (void*)m->perm, (void*)m->inv, (void*)m->eslot, (void*)m->counts, (void*)m->nvalid, (void*)m->err,
                   (void*)m->sums, (void*)m->acc, (void*)m->isums, (void*)m->t, (void*)m->perm_epoch})
-    gp_free(p);
+    gp_free_idle(p);
   delete m;
 }
 
 gp_status upload_tiles(gp_ctx* ctx, const std::vector<MTile>& h, MTile** d, int64_t* n) {
-  gp_free(*d);
+  gp_free(ctx, *d);
   *d = nullptr;
   *n = (int64_t)h.size();
   gp_status st = gp_alloc(ctx, d, h.size(), "multi tiles");
@@ -777,7 +778,6 @@ extern "C" gp_status gp_multi_create(gp_ctx* ctx, gp_band* const* bands, int32_t
 
 extern "C" void gp_multi_destroy(gp_multi* m) {
   if (!m) return;
-  cudaStreamSynchronize(m->ctx->stream);
   multi_free(m);
 }
 

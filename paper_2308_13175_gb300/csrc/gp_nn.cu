@@ -556,12 +556,12 @@ static gp_status build_emit_order(gp_band* b) {
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
-  gp_free(key[0]);
-  gp_free(key[1]);
-  gp_free(counts);
-  gp_free(val[cur ^ 1]);
+  gp_free(ctx, key[0]);
+  gp_free(ctx, key[1]);
+  gp_free(ctx, counts);
+  gp_free(ctx, val[cur ^ 1]);
   if (st || e != cudaSuccess) {
-    gp_free(val[cur]);
+    gp_free(ctx, val[cur]);
     return st ? st : gp_cuda_fail(ctx, e, "emission order");
   }
   b->emit_order = val[cur];
@@ -639,10 +639,10 @@ gp_status gp_build_points(gp_band* b, const float* pts_dev) {
     e = cudaGetLastError();
   }
   cudaStreamSynchronize(s);
-  gp_free(bid);
-  gp_free(start);
-  gp_free(cursor);
-  gp_free(by_block);
+  gp_free(ctx, bid);
+  gp_free(ctx, start);
+  gp_free(ctx, cursor);
+  gp_free(ctx, by_block);
   if (st) return st;
   if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "point cell list");
   g = make_grid(b);
@@ -731,7 +731,7 @@ extern "C" gp_status gp_nn_work(gp_band* b, const float* q_dev, int64_t n, const
     if (!st && e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
     *work_host = (int64_t)h;
   }
-  cudaFree(dev);
+  gp_free(ctx, dev);
   if (st) return st;
   if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "gp_nn_work");
   return GP_OK;

@@ -675,7 +675,7 @@ extern "C" gp_status gp_band_autotune(gp_band* b, const float* rec_dev, int64_t 
   gp_status st = gp_alloc(ctx, &grad, b->V_stored(), "autotune gradient");
   if (st) return st;
   if ((st = gp_alloc(ctx, &loss, 8, "autotune loss"))) {
-    cudaFree(grad);
+    gp_free(ctx, grad);
     return st;
   }
   Grid G;
@@ -782,8 +782,8 @@ extern "C" gp_status gp_band_autotune(gp_band* b, const float* rec_dev, int64_t 
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   cudaStreamSynchronize(s);
-  cudaFree(grad);
-  cudaFree(loss);
+  gp_free(ctx, grad);
+  gp_free(ctx, loss);
   if (e != cudaSuccess) return gp_cuda_fail(ctx, e, "gp_band_autotune");
   b->q_rpt = best_rpt;
   b->q_bps = best_bps;
