@@ -112,10 +112,12 @@ struct WindowSink {
   float* acc;  // shared: WIN_V sums
   const Win& W;
   int32_t* __restrict__ err;
-  __device__ __forceinline__ void cell(const int c[3], int slot, const float t[3], float A, const float Gt[3]) {
+  __device__ __forceinline__ void cell(const int c[3], int slot, const int*, const float t[3], float A, const float Gt[3]) {
     const int b0 = win_cell(W, c);
     if (b0 < 0) {
-      scatter8<false>(G, grad, nullptr, err, c, slot, t, A, Gt);
+      int s[8];
+      cell_slots(G, c, slot, s);
+      scatter8<false>(G, grad, nullptr, err, c, s, t, A, Gt);
       return;
     }
     float v[8];

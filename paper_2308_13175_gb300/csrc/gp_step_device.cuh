@@ -24,46 +24,57 @@ struct Eval {
   float gt[3];  // df/dt (t = local coordinate in cell units)
 };
 
-// The 8 corner values of cell c (corner k = dx + 2 dy + 4 dz).  Inside a
-// brick the two corners (x, x + 1) of each of the cell's four x edges are
-// adjacent floats: one 8-byte load per edge at even x, one aligned 16-byte
-// load from x - 1 at x = 1 mod 4, two 4-byte loads at x = 3 mod 4.  A cell
-// whose corners span bricks looks each corner's brick up.
-__device__ __forceinline__ void load_corners(const Grid& G, const int c[3], int slot, float d[8], bool& ok) {
-  if ((c[0] & 7) != 7 && (c[1] & 7) != 7 && (c[2] & 7) != 7) {
-    const float* base = G.D + gp_vaddr(slot, c[0], c[1], c[2]);
-    const int xm = c[0] & 3;
-    if ((xm & 1) == 0) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(base + (e & 1) * 8 + (e >> 1) * 64));
-        d[2 * e] = v.x;
-        d[2 * e + 1] = v.y;
-      }
-    } else if (xm == 1) {
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float4 v = __ldg(reinterpret_cast<const float4*>(base - 1 + (e & 1) * 8 + (e >> 1) * 64));
-        d[2 * e] = v.y;
-        d[2 * e + 1] = v.z;
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) d[k] = __ldg(base + (k & 1) + ((k >> 1) & 1) * 8 + (k >> 2) * 64);
-    }
-    return;
-  }
+// The slots of the bricks that hold the corners of cell c (corner
+// k = dx + 2 dy + 4 dz), slot being the cell's own.  Only corners in a
+// neighbouring brick are looked up; -1 where that brick is not stored.  One
+// path serves all cells, here and in the loads and sums below: with a path each
+// for cells inside a brick (by x mod 4) and across bricks, the lanes of a warp
+// took them all in turn (k_query_ilp: 206 -> 164 us for 2,097,152 records of a
+// 1024^3 band, 49 -> 40 us for 262,144 in no order on a 256^3 one, 521 -> 468 us
+// for 4,194,304 with the fixed-point sums; k_m_query 334 -> 226 us).
+__device__ __forceinline__ void cell_slots(const Grid& G, const int c[3], int slot, int s[8]) {
+  const int ox = (c[0] & 7) == 7 ? 1 : 0, oy = (c[1] & 7) == 7 ? G.nb : 0, oz = (c[2] & 7) == 7 ? G.nb * G.nb : 0;
+  const int32_t* T = G.table + ((int64_t)(c[2] >> 3) * G.nb + (c[1] >> 3)) * G.nb + (c[0] >> 3);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    int i = c[0] + (k & 1), j = c[1] + ((k >> 1) & 1), kk = c[2] + (k >> 2);
-    int s = gp_brick_slot(G.table, G.nb, i, j, kk);
-    if (s < 0) {
-      ok = false;
-      d[k] = 0.f;
+    const int off = ((k & 1) ? ox : 0) + ((k & 2) ? oy : 0) + ((k & 4) ? oz : 0);
+    s[k] = slot;
+    if (off) s[k] = __ldg(T + off);
+  }
+}
+
+// Place of corner k of cell c in its brick.
+__device__ __forceinline__ int corner_local(const int c[3], int k) {
+  return gp_local(c[0] + (k & 1), c[1] + ((k >> 1) & 1), c[2] + (k >> 2));
+}
+
+// The 8 corner values, along x in pairs: one 8-byte load at even x (both lie
+// in one brick), two single ones at odd x (an aligned 16-byte load for all of
+// them holds twice the registers: 178 -> 234 us on the first of those batches).
+// A missing brick turns ok false.
+__device__ __forceinline__ void load_corners_at(const Grid& G, const int c[3], const int s[8], float d[8], bool& ok) {
+  const bool even = (c[0] & 1) == 0;
+#pragma unroll
+  for (int e = 0; e < 8; e += 2) {
+    const bool have = s[e] >= 0 && s[e + 1] >= 0;
+    if (!have) ok = false;
+    const float* lo = G.D + ((int64_t)(have ? s[e] : s[0]) * 512 + corner_local(c, e));
+    const float* hi = G.D + ((int64_t)(have ? s[e + 1] : s[0]) * 512 + corner_local(c, e + 1));
+    if (even) {
+      const float2 v = __ldg(reinterpret_cast<const float2*>(lo));
+      d[e] = v.x;
+      d[e + 1] = v.y;
     } else {
-      d[k] = __ldg(G.D + gp_vaddr(s, i, j, kk));
+      d[e] = __ldg(lo);
+      d[e + 1] = __ldg(hi);
     }
   }
+}
+
+__device__ __forceinline__ void load_corners(const Grid& G, const int c[3], int slot, float d[8], bool& ok) {
+  int s[8];
+  cell_slots(G, c, slot, s);
+  load_corners_at(G, c, s, d, ok);
 }
 
 // Trilinear interpolation of Eq. 3.  f is a lerp along x, then y, then z.
@@ -147,77 +158,59 @@ __host__ __device__ __forceinline__ bool fix_split(float v, long long& hi, long 
   return true;
 }
 
-// Scatter of one cell's 8 corner contributions.
-template <bool DET>
-__device__ __forceinline__ void scatter8(const Grid& G, float* __restrict__ grad, unsigned long long* __restrict__ acc,
-                                         int32_t* __restrict__ err, const int c[3], int slot, const float t[3],
-                                         float A, const float Gt[3]) {
-  float wx[2] = {1.f - t[0], t[0]}, wy[2] = {1.f - t[1], t[1]}, wz[2] = {1.f - t[2], t[2]};
-  bool fast = (c[0] & 7) != 7 && (c[1] & 7) != 7 && (c[2] & 7) != 7;
-  if (!DET && fast && (c[0] & 3) != 3) {
-    // The corners (x, x + 1) of each of the 4 (y, z) edges are adjacent: one
-    // vector reduction per edge - 8 bytes at even x, 16 bytes from x - 1 (the
-    // outer two lanes adding zero) at x = 1 mod 4.
-    float* base = grad + gp_vaddr(slot, c[0], c[1], c[2]);
-    const bool odd = c[0] & 1;
+// dL/dd_c of the cell's corner c = dx + 2 dy + 4 dz from dL/df = A and
+// dL/dt = Gt at local coordinate t: A w_c(t) + sum_a Gt_a dw_c/dt_a, per x edge
+// the part that both corners share and the difference along x.
+__device__ __forceinline__ void corner_values(const float t[3], float A, const float Gt[3], float v[8]) {
+  const float wy[2] = {1.f - t[1], t[1]}, wz[2] = {1.f - t[2], t[2]};
+  const float gy[2] = {Gt[1] * wz[0], Gt[1] * wz[1]}, gz[2] = {Gt[2] * wy[0], Gt[2] * wy[1]};
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int dy = e & 1, dz = e >> 1;
-      const float sy = dy ? 1.f : -1.f, sz = dz ? 1.f : -1.f;
-      const float wyz = wy[dy] * wz[dz];
-      float v[2];
-#pragma unroll
-      for (int dx = 0; dx < 2; ++dx) {
-        const float sx = dx ? 1.f : -1.f;
-        v[dx] = A * wx[dx] * wyz + Gt[0] * sx * wyz + Gt[1] * wx[dx] * sy * wz[dz] + Gt[2] * wx[dx] * wy[dy] * sz;
-      }
-      if (odd)
-        red_add_v4(base - 1 + dy * 8 + dz * 64, 0.f, v[0], v[1], 0.f);
-      else
-        red_add_v2(base + dy * 8 + dz * 64, v[0], v[1]);
-    }
-    return;
-  }
-#pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
-    float sx = dx ? 1.f : -1.f, sy = dy ? 1.f : -1.f, sz = dz ? 1.f : -1.f;
-    float wyz = wy[dy] * wz[dz];
-    float val = A * wx[dx] * wyz + Gt[0] * sx * wyz + Gt[1] * wx[dx] * sy * wz[dz] + Gt[2] * wx[dx] * wy[dy] * sz;
-    int64_t addr;
-    if (fast) {
-      addr = gp_vaddr(slot, c[0], c[1], c[2]) + dx + dy * 8 + dz * 64;
-    } else {
-      int i = c[0] + dx, j = c[1] + dy, kk = c[2] + dz;
-      int s = gp_brick_slot(G.table, G.nb, i, j, kk);
-      if (s < 0) continue;
-      addr = gp_vaddr(s, i, j, kk);
-    }
-    if (DET) {
-      long long hi, lo;
-      if (!fix_split(val, hi, lo)) {
-        atomicOr(err, GP_EF_NUMERIC);
-        continue;
-      }
-      if (hi) atomicAdd(acc + 2 * addr, (unsigned long long)hi);
-      if (lo) atomicAdd(acc + 2 * addr + 1, (unsigned long long)lo);
-    } else {
-      atomicAdd(grad + addr, val);
-    }
+  for (int e = 0; e < 4; ++e) {
+    const int dy = e & 1, dz = e >> 1;
+    const float wyz = wy[dy] * wz[dz];
+    const float p = fmaf(A, wyz, (dy ? gy[dz] : -gy[dz]) + (dz ? gz[dy] : -gz[dy])), q = Gt[0] * wyz;
+    v[2 * e] = fmaf(p, 1.f - t[0], -q);
+    v[2 * e + 1] = fmaf(p, t[0], q);
   }
 }
 
+// One contribution into the fixed-point sums.
+__device__ __forceinline__ void scatter_fixed(unsigned long long* __restrict__ acc, int32_t* __restrict__ err,
+                                              int64_t at, float v) {
+  long long hi, lo;
+  if (!fix_split(v, hi, lo)) {
+    atomicOr(err, GP_EF_NUMERIC);
+    return;
+  }
+  if (hi) atomicAdd(acc + 2 * at, (unsigned long long)hi);
+  if (lo) atomicAdd(acc + 2 * at + 1, (unsigned long long)lo);
+}
 
-// dL/dd_c of the cell's corner c = dx + 2 dy + 4 dz from dL/df = A and
-// dL/dt = Gt at local coordinate t: A w_c(t) + sum_a Gt_a dw_c/dt_a.
-__device__ __forceinline__ void corner_values(const float t[3], float A, const float Gt[3], float v[8]) {
-  const float wx[2] = {1.f - t[0], t[0]}, wy[2] = {1.f - t[1], t[1]}, wz[2] = {1.f - t[2], t[2]};
+// Scatter of one cell's 8 corner contributions: computed once, then per edge
+// one vector reduction (8 bytes at even x, 16 bytes from x - 1 at x = 1 mod 4,
+// the outer two lanes adding zero) or, at x = 3 mod 4, two single ones.  Every
+// corner is stored: load_corners found them.
+template <bool DET>
+__device__ __forceinline__ void scatter8(const Grid& G, float* __restrict__ grad, unsigned long long* __restrict__ acc,
+                                         int32_t* __restrict__ err, const int c[3], const int s[8], const float t[3],
+                                         float A, const float Gt[3]) {
+  float v[8];
+  corner_values(t, A, Gt, v);
+  const int xm = c[0] & 3;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int dx = k & 1, dy = (k >> 1) & 1, dz = k >> 2;
-    const float sx = dx ? 1.f : -1.f, sy = dy ? 1.f : -1.f, sz = dz ? 1.f : -1.f;
-    const float wyz = wy[dy] * wz[dz];
-    v[k] = A * wx[dx] * wyz + Gt[0] * sx * wyz + Gt[1] * wx[dx] * sy * wz[dz] + Gt[2] * wx[dx] * wy[dy] * sz;
+  for (int e = 0; e < 8; e += 2) {
+    const int64_t lo = (int64_t)s[e] * 512 + corner_local(c, e), hi = (int64_t)s[e + 1] * 512 + corner_local(c, e + 1);
+    if (DET) {
+      scatter_fixed(acc, err, lo, v[e]);
+      scatter_fixed(acc, err, hi, v[e + 1]);
+      continue;
+    }
+    if (xm == 1) red_add_v4(grad + lo - 1, 0.f, v[e], v[e + 1], 0.f);
+    if (!(xm & 1)) red_add_v2(grad + lo, v[e], v[e + 1]);
+    if (xm == 3) {
+      atomicAdd(grad + lo, v[e]);
+      atomicAdd(grad + hi, v[e + 1]);
+    }
   }
 }
 
@@ -229,8 +222,9 @@ struct GlobalSink {
   float* __restrict__ grad;
   unsigned long long* __restrict__ acc;
   int32_t* __restrict__ err;
-  __device__ __forceinline__ void cell(const int c[3], int slot, const float t[3], float A, const float Gt[3]) {
-    scatter8<DET>(G, grad, acc, err, c, slot, t, A, Gt);
+  __device__ __forceinline__ void cell(const int c[3], int, const int s[8], const float t[3], float A,
+                                       const float Gt[3]) {
+    scatter8<DET>(G, grad, acc, err, c, s, t, A, Gt);
   }
 };
 
@@ -312,6 +306,7 @@ struct RecState {
   int lq, ls;
   uint32_t wq, ws;
   float dq[8], ds[8];
+  int sq[8], ss[8];  // the corners' brick slots (not set by the windowed forms)
   bool ok;       // still a candidate for a valid record
   bool corners;  // every corner was found in the band
 };
@@ -327,6 +322,8 @@ __device__ __forceinline__ void rec_phase_a(const Grid& G, const float q[3], con
   if (!R.ok) return;
   R.C.slot_q = gp_brick_slot(G.table, G.nb, R.C.cq[0], R.C.cq[1], R.C.cq[2]);
   R.C.slot_s = gp_brick_slot(G.table, G.nb, R.C.cs[0], R.C.cs[1], R.C.cs[2]);
+  cell_slots(G, R.C.cq, R.C.slot_q, R.sq);
+  cell_slots(G, R.C.cs, R.C.slot_s, R.ss);
 }
 
 __device__ __forceinline__ void rec_phase_b(const Grid& G, RecState& R) {
@@ -340,8 +337,8 @@ __device__ __forceinline__ void rec_phase_b(const Grid& G, RecState& R) {
   R.wq = __ldg(G.masks + (int64_t)R.C.slot_q * 48 + 32 + (R.lq >> 5));
   R.ws = __ldg(G.masks + (int64_t)R.C.slot_s * 48 + 32 + (R.ls >> 5));
   R.corners = true;
-  load_corners(G, R.C.cq, R.C.slot_q, R.dq, R.corners);
-  load_corners(G, R.C.cs, R.C.slot_s, R.ds, R.corners);
+  load_corners_at(G, R.C.cq, R.sq, R.dq, R.corners);
+  load_corners_at(G, R.C.cs, R.ss, R.ds, R.corners);
 }
 
 // Validity (cell(q) and cell(s) in the pull band, Sec. 3), the forward terms
@@ -380,8 +377,8 @@ __device__ __forceinline__ bool rec_phase_c(const Grid& G, RecState& R, float w,
   float Gq[3], Gs[3], dfq;
   backward_terms(q, s, f, nv, ns, lp, inv, invs, big, bigs, w, gamma, G.half_r, Gq, Gs, dfq);
   float dfs = fs > 0.f ? w * beta : (fs < 0.f ? -w * beta : 0.f);
-  sink.cell(C.cq, C.slot_q, C.tq, dfq, Gq);
-  sink.cell(C.cs, C.slot_s, C.ts, dfs, Gs);
+  sink.cell(C.cq, C.slot_q, R.sq, C.tq, dfq, Gq);
+  sink.cell(C.cs, C.slot_s, R.ss, C.ts, dfs, Gs);
   return true;
 }
 
