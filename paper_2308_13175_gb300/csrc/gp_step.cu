@@ -90,13 +90,40 @@ __device__ void finish_if_last(const double* __restrict__ partials, const FinalA
   if (threadIdx.x == 0) *fa.done = 0;
 }
 
-__global__ void k_count_valid(Grid G, const float* __restrict__ rec, int64_t B, int32_t* __restrict__ nvalid) {
+// B_v over the records: classify(), with the dependent reads (slots, then mask
+// words) of a thread's COUNT_RPT records issued level by level.  Bound by their
+// latency, so the grid fills the SM's COUNT_BLOCKS_PER_SM resident blocks.
+// 4,194,304 records of a 512^3 band 69.8 -> 42.8 us, 262,144 on a 256^3 one
+// 6.4 -> 5.9 us, against a record a thread in three blocks an SM.
+constexpr int COUNT_RPT = 2;
+constexpr int COUNT_BLOCKS_PER_SM = 6;
+__global__ void __launch_bounds__(Q_THREADS, COUNT_BLOCKS_PER_SM)
+    k_count_valid(Grid G, const float* __restrict__ rec, int64_t B, int32_t* __restrict__ nvalid) {
   int cnt = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < B; i += (int64_t)gridDim.x * blockDim.x) {
-    float q[3], s[3];
-    load_rec(rec, i, q, s);
-    Cells C;
-    cnt += classify(G, q, s, C) ? 1 : 0;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < B; i0 += COUNT_RPT * stride) {
+    int slot[COUNT_RPT][2], cell[COUNT_RPT][2];
+#pragma unroll
+    for (int r = 0; r < COUNT_RPT; ++r) {
+      const int64_t i = i0 + r * stride;
+      float q[3], s[3];
+      load_rec(rec, i < B ? i : i0, q, s);
+      Cells C;
+      slot[r][0] = slot[r][1] = -1;
+      if (i < B && classify_cells(G, q, s, C)) {
+        slot[r][0] = gp_brick_slot(G.table, G.nb, C.cq[0], C.cq[1], C.cq[2]);
+        slot[r][1] = gp_brick_slot(G.table, G.nb, C.cs[0], C.cs[1], C.cs[2]);
+        cell[r][0] = gp_local(C.cq[0], C.cq[1], C.cq[2]);
+        cell[r][1] = gp_local(C.cs[0], C.cs[1], C.cs[2]);
+      }
+    }
+    bool in[COUNT_RPT][2];
+#pragma unroll
+    for (int r = 0; r < COUNT_RPT; ++r)
+#pragma unroll
+      for (int p = 0; p < 2; ++p) in[r][p] = slot[r][p] >= 0 && gp_mask_bit(G.masks, slot[r][p], 2, cell[r][p]);
+#pragma unroll
+    for (int r = 0; r < COUNT_RPT; ++r) cnt += in[r][0] && in[r][1] ? 1 : 0;
   }
   int w = gp_warp_sum_i(cnt);
   if ((threadIdx.x & 31) == 0 && w) atomicAdd(nvalid, w);
@@ -526,6 +553,10 @@ unsigned q_grid(const gp_ctx* ctx, int64_t B) {
   return gp_blocks(B, Q_THREADS, cap);
 }
 
+unsigned count_grid(const gp_ctx* ctx, int64_t B) {
+  return gp_blocks(B, Q_THREADS * COUNT_RPT, (int64_t)ctx->num_sms * COUNT_BLOCKS_PER_SM);
+}
+
 unsigned tv_grid(const gp_ctx* ctx, int64_t n_bricks) {
   int64_t cap = (int64_t)ctx->num_sms * TV_BLOCKS_PER_SM;  // persistent: one wave
   if (cap > GP_MAX_PARTIAL_BLOCKS) cap = GP_MAX_PARTIAL_BLOCKS;
@@ -566,7 +597,7 @@ extern "C" gp_status gp_step(gp_band* b, const float* rec_dev, int64_t B, const 
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
     GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     if (B > 0) {
-      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<q_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
+      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
     }
     bv = cnt;
   }
@@ -692,7 +723,7 @@ extern "C" gp_status gp_band_autotune(gp_band* b, const float* rec_dev, int64_t 
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
     e = cudaMemsetAsync(cnt, 0, sizeof(int32_t), s);
     if (e == cudaSuccess) {
-      k_count_valid<<<q_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt);
+      k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt);
       e = cudaGetLastError();
     }
     bv = cnt;
@@ -849,7 +880,7 @@ extern "C" gp_status gp_step_update(gp_band* b, const float* rec_dev, int64_t B,
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
     GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     if (B > 0) {
-      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<q_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
+      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
     }
     bv = cnt;
   }
