@@ -65,7 +65,8 @@ void gp_prof_post(gp_ctx* ctx, const char* name);
 // Number of fp64 partial-sum slots the reduction kernels may use per call.
 constexpr int GP_MAX_PARTIAL_BLOCKS = 4096;
 // Device int slots of gp_band::dev_ints.
-enum { GP_DI_NVALID = 0, GP_DI_ERROR = 1, GP_DI_DONE = 2, GP_DI_COUNT = 8 };
+// GP_DI_TALLY is 64 bits wide (k_count_valid; 0 between launches).
+enum { GP_DI_NVALID = 0, GP_DI_ERROR = 1, GP_DI_DONE = 2, GP_DI_TALLY = 4, GP_DI_COUNT = 8 };
 // Error bits raised by kernels in dev_ints[GP_DI_ERROR].
 enum { GP_EF_NUMERIC = 1, GP_EF_TIMEOUT = 2, GP_EF_RANGE = 4 };
 

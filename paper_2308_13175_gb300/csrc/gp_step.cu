@@ -94,11 +94,16 @@ __device__ void finish_if_last(const double* __restrict__ partials, const FinalA
 // words) of a thread's COUNT_RPT records issued level by level.  Bound by their
 // latency, so the grid fills the SM's COUNT_BLOCKS_PER_SM resident blocks.
 // 4,194,304 records of a 512^3 band 69.8 -> 42.8 us, 262,144 on a 256^3 one
-// 6.4 -> 5.9 us, against a record a thread in three blocks an SM.
+// 6.4 -> 5.9 us, against a record a thread in three blocks an SM.  The blocks add
+// their counts and themselves to one 64-bit tally; the last one writes the
+// count and clears the tally, so no launch clears the count first: a step of
+// 262,144 records 71.5 -> 67.9 us.
 constexpr int COUNT_RPT = 2;
 constexpr int COUNT_BLOCKS_PER_SM = 6;
 __global__ void __launch_bounds__(Q_THREADS, COUNT_BLOCKS_PER_SM)
-    k_count_valid(Grid G, const float* __restrict__ rec, int64_t B, int32_t* __restrict__ nvalid) {
+    k_count_valid(Grid G, const float* __restrict__ rec, int64_t B, unsigned long long* __restrict__ tally,
+                  int32_t* __restrict__ nvalid) {
+  __shared__ int s_cnt[Q_THREADS / 32];
   int cnt = 0;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i0 < B; i0 += COUNT_RPT * stride) {
@@ -125,8 +130,18 @@ __global__ void __launch_bounds__(Q_THREADS, COUNT_BLOCKS_PER_SM)
 #pragma unroll
     for (int r = 0; r < COUNT_RPT; ++r) cnt += in[r][0] && in[r][1] ? 1 : 0;
   }
-  int w = gp_warp_sum_i(cnt);
-  if ((threadIdx.x & 31) == 0 && w) atomicAdd(nvalid, w);
+  const int w = gp_warp_sum_i(cnt);
+  if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = w;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long mine = 1ull << 32;
+    for (int k = 0; k < Q_THREADS / 32; ++k) mine += s_cnt[k];
+    const unsigned long long all = atomicAdd(tally, mine) + mine;
+    if ((unsigned)(all >> 32) == gridDim.x) {
+      *nvalid = (int32_t)(all & 0xffffffffull);
+      *tally = 0;
+    }
+  }
 }
 
 // Block reduction of three float sums into partials[block*8 + 0..2] (fp64).
@@ -553,8 +568,11 @@ unsigned q_grid(const gp_ctx* ctx, int64_t B) {
   return gp_blocks(B, Q_THREADS, cap);
 }
 
-unsigned count_grid(const gp_ctx* ctx, int64_t B) {
-  return gp_blocks(B, Q_THREADS * COUNT_RPT, (int64_t)ctx->num_sms * COUNT_BLOCKS_PER_SM);
+// B_v into the band's counter, B > 0.
+void launch_count(gp_band* b, const Grid& G, const float* rec, int64_t B, cudaStream_t s) {
+  const unsigned grid = gp_blocks(B, Q_THREADS * COUNT_RPT, (int64_t)b->ctx->num_sms * COUNT_BLOCKS_PER_SM);
+  k_count_valid<<<grid, Q_THREADS, 0, s>>>(G, rec, B, reinterpret_cast<unsigned long long*>(b->dev_ints + GP_DI_TALLY),
+                                           b->dev_ints + GP_DI_NVALID);
 }
 
 unsigned tv_grid(const gp_ctx* ctx, int64_t n_bricks) {
@@ -595,9 +613,10 @@ extern "C" gp_status gp_step(gp_band* b, const float* rec_dev, int64_t B, const 
   const int32_t* bv = nvalid_dev;
   if (!bv) {
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
-    GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     if (B > 0) {
-      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
+      GP_KERNEL(ctx, "k_count_valid", launch_count(b, G, rec_dev, B, s));
+    } else {
+      GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     }
     bv = cnt;
   }
@@ -721,11 +740,8 @@ extern "C" gp_status gp_band_autotune(gp_band* b, const float* rec_dev, int64_t 
   cudaError_t e = cudaSuccess;
   if (!bv) {
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
-    e = cudaMemsetAsync(cnt, 0, sizeof(int32_t), s);
-    if (e == cudaSuccess) {
-      k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt);
-      e = cudaGetLastError();
-    }
+    launch_count(b, G, rec_dev, B, s);
+    e = cudaGetLastError();
     bv = cnt;
   }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -878,9 +894,10 @@ extern "C" gp_status gp_step_update(gp_band* b, const float* rec_dev, int64_t B,
   const int32_t* bv = nvalid_dev;
   if (!bv) {
     int32_t* cnt = b->dev_ints + GP_DI_NVALID;
-    GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     if (B > 0) {
-      GP_KERNEL(ctx, "k_count_valid", k_count_valid<<<count_grid(ctx, B), Q_THREADS, 0, s>>>(G, rec_dev, B, cnt));
+      GP_KERNEL(ctx, "k_count_valid", launch_count(b, G, rec_dev, B, s));
+    } else {
+      GP_CUDA(ctx, cudaMemsetAsync(cnt, 0, sizeof(int32_t), s));
     }
     bv = cnt;
   }
