@@ -76,10 +76,12 @@ def alg_bytes(name, n, J, Vs, Vt):
         "k_order_emit": 20 * J + 32 * n,
         "k_nn": 36 * n + 16 * J,
         "k_nn_sorted": 36 * n + 16 * J,
+        "k_seed_points": 28 * J,  # a band without normals: points read, seeds written (at set-up)
         "k_count_valid": 24 * n,
         "k_tv": 8 * Vs,
-        # the two-pass L_TV of gp_step: D read and 1/TV written; D and 1/TV
-        # read and the gradient written
+        # the sweep without a gradient, and with the fixed-point sums folded in,
+        # under the names and bytes of the two passes that stored 1/TV between
+        # them (the first now only reads D: 4 bytes a slot)
         "k_tv_inv": 8 * Vs,
         "k_tv_grad": 12 * Vs,
         "k_query": 24 * n + 8 * Vt,
@@ -989,9 +991,8 @@ def run_collection(args, world, rank, local):
                             "alg_bytes": int(by), "gbs": round(by / (avg_ms / 1e3) / 1e9, 1) if by else None}
     fba = fwd_bwd_adam(per_kernel, ("k_m_tv", "k_m_query", "k_m_adam", "k_m_finish"), q_prof / Kp, Vt, peak)
     dom = max(kern.items(), key=lambda kv: kv[1][1])[0]
-    # The search's candidate distances: k_m_nn walks each record's ball as
-    # gp_nn does (same seeds, same walk), so gp_nn_work on every cloud's
-    # records of the last step counts them.
+    # The search's candidate distances: k_m_nn searches as gp_nn does, so
+    # gp_nn_work on every cloud's records of the last step counts them.
     cand, nrec = 0, 0
     for k, band in enumerate(bands):
         rec_k, src_k, _ = gb.gp_multi_buffers(multi, k)

@@ -465,7 +465,7 @@ typedef struct gp_multi gp_multi;
 typedef struct gp_multi_info {
   int32_t n;                    /* clouds                                      */
   uint32_t flags;               /* creation flags                              */
-  int32_t records_per_tile;     /* also the block size of the record kernels   */
+  int32_t records_per_tile;     /* records of a work tile (NN and query)       */
   int32_t blocks_per_sm_nn;     /* persistent blocks per SM, NN stage          */
   int32_t blocks_per_sm_tv;     /* ... L_TV sweep                              */
   int32_t blocks_per_sm_query;  /* ... fused query forward + backward          */
