@@ -13,7 +13,7 @@ from . import binding as gb
 class GridPullLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, values, band, rec, B, weights=(1.0, 1.0, 0.005), flags=0):
-        loss = torch.zeros(8, dtype=torch.float32, device=values.device)
+        loss = torch.empty(8, dtype=torch.float32, device=values.device)
         gb.gp_step(band, rec, int(B), None, loss, weights, d=values.detach().contiguous(),
                    flags=int(flags) | gb.GP_STEP_LOSS_ONLY)
         ctx.band, ctx.B, ctx.weights, ctx.flags = band, int(B), weights, int(flags)
@@ -24,7 +24,7 @@ class GridPullLoss(torch.autograd.Function):
     def backward(ctx, grad_out):
         values, rec = ctx.saved_tensors
         grad = torch.empty_like(values)
-        loss = torch.zeros(8, dtype=torch.float32, device=values.device)
+        loss = torch.empty(8, dtype=torch.float32, device=values.device)
         gb.gp_step(ctx.band, rec, ctx.B, grad, loss, ctx.weights, d=values.detach().contiguous(), flags=ctx.flags)
         return grad * grad_out, None, None, None, None, None
 
