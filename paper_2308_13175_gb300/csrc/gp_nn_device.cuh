@@ -445,7 +445,7 @@ struct NNWarp {
 // Measured (GB300, seeded batches, whole search): with one thread walking its
 // query's rows of cells, 8 of 32 lanes active, 1,116 us for 2,097,152 queries
 // among 10 M points and 206 us for 262,144 among 100,000; with step 2 lane by
-// lane 730 and 210; shared 530 and 104.  It is then bound by the L1 (81% of its
+// lane 730 and 210; shared 503 and 111.  It is then bound by the L1 (81% of its
 // wavefronts: a lane's chunk is a line of its own) and by issue (56%).
 // Sorting a block's queries by radius instead of sharing gave 700 and 190.
 template <bool COUNT>
