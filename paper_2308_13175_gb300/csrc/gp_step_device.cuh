@@ -421,7 +421,8 @@ __device__ __forceinline__ bool query_record(const Grid& G, const float q[3], co
 // The band stores every in-grid axis neighbour of a T vertex, so a value the
 // sums use is always present: absent bricks are staged as zeros.  In bricks at
 // the grid's boundary the vertices just outside take the values of their
-// in-grid neighbours (difference 0), and padding slots get gradient 0.
+// in-grid neighbours (difference 0); padding slots get gradient 0, and their own
+// values go to out().
 constexpr int TV_SWEEP_THREADS = 128;
 constexpr int TV_SWEEP_WARPS = TV_SWEEP_THREADS / 32;
 constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM: 43 KB of shared memory, 102 registers a thread
@@ -717,15 +718,19 @@ __device__ __forceinline__ void tv_sweep(const Src& src, int64_t n, TvShared& sh
       const float ileft = xq ? s.inv[ir + 3] : s.side[0][8 * z + y], iright = xq ? s.side[1][8 * z + y] : s.inv[ir + 4];
       float4 g = tv_grad4(c, left, right, tv_ld4(s.d + r - 8 + 4 * xq), tv_ld4(s.d + r + 8 + 4 * xq), zm, zp, ic, ileft,
                           iright, tv_ld4(s.inv + ir - 8 + 4 * xq), tv_ld4(s.inv + ir + 8 + 4 * xq), izm, izp);
+      float4 own = c;
       if (edge) {
-        const bool row = bk.oy + y <= bk.R && bk.oz + z <= bk.R;
-        const int x = bk.ox + 4 * xq;
-        g.x = row && x <= bk.R ? g.x : 0.f;
-        g.y = row && x + 1 <= bk.R ? g.y : 0.f;
-        g.z = row && x + 2 <= bk.R ? g.z : 0.f;
-        g.w = row && x + 3 <= bk.R ? g.w : 0.f;
+        // Padding slots: gradient 0 and the values the band holds there, not
+        // those tv_close_grid put beside the grid.
+        const int slot = __shfl_sync(0xffffffffu, nbr, 13);  // the brick's own
+        const int in = bk.oy + y <= bk.R && bk.oz + z <= bk.R ? bk.R - (bk.ox + 4 * xq) : -1;  // the last one in the grid
+        if (in < 3) {
+          const float4 held = __ldg(reinterpret_cast<const float4*>(bk.D + (int64_t)slot * 512 + 4 * q));
+          g = make_float4(in >= 0 ? g.x : 0.f, in >= 1 ? g.y : 0.f, in >= 2 ? g.z : 0.f, 0.f);
+          own = make_float4(in >= 0 ? c.x : held.x, in >= 1 ? c.y : held.y, in >= 2 ? c.z : held.z, held.w);
+        }
       }
-      out(i, q, c, g, got);
+      out(i, q, own, g, got);
       zm = c;
       c = zp;
       izm = ic;
