@@ -164,11 +164,28 @@ inline void gp_free(gp_ctx* ctx, void* p) {
   if (p) cudaFreeAsync(p, ctx->stream);
 }
 
-// Memory that any stream may have used: freed after the caller has
-// synchronised the device (the context's stream may be gone by then).
+// Memory that any stream may have used: freed after the caller has made its
+// device current and synchronised it (the context's stream may be gone by then).
 inline void gp_free_idle(void* p) {
   if (p) cudaFreeAsync(p, nullptr);
 }
+
+// Makes `dev` the calling thread's current device for its scope and puts the
+// caller's device back on every return path, so a call never leaves the thread
+// on another device than it found it on.
+struct DeviceScope {
+  int prev = -1;
+  cudaError_t err = cudaSuccess;
+  explicit DeviceScope(int dev) {
+    err = cudaGetDevice(&prev);
+    if (err == cudaSuccess && prev != dev) err = cudaSetDevice(dev);
+    if (err != cudaSuccess) cudaGetLastError();
+  }
+  ~DeviceScope() {
+    int cur = -1;
+    if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
+  }
+};
 
 inline unsigned gp_blocks(int64_t n, int threads, int64_t cap = 1 << 30) {
   int64_t b = (n + threads - 1) / threads;

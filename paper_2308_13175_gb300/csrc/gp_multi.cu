@@ -495,6 +495,7 @@ enum { ST_NN, ST_TV, ST_QUERY, ST_TUNED };
 
 struct gp_multi {
   gp_ctx* ctx = nullptr;
+  int device = 0;
   int n = 0;
   uint64_t seed = 0;
   uint32_t flags = 0;
@@ -520,12 +521,15 @@ namespace {
 
 void multi_free(gp_multi* m) {
   if (!m) return;
+  // A collector may destroy a multi while another device is current.
+  DeviceScope scope(m->device);
   cudaDeviceSynchronize();  // any stream may have worked on the buffers
   for (void* p : {(void*)m->shapes, (void*)m->rec_tiles, (void*)m->pt_tiles, (void*)m->brick_tiles,
                   (void*)m->active_tiles, (void*)m->q, (void*)m->rec, (void*)m->grad, (void*)m->src,
                   (void*)m->perm, (void*)m->inv, (void*)m->eslot, (void*)m->counts, (void*)m->nvalid, (void*)m->err,
                   (void*)m->sums, (void*)m->acc, (void*)m->isums, (void*)m->t, (void*)m->perm_epoch})
     gp_free_idle(p);
+  cudaGetLastError();
   delete m;
 }
 
@@ -658,6 +662,7 @@ extern "C" gp_status gp_multi_create(gp_ctx* ctx, gp_band* const* bands, int32_t
   gp_multi* m = new (std::nothrow) gp_multi();
   if (!m) return gp_fail(ctx, GP_ERR_OOM, "gp_multi_create: host allocation");
   m->ctx = ctx;
+  m->device = ctx->device;
   m->n = n;
   m->seed = seed;
   m->flags = flags;

@@ -270,23 +270,6 @@ __global__ void __launch_bounds__(NA_THREADS) k_na_query(int R, const float* __r
   }
 }
 
-// Makes `dev` the calling thread's current device for the scope of the call
-// and puts the caller's device back on every return path, so the call never
-// leaves the thread on another device than it found it on.
-struct DeviceScope {
-  int prev = -1;
-  cudaError_t err = cudaSuccess;
-  explicit DeviceScope(int dev) {
-    err = cudaGetDevice(&prev);
-    if (err == cudaSuccess && prev != dev) err = cudaSetDevice(dev);
-    if (err != cudaSuccess) cudaGetLastError();
-  }
-  ~DeviceScope() {
-    int cur = -1;
-    if (prev >= 0 && cudaGetDevice(&cur) == cudaSuccess && cur != prev) cudaSetDevice(prev);
-  }
-};
-
 // Device address of the scratch array on the current device (the context's,
 // made current by the caller's DeviceScope); looked up once per device by the
 // first call.

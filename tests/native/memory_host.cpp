@@ -1,0 +1,56 @@
+// Host program for tests/test_device_memory.py: runs the library's calls on the
+// stand-in runtime and prints what it saw, one "name value" a line.
+#include <cuda_runtime_api.h>
+#include <stdio.h>
+#include <string.h>
+
+#include <vector>
+
+#include "fake_cudart.h"
+#include "gridpull.h"
+
+static gp_band* make_band(gp_ctx* ctx, int64_t J) {
+  void* pts = nullptr;
+  cudaMalloc(&pts, 3 * J * sizeof(float));
+  gp_grid_desc d = {16, 1, 1, 4, 0, 0};
+  gp_band* b = nullptr;
+  if (gp_build_band(ctx, (const float*)pts, J, &d, &b)) printf("error %s\n", gp_last_error(ctx));
+  cudaFree(pts);
+  return b;
+}
+
+static gp_multi* make_multi(gp_ctx* ctx, gp_band* b, int64_t B) {
+  gp_multi* m = nullptr;
+  if (gp_multi_create(ctx, &b, 1, &B, &B, 1, GP_SAMPLE_SPATIAL, &m)) printf("error %s\n", gp_last_error(ctx));
+  return m;
+}
+
+static void step(gp_multi* m) {
+  const gp_loss_w w = {1.f, 1.f, 0.005f};
+  const gp_adam hp = {1e-3f, 0.9f, 0.999f, 1e-8f};
+  static float loss[8];
+  if (gp_multi_step(m, &w, &hp, 1.f, 0, loss)) printf("error step\n");
+}
+
+static void report() {
+  int dev = -1;
+  cudaGetDevice(&dev);
+  printf("device %d\nraces %d\nwrong_device %d\n", dev, fake::races, fake::wrong_device);
+}
+
+int main(int argc, char** argv) {
+  const char* what = argc > 1 ? argv[1] : "";
+  const cudaStream_t s1 = (cudaStream_t)0x10;
+  if (!strcmp(what, "other_device")) {
+    // A step of a multi of device 1 is in flight; it is destroyed while device 0 is current.
+    gp_ctx* ctx = nullptr;
+    gp_create(&ctx, 1, s1);
+    gp_band* b = make_band(ctx, 100);
+    gp_multi* m = make_multi(ctx, b, 1000);
+    step(m);
+    cudaSetDevice(0);
+    gp_multi_destroy(m);
+    report();
+  }
+  return 0;
+}

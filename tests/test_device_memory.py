@@ -1,0 +1,40 @@
+"""The library's host code around device memory and launches, run on a stand-in
+for the CUDA runtime (tests/native/fake_cudart.cpp): two devices, kernels that do
+nothing, and a record of which stream still had work in flight when memory was
+freed and of what the memory pools hold.  No GPU is needed."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+NATIVE = os.path.join(ROOT, "tests", "native")
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    nvcc = next((c for c in ("/usr/local/cuda/bin/nvcc", shutil.which("nvcc")) if c and os.path.exists(c)), None)
+    if nvcc is None or shutil.which("g++") is None:
+        pytest.skip("no CUDA toolkit")
+    from paper_2308_13175_gb300 import build
+    build.build()
+    objs = [os.path.join(build.BUILD, s.replace(".cu", ".o")) for s in build.SOURCES]
+    exe = str(tmp_path_factory.mktemp("memory") / "memory_host")
+    include = os.path.join(os.path.dirname(os.path.dirname(nvcc)), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", include, "-I", os.path.join(ROOT, "include"), "-I", NATIVE,
+                    os.path.join(NATIVE, "memory_host.cpp"), os.path.join(NATIVE, "fake_cudart.cpp"), *objs, "-o", exe],
+                   check=True, capture_output=True)
+
+    def call(what):
+        out = subprocess.run([exe, what], check=True, capture_output=True, text=True).stdout
+        assert "error" not in out, out
+        return {k: int(v) for k, v in (line.split() for line in out.splitlines())}
+    return call
+
+
+def test_multi_destroyed_while_another_device_is_current(run):
+    """Its device is waited for before its memory goes, and the caller's device
+    is current again afterwards."""
+    got = run("other_device")
+    assert got == {"device": 0, "races": 0, "wrong_device": 0}
