@@ -534,7 +534,10 @@ void multi_free(gp_multi* m) {
 }
 
 gp_status upload_tiles(gp_ctx* ctx, const std::vector<MTile>& h, MTile** d, int64_t* n) {
-  gp_free(ctx, *d);
+  if (*d) {  // steps on an earlier stream of the context may still read it
+    GP_CUDA(ctx, cudaDeviceSynchronize());
+    gp_free_idle(*d);
+  }
   *d = nullptr;
   *n = (int64_t)h.size();
   gp_status st = gp_alloc(ctx, d, h.size(), "multi tiles");

@@ -40,7 +40,7 @@ static void report() {
 
 int main(int argc, char** argv) {
   const char* what = argc > 1 ? argv[1] : "";
-  const cudaStream_t s1 = (cudaStream_t)0x10;
+  const cudaStream_t s1 = (cudaStream_t)0x10, s2 = (cudaStream_t)0x20;
   if (!strcmp(what, "other_device")) {
     // A step of a multi of device 1 is in flight; it is destroyed while device 0 is current.
     gp_ctx* ctx = nullptr;
@@ -50,6 +50,16 @@ int main(int argc, char** argv) {
     step(m);
     cudaSetDevice(0);
     gp_multi_destroy(m);
+    report();
+  } else if (!strcmp(what, "tiles")) {
+    // A step is in flight on one stream when the multi is tuned on another.
+    gp_ctx* ctx = nullptr;
+    gp_create(&ctx, 0, s1);
+    gp_multi* m = make_multi(ctx, make_band(ctx, 100), 1000);
+    step(m);
+    gp_set_stream(ctx, s2);
+    const gp_loss_w w = {1.f, 1.f, 0.005f};
+    if (gp_multi_autotune(m, &w)) printf("error autotune\n");
     report();
   }
   return 0;

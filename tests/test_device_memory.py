@@ -38,3 +38,8 @@ def test_multi_destroyed_while_another_device_is_current(run):
     is current again afterwards."""
     got = run("other_device")
     assert got == {"device": 0, "races": 0, "wrong_device": 0}
+
+
+def test_tuning_on_another_stream_than_the_last_step(run):
+    """The tile list that a step still reads is not given back under it."""
+    assert run("tiles") == {"device": 0, "races": 0, "wrong_device": 0}
