@@ -330,6 +330,7 @@ void band_free(gp_band* b) {
   gp_free_idle(b->emit_pts);
   gp_free_idle(b->partials);
   gp_free_idle(b->dev_ints);
+  gp_free_idle_done();
   delete b;
 }
 

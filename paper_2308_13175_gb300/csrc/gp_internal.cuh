@@ -170,6 +170,11 @@ inline void gp_free_idle(void* p) {
   if (p) cudaFreeAsync(p, nullptr);
 }
 
+// After the last gp_free_idle of an object: a pool gives back what exceeds the
+// bytes it keeps, and a trim finds the rest, only once the host has seen the
+// frees complete.
+inline void gp_free_idle_done() { cudaStreamSynchronize(nullptr); }
+
 // Makes `dev` the calling thread's current device for its scope and puts the
 // caller's device back on every return path, so a call never leaves the thread
 // on another device than it found it on.

@@ -529,6 +529,7 @@ void multi_free(gp_multi* m) {
                   (void*)m->perm, (void*)m->inv, (void*)m->eslot, (void*)m->counts, (void*)m->nvalid, (void*)m->err,
                   (void*)m->sums, (void*)m->acc, (void*)m->isums, (void*)m->t, (void*)m->perm_epoch})
     gp_free_idle(p);
+  gp_free_idle_done();
   cudaGetLastError();
   delete m;
 }

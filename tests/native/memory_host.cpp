@@ -61,6 +61,24 @@ int main(int argc, char** argv) {
     const gp_loss_w w = {1.f, 1.f, 0.005f};
     if (gp_multi_autotune(m, &w)) printf("error autotune\n");
     report();
+  } else if (!strcmp(what, "given_back")) {
+    // A band beyond what the pool keeps, then the last context of the device.
+    gp_ctx *ctx = nullptr, *other = nullptr;
+    gp_create(&ctx, 0, s1);
+    gp_create(&other, 0, s2);
+    const size_t keep = fake::lowest_threshold();
+    gp_band* b = make_band(ctx, (int64_t)keep / 12 + 1);
+    printf("above_while_alive %d\n", fake::reserved() > keep);
+    gp_band_destroy(b);
+    printf("above_after_the_band %d\n", fake::reserved() > keep);
+    gp_destroy(other);
+    b = make_band(ctx, 100);
+    gp_multi* m = make_multi(ctx, b, 1000);
+    step(m);
+    gp_multi_destroy(m);
+    gp_destroy(ctx);
+    gp_band_destroy(b);
+    printf("after_the_last_context %d\n", (int)fake::reserved());
   }
   return 0;
 }

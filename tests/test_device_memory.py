@@ -43,3 +43,9 @@ def test_multi_destroyed_while_another_device_is_current(run):
 def test_tuning_on_another_stream_than_the_last_step(run):
     """The tile list that a step still reads is not given back under it."""
     assert run("tiles") == {"device": 0, "races": 0, "wrong_device": 0}
+
+
+def test_pool_gives_memory_back(run):
+    """What a destroyed band leaves beyond the bytes that the pool keeps goes
+    back at once, and everything goes with the last context of the device."""
+    assert run("given_back") == {"above_while_alive": 1, "above_after_the_band": 0, "after_the_last_context": 0}
