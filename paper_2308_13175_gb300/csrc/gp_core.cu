@@ -44,7 +44,11 @@ cudaError_t gp_pool_acquire(int device, cudaMemPool_t* pool) {
     }
     uint64_t keep = GP_POOL_KEEP;
     e = cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {  // not left for the next context without its threshold
+      cudaMemPoolDestroy(d.pool);
+      d.pool = nullptr;
+      return e;
+    }
   }
   d.users += 1;
   *pool = d.pool;

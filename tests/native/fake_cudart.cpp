@@ -81,7 +81,7 @@ void forget(void* p, const Stream& order) {
 }  // namespace
 
 namespace fake {
-int races = 0, wrong_device = 0, fail_set_attribute = 0, pools_made = 0;
+int races = 0, wrong_device = 0, fail_set_attribute = 0;
 std::map<std::string, unsigned> last_grid;
 
 size_t reserved() {
@@ -196,7 +196,6 @@ cudaError_t cudaGetSymbolAddress(void** p, const void*) {
 cudaError_t cudaMemPoolCreate(cudaMemPool_t* pool, const cudaMemPoolProps* props) {
   *pool = (cudaMemPool_t)malloc(1);
   g_pools[*pool].device = props->location.id;
-  ++fake::pools_made;
   return cudaSuccess;
 }
 cudaError_t cudaMemPoolDestroy(cudaMemPool_t pool) {

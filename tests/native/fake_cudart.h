@@ -11,7 +11,6 @@ namespace fake {
 extern int races;               // frees of memory while another stream of its device had work in flight
 extern int wrong_device;        // frees ordered after a stream of another device than the memory's
 extern int fail_set_attribute;  // calls of cudaMemPoolSetAttribute still to fail
-extern int pools_made;
 extern std::map<std::string, unsigned> last_grid;  // blocks of each kernel's last launch
 size_t reserved();            // bytes the pools hold: in use, freed and kept, freed and not yet seen to be
 uint64_t lowest_threshold();  // of the pools there are

@@ -79,6 +79,13 @@ int main(int argc, char** argv) {
     gp_destroy(ctx);
     gp_band_destroy(b);
     printf("after_the_last_context %d\n", (int)fake::reserved());
+  } else if (!strcmp(what, "no_threshold")) {
+    // The pool's threshold cannot be set at the first context, then it can.
+    gp_ctx* ctx = nullptr;
+    fake::fail_set_attribute = 1;
+    const gp_status first = gp_create(&ctx, 0, s1);
+    const gp_status second = gp_create(&ctx, 0, s1);
+    printf("first %d\nsecond %d\nkeeps %d\n", first, second, fake::lowest_threshold() > 0);
   }
   return 0;
 }

@@ -49,3 +49,9 @@ def test_pool_gives_memory_back(run):
     """What a destroyed band leaves beyond the bytes that the pool keeps goes
     back at once, and everything goes with the last context of the device."""
     assert run("given_back") == {"above_while_alive": 1, "above_after_the_band": 0, "after_the_last_context": 0}
+
+
+def test_pool_without_its_threshold_is_not_kept(run):
+    """A context whose pool cannot be set up fails; the next one gets a pool
+    that is."""
+    assert run("no_threshold") == {"first": 3, "second": 0, "keeps": 1}  # GP_ERR_CUDA, GP_OK
