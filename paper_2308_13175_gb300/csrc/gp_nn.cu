@@ -93,15 +93,16 @@ __device__ __forceinline__ void least_spread(const float S[6], float n[3]) {
   for (int k = 0; k < 3; ++k) n[k] = inv > 0.f ? n[k] * inv : 0.f;
 }
 
-// A block's 64 cell counts, in shared memory, from its points [first, last).
-__device__ __forceinline__ void block_histogram(const NNGrid& g, const float4* __restrict__ by_block, int first,
-                                                int last, int* cell) {
+// A block's 64 cell counts, in shared memory, from its points [first, last)
+// (unsigned: the last of J < 2^31 points plus a warp's stride).
+__device__ __forceinline__ void block_histogram(const NNGrid& g, const float4* __restrict__ by_block, uint32_t first,
+                                                uint32_t last, unsigned* cell) {
   const int lane = threadIdx.x & 31;
   __syncwarp();
   cell[lane] = 0;
   cell[lane + 32] = 0;
   __syncwarp();
-  for (int p = first + lane; p < last; p += 32) atomicAdd(cell + nn_local_cell(by_block[p], g), 1);
+  for (uint32_t p = first + lane; p < last; p += 32) atomicAdd(cell + nn_local_cell(by_block[p], g), 1u);
   __syncwarp();
 }
 
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_count(NNGrid g, c
                                                                      const float4* __restrict__ by_block, int64_t nblk,
                                                                      int32_t* __restrict__ table,
                                                                      int32_t* __restrict__ totals) {
-  __shared__ int s_cell[NN_BUILD_WARPS][64];
+  __shared__ unsigned s_cell[NN_BUILD_WARPS][64];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   for (int64_t b0 = ((int64_t)blockIdx.x * NN_BUILD_WARPS + w) * NN_BUILD_RUN; b0 < nblk;
        b0 += (int64_t)gridDim.x * NN_BUILD_WARPS * NN_BUILD_RUN) {
@@ -133,9 +134,9 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_count(NNGrid g, c
     for (unsigned left = some; left; left &= left - 1u) {
       const int k = __ffs(left) - 1;
       block_histogram(g, by_block, __shfl_sync(0xffffffffu, f, k), __shfl_sync(0xffffffffu, l, k), s_cell[w]);
-      const int n0 = s_cell[w][lane], n1 = s_cell[w][lane + 32];
+      const unsigned n0 = s_cell[w][lane], n1 = s_cell[w][lane + 32];
       occ += (n0 > 0) + (n1 > 0) + (lane == 0);
-      chunks += ((n0 + 3) >> 2) + ((n1 + 3) >> 2);
+      chunks += (int)((n0 + 3u) >> 2) + (int)((n1 + 3u) >> 2);
     }
     occ = gp_warp_sum_i(occ);
     chunks = gp_warp_sum_i(chunks);
@@ -154,16 +155,16 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
     NNGrid g, const int32_t* __restrict__ start, const float4* __restrict__ by_block, int64_t nblk,
     const int32_t* __restrict__ table, int32_t* __restrict__ totals, float* __restrict__ pts, int32_t* __restrict__ occ,
     float4* __restrict__ blk, unsigned long long* __restrict__ sup) {
-  __shared__ int s_cell[NN_BUILD_WARPS][64];
+  __shared__ unsigned s_cell[NN_BUILD_WARPS][64];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  int* cell = s_cell[w];
+  unsigned* cell = s_cell[w];
   for (int64_t b0 = ((int64_t)blockIdx.x * NN_BUILD_WARPS + w) * NN_BUILD_RUN; b0 < nblk;
        b0 += (int64_t)gridDim.x * NN_BUILD_WARPS * NN_BUILD_RUN) {
     const int64_t mine = lane < NN_BUILD_RUN ? b0 + lane : nblk;
     const int fl = mine < nblk ? start[mine] : 0, ll = mine < nblk ? start[mine + 1] : 0;
     for (unsigned left = __ballot_sync(0xffffffffu, ll > fl); left; left &= left - 1u) {
       const int kb = __ffs(left) - 1;
-      const int first = __shfl_sync(0xffffffffu, fl, kb), last = __shfl_sync(0xffffffffu, ll, kb);
+      const uint32_t first = __shfl_sync(0xffffffffu, fl, kb), last = __shfl_sync(0xffffffffu, ll, kb);
       const int64_t b = b0 + kb;
       const int bi = table[b];
       const int bx = (int)(b % g.nbk), by = (int)((b / g.nbk) % g.nbk), bz = (int)(b / ((int64_t)g.nbk * g.nbk));
@@ -171,8 +172,8 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
       block_histogram(g, by_block, first, last, cell);
       // Exclusive scans of the cells' chunks and occupancy, two consecutive
       // cells per lane, and the block's share of the arrays.
-      const int n0 = cell[2 * lane], n1 = cell[2 * lane + 1];
-      const int h0 = (n0 + 3) >> 2, h1 = (n1 + 3) >> 2;
+      const unsigned n0 = cell[2 * lane], n1 = cell[2 * lane + 1];
+      const int h0 = (int)((n0 + 3u) >> 2), h1 = (int)((n1 + 3u) >> 2);
       int incl = h0 + h1;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -193,17 +194,17 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
       if (n1) occ[o0 + k0 + (n0 > 0)] = at1;
       if (lane == 31) occ[o0 + nocc] = base + incl;
       __syncwarp();
-      cell[2 * lane] = 4 * at0;
-      cell[2 * lane + 1] = 4 * at1;
+      cell[2 * lane] = 4u * (unsigned)(at0 - base);  // the cell's next place (nn_place)
+      cell[2 * lane + 1] = 4u * (unsigned)(at1 - base);
       __syncwarp();
       float m[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
       bool inside = true;
-      for (int p = first + lane; p < last; p += 32) {
+      for (uint32_t p = first + lane; p < last; p += 32) {
         const float4 P = by_block[p];
-        const int at = atomicAdd(cell + nn_local_cell(P, g), 1);
+        const unsigned at = atomicAdd(cell + nn_local_cell(P, g), 1u);
         const float v[4] = {P.x, P.y, P.z, P.w};
 #pragma unroll
-        for (int k = 0; k < 4; ++k) pts[4 * nn_part(at >> 2, k) + (at & 3)] = v[k];
+        for (int k = 0; k < 4; ++k) pts[nn_place(base, at, k)] = v[k];
         inside = inside && fabsf(P.x) <= 1.01f && fabsf(P.y) <= 1.01f && fabsf(P.z) <= 1.01f;
         const float x = P.x - c0, y = P.y - c1, z = P.z - c2;
         m[0] += x;
@@ -220,11 +221,10 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
       // The places left in each cell's last chunk.
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        const int end = 4 * (k ? at1 + h1 : at0 + h0);
-        for (int at = cell[2 * lane + k]; at < end; ++at) {
+        const unsigned end = 4u * (unsigned)((k ? at1 + h1 : at0 + h0) - base);
+        for (unsigned at = cell[2 * lane + k]; at < end; ++at) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            pts[4 * nn_part(at >> 2, j) + (at & 3)] = j < 3 ? INFINITY : __int_as_float(-1);
+          for (int j = 0; j < 4; ++j) pts[nn_place(base, at, j)] = j < 3 ? INFINITY : __int_as_float(-1);
         }
       }
       inside = __all_sync(0xffffffffu, inside);
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(32 * NN_BUILD_WARPS) k_block_build(
         least_spread(S, n);
       }
       float lo = INFINITY, hi = -INFINITY;
-      for (int p = first + lane; p < last; p += 32) {
+      for (uint32_t p = first + lane; p < last; p += 32) {
         const float4 P = by_block[p];
         const float v = n[0] * P.x + n[1] * P.y + n[2] * P.z;
         lo = fminf(lo, v);

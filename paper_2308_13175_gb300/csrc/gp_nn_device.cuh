@@ -119,6 +119,14 @@ __host__ __device__ __forceinline__ int64_t nn_part(int64_t c, int k) {
   return 4 * c + ((k + (int)(c >> 1)) & 3);
 }
 
+// Where part k of a point of a block lies, in floats: `at` is its place counted
+// from the block's first chunk (4 chunk + place in the chunk).  A cell's last
+// chunk is filled up, so places counted from the start of the cloud pass 2^31
+// for clouds that gp_build_band takes; a block's own stay below 2^32.
+__host__ __device__ __forceinline__ int64_t nn_place(int64_t first_chunk, uint32_t at, int k) {
+  return 4 * nn_part(first_chunk + (at >> 2), k) + (at & 3u);
+}
+
 // Part k of the point at place i (4 chunk + place in the chunk).
 __device__ __forceinline__ float nn_value(const float4* __restrict__ pts, int64_t i, int k) {
   return __ldg(reinterpret_cast<const float*>(pts + nn_part(i >> 2, k)) + (i & 3));
