@@ -29,7 +29,11 @@
  *   - Memory.  Pointers named *_dev are device pointers on the context's device
  *     owned by the caller; the library never frees them and never keeps them
  *     after the call returns.  The library owns the band (brick table, D, Adam
- *     moments, point cell list, scratch) and frees it in gp_band_destroy.
+ *     moments, point cell list, scratch) and frees it in gp_band_destroy.  The
+ *     pointers of gp_band_values and gp_multi_buffers lie in memory of
+ *     cudaMalloc; everything else comes from a stream-ordered pool.  Up to 320
+ *     MB of what was freed stays with the library until the last context of the
+ *     device is destroyed.
  *   - Streams.  Every call is asynchronous on the context's stream, except
  *     gp_build_band and the gp_band_* queries that return host values, which
  *     synchronise that stream.  gp_sample, gp_nn, gp_step and gp_update never

@@ -308,11 +308,8 @@ void band_free(gp_band* b) {
   gp_free_idle(b->brick_nbr);
   gp_free_idle(b->masks);
   gp_free_idle(b->active);
-  gp_free_idle(b->D);
-  gp_free_idle(b->m);
-  gp_free_idle(b->v);
+  gp_shown_give(b->ctx->device, &b->shown);
   gp_free_idle(b->acc);
-  gp_free_idle(b->D_alt);
   gp_free_idle(b->qgrad);
   gp_free_idle(b->pts);
   gp_free_idle(b->pts_sorted);
@@ -330,7 +327,7 @@ void band_free(gp_band* b) {
   gp_free_idle(b->emit_pts);
   gp_free_idle(b->partials);
   gp_free_idle(b->dev_ints);
-  gp_free_idle_done();
+  gp_free_idle_done(b->ctx->device);
   delete b;
 }
 
@@ -484,21 +481,20 @@ extern "C" gp_status gp_build_band(gp_ctx* ctx, const float* pts_dev, int64_t J,
   b->G = desc->nn_grid;
   gp_status st = build_band_sets(b, pts_dev);
   int64_t V = b->V_stored();
-  if (!st) st = gp_alloc(ctx, &b->D, V, "values");
-  if (!st) st = gp_alloc(ctx, &b->m, V, "adam m");
-  if (!st) st = gp_alloc(ctx, &b->v, V, "adam v");
+  if (!st) st = gp_alloc_shown(ctx, &b->shown, &b->D, 4 * (size_t)V, "values and Adam moments");
+  if (!st) {
+    b->D_alt = b->D + V;
+    b->m = b->D + 2 * V;
+    b->v = b->D + 3 * V;
+  }
   if (!st && (b->flags & GP_BAND_DETERMINISTIC)) st = gp_alloc(ctx, &b->acc, 2 * V, "fixed-point accumulator");
-  if (!st) st = gp_alloc(ctx, &b->D_alt, V, "second value buffer");
   if (!st) st = gp_alloc(ctx, &b->qgrad, V, "query gradient");
   if (!st) st = gp_alloc(ctx, &b->partials, (size_t)GP_MAX_PARTIAL_BLOCKS * 8, "partials");
   if (!st) st = gp_alloc(ctx, &b->dev_ints, GP_DI_COUNT, "device ints");
   if (!st) {
     cudaStream_t s = ctx->stream;
-    cudaError_t e = cudaMemsetAsync(b->D, 0, V * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->m, 0, V * sizeof(float), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->v, 0, V * sizeof(float), s);
+    cudaError_t e = cudaMemsetAsync(b->D, 0, 4 * V * sizeof(float), s);
     if (e == cudaSuccess && b->acc) e = cudaMemsetAsync(b->acc, 0, 2 * V * sizeof(unsigned long long), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->D_alt, 0, V * sizeof(float), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->qgrad, 0, V * sizeof(float), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->dev_ints, 0, GP_DI_COUNT * sizeof(int32_t), s);
     if (e != cudaSuccess) st = gp_cuda_fail(ctx, e, "gp_build_band: memset");

@@ -3,6 +3,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <utility>
 
 #include "gp_internal.cuh"
 
@@ -21,11 +22,24 @@ namespace {
 struct DevicePool {
   cudaMemPool_t pool = nullptr;
   int64_t users = 0;
+  gp_shown idle[GP_SHOWN_BLOCKS];  // blocks given back
+  size_t idle_bytes = 0;
 };
 std::mutex g_pool_mutex;
 std::map<int, DevicePool>& device_pools() {
   static std::map<int, DevicePool>* pools = new std::map<int, DevicePool>();  // outlives every context
   return *pools;
+}
+void drop_idle(DevicePool& d) {
+  for (gp_shown& b : d.idle) {
+    if (b.p) cudaFree(b.p);
+    b = gp_shown{};
+  }
+  d.idle_bytes = 0;
+}
+void empty_pool(DevicePool& d) {
+  drop_idle(d);
+  if (d.pool) cudaMemPoolTrimTo(d.pool, 0);
 }
 }  // namespace
 
@@ -59,7 +73,55 @@ void gp_pool_release(int device) {
   std::lock_guard<std::mutex> lock(g_pool_mutex);
   DevicePool& d = device_pools()[device];
   if (d.users > 0) d.users -= 1;
-  if (d.users == 0 && d.pool) cudaMemPoolTrimTo(d.pool, 0);
+  if (d.users == 0) empty_pool(d);
+}
+
+cudaError_t gp_shown_take(int device, size_t bytes, gp_shown* block) {
+  *block = gp_shown{};
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = device_pools()[device];
+  gp_shown* best = nullptr;
+  for (gp_shown& b : d.idle)
+    if (b.p && b.bytes >= bytes && b.bytes <= 2 * bytes && (!best || b.bytes < best->bytes)) best = &b;
+  if (best) {
+    std::swap(*block, *best);
+    d.idle_bytes -= block->bytes;
+    return cudaSuccess;
+  }
+  DeviceScope scope(device);
+  if (scope.err != cudaSuccess) return scope.err;
+  void* p = nullptr;
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaErrorMemoryAllocation && d.idle_bytes > 0) {
+    cudaGetLastError();
+    drop_idle(d);
+    e = cudaMalloc(&p, bytes);
+  }
+  if (e == cudaSuccess) *block = gp_shown{p, bytes};
+  return e;
+}
+
+void gp_shown_give(int device, gp_shown* block) {
+  const gp_shown b = *block;
+  *block = gp_shown{};
+  if (!b.p) return;
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = device_pools()[device];
+  if (d.users > 0 && d.idle_bytes + b.bytes <= GP_SHOWN_KEEP)
+    for (gp_shown& slot : d.idle)
+      if (!slot.p) {
+        slot = b;
+        d.idle_bytes += b.bytes;
+        return;
+      }
+  cudaFree(b.p);
+}
+
+void gp_free_idle_done(int device) {
+  cudaStreamSynchronize(nullptr);
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  DevicePool& d = device_pools()[device];
+  if (d.users == 0) empty_pool(d);
 }
 
 extern "C" gp_status gp_create(gp_ctx** out, int device, void* stream) {

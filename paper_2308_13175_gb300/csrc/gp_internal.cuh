@@ -45,6 +45,28 @@ constexpr uint64_t GP_POOL_KEEP = uint64_t(256) << 20;
 cudaError_t gp_pool_acquire(int device, cudaMemPool_t* pool);
 void gp_pool_release(int device);
 
+// Memory whose address callers receive (gp_band_values, gp_multi_buffers) is
+// cudaMalloc's: a pool's is not opened to other devices by
+// cudaDeviceEnablePeerAccess, not copied between devices by cudaMemcpyAsync and
+// has no cudaIpcMemHandle.  A malloc and a free of 10 MB take 89 us and more
+// beside a build (a band of 100,000 points 1,123 -> 1,312 us), so up to
+// GP_SHOWN_KEEP bytes of blocks given back stay with the device, as the pool's
+// memory does, for requests of at least half their size (the same build:
+// 1,104 us).  A block is given back by gp_shown_give only when no stream uses it.
+constexpr size_t GP_SHOWN_KEEP = size_t(64) << 20;
+constexpr int GP_SHOWN_BLOCKS = 32;  // blocks kept at most
+struct gp_shown {
+  void* p = nullptr;
+  size_t bytes = 0;
+};
+cudaError_t gp_shown_take(int device, size_t bytes, gp_shown* block);
+void gp_shown_give(int device, gp_shown* block);
+
+// After the last gp_free_idle of an object: a pool gives back what exceeds the
+// bytes it keeps, and a trim finds the rest, only once the host has seen the
+// frees complete.  Without a context on the device everything goes.
+void gp_free_idle_done(int device);
+
 // Release a context's memory (called when no band refers to it any more).
 void gp_ctx_release(gp_ctx* ctx);
 
@@ -83,6 +105,7 @@ struct gp_band {
   int32_t* brick_nbr = nullptr;    // n_bricks x 27: slots of the 3x3x3 bricks around each (x fastest, -1 absent)
   uint32_t* masks = nullptr;       // n_bricks x 48 words: [T 16][trainable 16][pull 16]
   int32_t* active = nullptr;       // slots of bricks with a trainable vertex
+  gp_shown shown;                  // the memory of D, D_alt, m and v
   float* D = nullptr;              // values, V_stored
   float* m = nullptr;              // Adam first moment
   float* v = nullptr;              // Adam second moment
@@ -159,6 +182,19 @@ gp_status gp_alloc(gp_ctx* ctx, T** p, size_t count, const char* what) {
   return GP_OK;
 }
 
+// Device memory whose address callers receive (gp_shown_take).
+template <typename T>
+gp_status gp_alloc_shown(gp_ctx* ctx, gp_shown* block, T** p, size_t count, const char* what) {
+  const cudaError_t e = gp_shown_take(ctx->device, (count ? count : 1) * sizeof(T), block);
+  *p = (T*)block->p;
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return gp_fail(ctx, e == cudaErrorMemoryAllocation ? GP_ERR_OOM : GP_ERR_CUDA,
+                   std::string("allocation failed for ") + what + ": " + cudaGetErrorString(e));
+  }
+  return GP_OK;
+}
+
 // Scratch of a call on the context's stream: freed in stream order.
 inline void gp_free(gp_ctx* ctx, void* p) {
   if (p) cudaFreeAsync(p, ctx->stream);
@@ -169,11 +205,6 @@ inline void gp_free(gp_ctx* ctx, void* p) {
 inline void gp_free_idle(void* p) {
   if (p) cudaFreeAsync(p, nullptr);
 }
-
-// After the last gp_free_idle of an object: a pool gives back what exceeds the
-// bytes it keeps, and a trim finds the rest, only once the host has seen the
-// frees complete.
-inline void gp_free_idle_done() { cudaStreamSynchronize(nullptr); }
 
 // Makes `dev` the calling thread's current device for its scope and puts the
 // caller's device back on every return path, so a call never leaves the thread

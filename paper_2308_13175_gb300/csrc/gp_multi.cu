@@ -507,6 +507,7 @@ struct gp_multi {
   MShape* shapes = nullptr;
   MTile *rec_tiles = nullptr, *pt_tiles = nullptr, *brick_tiles = nullptr, *active_tiles = nullptr;
   int64_t n_rec_tiles = 0, n_pt_tiles = 0, n_brick_tiles = 0, n_active_tiles = 0;
+  gp_shown shown[3];  // the memory of grad, src and rec
   float *q = nullptr, *rec = nullptr, *grad = nullptr;
   int32_t *src = nullptr, *perm = nullptr, *inv = nullptr, *eslot = nullptr, *counts = nullptr, *nvalid = nullptr,
           *err = nullptr;
@@ -525,11 +526,11 @@ void multi_free(gp_multi* m) {
   DeviceScope scope(m->device);
   cudaDeviceSynchronize();  // any stream may have worked on the buffers
   for (void* p : {(void*)m->shapes, (void*)m->rec_tiles, (void*)m->pt_tiles, (void*)m->brick_tiles,
-                  (void*)m->active_tiles, (void*)m->q, (void*)m->rec, (void*)m->grad, (void*)m->src,
-                  (void*)m->perm, (void*)m->inv, (void*)m->eslot, (void*)m->counts, (void*)m->nvalid, (void*)m->err,
+                  (void*)m->active_tiles, (void*)m->q, (void*)m->perm, (void*)m->inv, (void*)m->eslot, (void*)m->counts, (void*)m->nvalid, (void*)m->err,
                   (void*)m->sums, (void*)m->acc, (void*)m->isums, (void*)m->t, (void*)m->perm_epoch})
     gp_free_idle(p);
-  gp_free_idle_done();
+  for (gp_shown& s : m->shown) gp_shown_give(m->device, &s);
+  gp_free_idle_done(m->device);
   cudaGetLastError();
   delete m;
 }
@@ -706,7 +707,7 @@ extern "C" gp_status gp_multi_create(gp_ctx* ctx, gp_band* const* bands, int32_t
     return gp_fail(ctx, GP_ERR_ARG, "gp_multi_create: sum of the batch sizes must stay below 2^31");
   }
   gp_status st = GP_OK;
-  if (!st) st = gp_alloc(ctx, &m->grad, m->V_total, "multi gradient");
+  if (!st) st = gp_alloc_shown(ctx, &m->shown[0], &m->grad, m->V_total, "multi gradient");
   if (!st && (flags & GP_MULTI_DETERMINISTIC)) st = gp_alloc(ctx, &m->acc, 2 * m->V_total, "multi fixed-point sums");
   if (!st && (flags & GP_MULTI_DETERMINISTIC)) st = gp_alloc(ctx, &m->isums, 4 * (size_t)n, "multi integer sums");
   if (!st) st = gp_alloc(ctx, &m->perm, m->J_total, "multi permutation");
@@ -714,8 +715,8 @@ extern "C" gp_status gp_multi_create(gp_ctx* ctx, gp_band* const* bands, int32_t
   if (!st) st = gp_alloc(ctx, &m->eslot, m->J_total, "multi emission slots");
   if (!st) st = gp_alloc(ctx, &m->shapes, (size_t)n, "multi shapes");
   if (!st) st = gp_alloc(ctx, &m->q, 3 * m->total_B, "multi queries");
-  if (!st) st = gp_alloc(ctx, &m->src, m->total_B, "multi sources");
-  if (!st) st = gp_alloc(ctx, &m->rec, 6 * m->total_B, "multi records");
+  if (!st) st = gp_alloc_shown(ctx, &m->shown[1], &m->src, m->total_B, "multi sources");
+  if (!st) st = gp_alloc_shown(ctx, &m->shown[2], &m->rec, 6 * m->total_B, "multi records");
   if (!st) st = gp_alloc(ctx, &m->counts, pt.size(), "multi order counts");
   if (!st) st = gp_alloc(ctx, &m->nvalid, (size_t)n, "multi counts");
   if (!st) st = gp_alloc(ctx, &m->sums, 4 * (size_t)n, "multi sums");

@@ -97,6 +97,7 @@ uint64_t lowest_threshold() {
   for (auto& p : g_pools) t = p.second.threshold < t ? p.second.threshold : t;
   return t;
 }
+int blocks() { return (int)g_blocks.size(); }
 bool from_pool(const void* p) {
   for (auto& b : g_blocks) {
     const char* at = (const char*)b.first;

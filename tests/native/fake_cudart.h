@@ -15,4 +15,5 @@ extern std::map<std::string, unsigned> last_grid;  // blocks of each kernel's la
 size_t reserved();            // bytes the pools hold: in use, freed and kept, freed and not yet seen to be
 uint64_t lowest_threshold();  // of the pools there are
 bool from_pool(const void* p);
+int blocks();                 // allocations there are
 }  // namespace fake

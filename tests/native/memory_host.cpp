@@ -86,6 +86,29 @@ int main(int argc, char** argv) {
     const gp_status first = gp_create(&ctx, 0, s1);
     const gp_status second = gp_create(&ctx, 0, s1);
     printf("first %d\nsecond %d\nkeeps %d\n", first, second, fake::lowest_threshold() > 0);
+  } else if (!strcmp(what, "shown")) {
+    // Where the pointers that callers receive lie.
+    gp_ctx* ctx = nullptr;
+    gp_create(&ctx, 0, s1);
+    gp_band* b = make_band(ctx, 100);
+    gp_multi* m = make_multi(ctx, b, 1000);
+    float *d = nullptr, *am = nullptr, *av = nullptr, *rec = nullptr, *grad = nullptr;
+    int32_t* src = nullptr;
+    gp_band_values(b, &d, &am, &av);
+    gp_multi_buffers(m, 0, &rec, &src, &grad);
+    printf("values %d\nmoments %d\n", fake::from_pool(d), fake::from_pool(am) + fake::from_pool(av));
+    printf("multi %d\n", fake::from_pool(rec) + fake::from_pool(src) + fake::from_pool(grad));
+    gp_multi_destroy(m);
+    gp_band_destroy(b);
+    b = make_band(ctx, 100);
+    float* again = nullptr;
+    gp_band_values(b, &again, nullptr, nullptr);
+    printf("kept %d\n", again == d || again == grad);
+    m = make_multi(ctx, b, 1000);
+    gp_band_destroy(b);
+    gp_destroy(ctx);
+    gp_multi_destroy(m);  // last, as a collector may have it
+    printf("left %d\n", (int)fake::reserved() + fake::blocks());
   }
   return 0;
 }

@@ -55,3 +55,10 @@ def test_pool_without_its_threshold_is_not_kept(run):
     """A context whose pool cannot be set up fails; the next one gets a pool
     that is."""
     assert run("no_threshold") == {"first": 3, "second": 0, "keeps": 1}  # GP_ERR_CUDA, GP_OK
+
+
+def test_pointers_handed_out_are_ordinary_allocations(run):
+    """Callers may open them to other devices and processes, which a pool's
+    memory is not.  A block given back serves the next band; none is left after
+    the last context, nor after an object that outlived it."""
+    assert run("shown") == {"values": 0, "moments": 0, "multi": 0, "kept": 1, "left": 0}

@@ -43,3 +43,28 @@ def test_memory_goes_back_with_the_band_and_the_context():
     assert built > 2 * KEPT               # points, seeds and chunks: at least 12 + 16 + 16 bytes a point
     assert closed <= KEPT + SLACK, f"{closed >> 20} MiB still held after the band"
     assert gone <= SLACK, f"{gone >> 20} MiB still held after the last context"
+
+
+def test_pointers_handed_out_have_an_ipc_handle():
+    """The values, both value buffers in turn, the moments and a multi's buffers
+    can be opened by another process (the driver's own word for the pointer)."""
+    if not have_gpu():
+        pytest.skip("no CUDA device")
+    build_lib()
+    import ctypes
+    import torch
+    from paper_2308_13175_gb300 import binding as gb
+    cuda = ctypes.CDLL("libcuda.so.1")
+    band = gb.gp_build_band(gb.gp_create(0), torch.rand(500, 3, device="cuda"), 16, 1, 1, 8)
+    multi = gb.gp_multi_create(band.ctx, [band], [1000], [500])
+    shown = list(gb.gp_multi_buffers(multi, 0)) + list(gb.gp_band_values(band))
+    rec = torch.zeros(6, device="cuda")
+    gb.gp_step_update(band, rec, 1, torch.zeros(8, device="cuda"), 0.0, 1)
+    shown.append(gb.gp_band_values(band)[0])
+    assert shown[-1].data_ptr() != shown[3].data_ptr()
+    for t in shown:
+        capable = ctypes.c_int(-1)
+        attribute = 10  # CU_POINTER_ATTRIBUTE_IS_LEGACY_CUDA_IPC_CAPABLE
+        assert cuda.cuPointerGetAttribute(ctypes.byref(capable), attribute, ctypes.c_uint64(t.data_ptr())) == 0
+        assert capable.value == 1
+    multi.close()
