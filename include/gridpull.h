@@ -470,7 +470,8 @@ typedef struct gp_multi_info {
   int32_t n;                    /* clouds                                      */
   uint32_t flags;               /* creation flags                              */
   int32_t records_per_tile;     /* records of a work tile (NN and query)       */
-  int32_t blocks_per_sm_nn;     /* persistent blocks per SM, NN stage          */
+  int32_t blocks_per_sm_nn;     /* persistent blocks per SM, NN stage (of 128
+                                   threads)                                    */
   int32_t blocks_per_sm_tv;     /* ... L_TV sweep                              */
   int32_t blocks_per_sm_query;  /* ... fused query forward + backward          */
   int32_t error_bits;           /* kernel error flags raised so far (0 = none) */

@@ -502,8 +502,8 @@ struct gp_multi {
   std::vector<gp_band*> bands;
   std::vector<int64_t> B, rec_off, grad_off;
   int64_t total_B = 0, V_total = 0, J_total = 0;
-  int tq = 256;                    // records per tile = block size of the record kernels
-  int bpsm[ST_TUNED] = {4, TV_BLOCKS_PER_SM, 4};  // persistent blocks per SM of the tuned stages
+  int tq = 256;                    // records per tile; a query block has min(tq, 256) threads
+  int bpsm[ST_TUNED] = {8, TV_BLOCKS_PER_SM, 4};  // persistent blocks per SM of the tuned stages, whatever tq
   MShape* shapes = nullptr;
   MTile *rec_tiles = nullptr, *pt_tiles = nullptr, *brick_tiles = nullptr, *active_tiles = nullptr;
   int64_t n_rec_tiles = 0, n_pt_tiles = 0, n_brick_tiles = 0, n_active_tiles = 0;
@@ -568,8 +568,8 @@ unsigned persistent_grid(const gp_multi* m, int bpsm, int64_t ntiles) {
 gp_status launch_nn(gp_multi* m) {
   gp_ctx* ctx = m->ctx;
   GP_KERNEL(ctx, "k_m_nn",
-            k_m_nn<<<persistent_grid(m, m->bpsm[ST_NN] * m->tq / M_NN_THREADS, m->n_rec_tiles * m->tq / M_NN_THREADS),
-                     M_NN_THREADS, 0, ctx->stream>>>(
+            k_m_nn<<<persistent_grid(m, m->bpsm[ST_NN], m->n_rec_tiles * m->tq / M_NN_THREADS), M_NN_THREADS, 0,
+                     ctx->stream>>>(
                 m->shapes, m->rec_tiles, m->n_rec_tiles, m->tq, m->q, m->src, m->rec, m->nvalid));
   return GP_OK;
 }

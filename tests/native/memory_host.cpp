@@ -109,6 +109,22 @@ int main(int argc, char** argv) {
     gp_destroy(ctx);
     gp_multi_destroy(m);  // last, as a collector may have it
     printf("left %d\n", (int)fake::reserved() + fake::blocks());
+  } else if (!strcmp(what, "tuned")) {
+    // Blocks of the search's launch against gp_multi_info, before and after the
+    // autotuner (which here finds the longest tiles the fastest).
+    gp_ctx* ctx = nullptr;
+    gp_create(&ctx, 0, s1);
+    gp_multi* m = make_multi(ctx, make_band(ctx, 100), 100000);
+    gp_multi_info i;
+    const gp_loss_w w = {1.f, 1.f, 0.005f};
+    step(m);
+    gp_multi_get_info(m, &i);
+    printf("default %d\n", (int)fake::last_grid["k_m_nn"] - 8 * i.blocks_per_sm_nn);
+    if (gp_multi_autotune(m, &w)) printf("error autotune\n");
+    step(m);
+    gp_multi_get_info(m, &i);
+    printf("records_per_tile %d\ntuned %d\n", i.records_per_tile,
+           (int)fake::last_grid["k_m_nn"] - 8 * i.blocks_per_sm_nn);
   }
   return 0;
 }

@@ -62,3 +62,9 @@ def test_pointers_handed_out_are_ordinary_allocations(run):
     memory is not.  A block given back serves the next band; none is left after
     the last context, nor after an object that outlived it."""
     assert run("shown") == {"values": 0, "moments": 0, "multi": 0, "kept": 1, "left": 0}
+
+
+def test_search_runs_the_blocks_that_were_tuned(run):
+    """The search's blocks per SM stay what gp_multi_info says and what the
+    autotuner timed, whichever tile length the query stage then takes."""
+    assert run("tuned") == {"default": 0, "records_per_tile": 512, "tuned": 0}
