@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(TV_SWEEP_THREADS, TV_BLOCKS_PER_SM) k_m_tv(con
     }
     *reinterpret_cast<float4*>(S.grad + at) = make_float4(v[0], v[1], v[2], v[3]);
   };
-  tv_sweep<true>(MultiTvSrc{shapes, tiles}, ntiles, sh, fetch, out, [&](int64_t ti, float ts) {
+  tv_sweep<true, false>(MultiTvSrc{shapes, tiles}, ntiles, sh, fetch, out, [&](int64_t ti, float ts) {
     const int shape = tiles[ti].shape;
     if (shape != cur) {
       if (cur >= 0) flush();

@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(TV_THREADS, TV_BLOCKS_PER_SM) k_tv(Grid G, con
   };
   if (TV) {
     __shared__ TvShared sh;
-    tv_sweep<GRAD>(
+    tv_sweep<GRAD, false>(
         BandTvSrc{G, coord, nbrs}, n_bricks, sh, fetch,
         [&](int64_t slot, int q, float4, float4 g, const FixQuad& f) { emit(slot, q, g, f); },
         [&](int64_t, float ts) { tsum += ts; });
@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(TV_THREADS, TV_BLOCKS_PER_SM) k_tv_adam(
   };
   if (TV) {
     __shared__ TvShared sh;
-    tv_sweep<true>(BandTvSrc{G, coord, nbrs}, n_bricks, sh, fetch, update, [&](int64_t, float ts) { tsum += ts; });
+    tv_sweep<true, true>(BandTvSrc{G, coord, nbrs}, n_bricks, sh, fetch, update, [&](int64_t, float ts) { tsum += ts; });
   } else {
     const int64_t n = n_bricks * 128;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {

@@ -421,8 +421,8 @@ __device__ __forceinline__ bool query_record(const Grid& G, const float q[3], co
 // The band stores every in-grid axis neighbour of a T vertex, so a value the
 // sums use is always present: absent bricks are staged as zeros.  In bricks at
 // the grid's boundary the vertices just outside take the values of their
-// in-grid neighbours (difference 0); padding slots get gradient 0, and their own
-// values go to out().
+// in-grid neighbours (difference 0); padding slots get gradient 0 and, with
+// VALUES, out() their own values.
 constexpr int TV_SWEEP_THREADS = 128;
 constexpr int TV_SWEEP_WARPS = TV_SWEEP_THREADS / 32;
 constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM: 43 KB of shared memory, 102 registers a thread
@@ -605,8 +605,8 @@ __device__ __forceinline__ float4 tv_grad4(float4 c, float left, float right, fl
 // stencil work then hides, and out(i, q, d, g, fetched) with the quad's values
 // and unscaled gradient; done(i, tsum) is called by every lane after each item
 // with its share of the sum of TV_i.  All lanes of the warp call these together.
-// GRAD = false: the sums only (no layers, no fetch, no out).
-template <bool GRAD, class Src, class Fetch, class Out, class Done>
+// GRAD = false: the sums only (no layers, no fetch, no out).  VALUES: out() uses d.
+template <bool GRAD, bool VALUES, class Src, class Fetch, class Out, class Done>
 __device__ __forceinline__ void tv_sweep(const Src& src, int64_t n, TvShared& sh, Fetch&& fetch, Out&& out,
                                          Done&& done) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -720,14 +720,22 @@ __device__ __forceinline__ void tv_sweep(const Src& src, int64_t n, TvShared& sh
                           iright, tv_ld4(s.inv + ir - 8 + 4 * xq), tv_ld4(s.inv + ir + 8 + 4 * xq), izm, izp);
       float4 own = c;
       if (edge) {
-        // Padding slots: gradient 0 and the values the band holds there, not
-        // those tv_close_grid put beside the grid.
-        const int slot = __shfl_sync(0xffffffffu, nbr, 13);  // the brick's own
-        const int in = bk.oy + y <= bk.R && bk.oz + z <= bk.R ? bk.R - (bk.ox + 4 * xq) : -1;  // the last one in the grid
-        if (in < 3) {
-          const float4 held = __ldg(reinterpret_cast<const float4*>(bk.D + (int64_t)slot * 512 + 4 * q));
-          g = make_float4(in >= 0 ? g.x : 0.f, in >= 1 ? g.y : 0.f, in >= 2 ? g.z : 0.f, 0.f);
-          own = make_float4(in >= 0 ? c.x : held.x, in >= 1 ? c.y : held.y, in >= 2 ? c.z : held.z, held.w);
+        const bool row = bk.oy + y <= bk.R && bk.oz + z <= bk.R;
+        const int x = bk.ox + 4 * xq;
+        g.x = row && x <= bk.R ? g.x : 0.f;
+        g.y = row && x + 1 <= bk.R ? g.y : 0.f;
+        g.z = row && x + 2 <= bk.R ? g.z : 0.f;
+        g.w = row && x + 3 <= bk.R ? g.w : 0.f;
+        if (VALUES) {
+          // Not those that tv_close_grid put beside the grid.
+          const int slot = __shfl_sync(0xffffffffu, nbr, 13);
+          if (!row || x + 3 > bk.R) {
+            const float4 held = __ldg(reinterpret_cast<const float4*>(bk.D + (int64_t)slot * 512 + 4 * q));
+            own.x = row && x <= bk.R ? c.x : held.x;
+            own.y = row && x + 1 <= bk.R ? c.y : held.y;
+            own.z = row && x + 2 <= bk.R ? c.z : held.z;
+            own.w = held.w;
+          }
         }
       }
       out(i, q, own, g, got);
