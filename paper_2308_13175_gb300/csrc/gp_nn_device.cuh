@@ -10,6 +10,13 @@
 
 constexpr float NN_EPS = 3.814697265625e-06f;  // 2^-18
 constexpr float NN_TINY = 1e-30f;
+// A hint more than this many cells away (twice as many where the query's own
+// block is empty) is passed over: it says nothing about where the nearest point
+// is, and the ball of what is found beside it holds much of the cloud (262,144
+// queries among 100,000 points of a surface, random points as hints: 7,200 us,
+// and 160 with them passed over).  A query's own source point lies within four
+// sigma, six cells at the usual 50 neighbours and 6.5 points a cell.
+constexpr float NN_FAR_HINT = 8.f;
 
 // The cloud in a uniform grid of G^3 cells, grouped into blocks of 4^3 cells
 // and super-blocks of 4^3 blocks.  Only what holds points is stored.
@@ -345,6 +352,12 @@ static __device__ __noinline__ int nn_near_block(float q0, float q1, float q2, c
   return at;
 }
 
+// Whether the block q lies in holds no point.
+__device__ __forceinline__ bool nn_block_empty(const float q[3], const NNGrid& g) {
+  const int bx = nn_cell(q[0], g) >> 2, by = nn_cell(q[1], g) >> 2, bz = nn_cell(q[2], g) >> 2;
+  return __ldg(g.table + ((int64_t)bz * g.nbk + by) * g.nbk + bx) < 0;
+}
+
 // Step 1 of a search: a first point.  hint: index of a cloud point
 // to start from (-1: none); a record of `seeds` is a point s and its normal n
 // as three 10-bit signed fractions of 511 (0: unknown).  The nearest point is
@@ -362,12 +375,14 @@ __device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, c
   t = NNTop{INFINITY, INFINITY, -1};
   float f[3] = {q[0], q[1], q[2]};
   float4 s = make_float4(q[0], q[1], q[2], 0.f);
-  const bool hinted = hint >= 0 && hint < J;
+  bool hinted = hint >= 0 && hint < J;
   if (hinted) {
-    s = __ldg(seeds + hint);
-    const float d = nn_d32(q, s.x, s.y, s.z);
+    const float4 p = __ldg(seeds + hint);
+    const float d = nn_d32(q, p.x, p.y, p.z), far = NN_FAR_HINT * g.cs;
     if (COUNT) ++work;
-    if (d < INFINITY) {
+    hinted = d <= far * far || (d <= 4.f * far * far && nn_block_empty(q, g));
+    if (hinted) {
+      s = p;
       const int w = __float_as_int(s.w);
       const float n0 = (float)((w << 22) >> 22) * (1.0f / 511.0f), n1 = (float)((w << 12) >> 22) * (1.0f / 511.0f),
                   n2 = (float)((w << 2) >> 22) * (1.0f / 511.0f);
