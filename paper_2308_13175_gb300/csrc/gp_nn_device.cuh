@@ -280,7 +280,9 @@ __device__ __forceinline__ void nn_super(const float q[3], const NNGrid& g, floa
 }
 
 // Visit the cells that can hold a point within squared distance thr of q, thr
-// known: the blocks that the box of that ball meets.  It ranks near ties, in which
+// known: the blocks that the box of that ball meets, in super-blocks the ball
+// meets (of a query far outside, the box is most of the grid: 20,000 queries at
+// six radii 22.7 ms without that test, 13.2 with it).  It ranks near ties, in which
 // a lane works by itself while its warp waits: with nn_walk, which tests every
 // block of the super-block, 200,000 queries with 8-way ties took 1,419 us, now
 // 676, and 262,144 queries among a noisy object's points 116, now 89 (as a
@@ -296,9 +298,13 @@ __device__ __forceinline__ void nn_ball(const float q[3], const NNGrid& g, float
   }
   for (int sz = lo[2] >> 2; sz <= hi[2] >> 2; ++sz)
     for (int sy = lo[1] >> 2; sy <= hi[1] >> 2; ++sy)
-      for (int sx = lo[0] >> 2; sx <= hi[0] >> 2; ++sx)
+      for (int sx = lo[0] >> 2; sx <= hi[0] >> 2; ++sx) {
+        const float dx = nn_super_gap(q[0], sx, g, margin), dy = nn_super_gap(q[1], sy, g, margin),
+                    dz = nn_super_gap(q[2], sz, g, margin);
+        if (dx * dx + dy * dy + dz * dz > thr) continue;
         nn_super(q, g, margin, thr, sx, sy, sz,
                  __ldg(g.sup + ((int64_t)sz * g.nsup + sy) * g.nsup + sx) & nn_box_mask(lo, hi, sx, sy, sz), visit);
+      }
 }
 
 // Visit, in rings of super-blocks around q, the cells that can hold a point
