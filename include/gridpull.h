@@ -31,7 +31,7 @@
  *     after the call returns.  The library owns the band (brick table, D, Adam
  *     moments, point cell list, scratch) and frees it in gp_band_destroy.  The
  *     pointers of gp_band_values and gp_multi_buffers lie in memory of
- *     cudaMalloc; everything else comes from a stream-ordered pool.  Up to 320
+ *     cudaMalloc; everything else comes from a stream-ordered pool.  Up to 512
  *     MB of what was freed stays with the library until the last context of the
  *     device is destroyed.
  *   - Streams.  Every call is asynchronous on the context's stream, except

@@ -48,12 +48,13 @@ void gp_pool_release(int device);
 // Memory whose address callers receive (gp_band_values, gp_multi_buffers) is
 // cudaMalloc's: a pool's is not opened to other devices by
 // cudaDeviceEnablePeerAccess, not copied between devices by cudaMemcpyAsync and
-// has no cudaIpcMemHandle.  A malloc and a free of 10 MB take 89 us and more
-// beside a build (a band of 100,000 points 1,123 -> 1,312 us), so up to
-// GP_SHOWN_KEEP bytes of blocks given back stay with the device, as the pool's
-// memory does, for requests of at least half their size (the same build:
-// 1,104 us).  A block is given back by gp_shown_give only when no stream uses it.
-constexpr size_t GP_SHOWN_KEEP = size_t(64) << 20;
+// has no cudaIpcMemHandle.  A malloc and a free of 10 MB take 89 us, and more in
+// a build (a band of 100,000 points 1,123 -> 1,312 us, one of 40,252 points with
+// 80 MB of such arrays 896 -> 1,154), so up to GP_SHOWN_KEEP bytes of blocks given
+// back stay with the device, as the pool's memory does, for requests of at least
+// half their size (the same builds: 1,096 and 889 us).  A block is given back by
+// gp_shown_give only when no stream uses it.
+constexpr size_t GP_SHOWN_KEEP = size_t(256) << 20;
 constexpr int GP_SHOWN_BLOCKS = 32;  // blocks kept at most
 struct gp_shown {
   void* p = nullptr;
