@@ -397,8 +397,11 @@ __device__ __forceinline__ bool nn_block_empty(const float q[3], const NNGrid& g
 // Step 1 of a search: a first point.  hint: index of a cloud point
 // to start from (-1: none); a record of `seeds` is a point s and its normal n
 // as three 10-bit signed fractions of 511 (0: unknown).  The nearest point is
-// expected around the foot of q on the tangent plane of s, then on the plane
-// of the block there (of the block of s, where that one holds no point); the
+// expected around the foot of q on the tangent plane of s, then, if that lies
+// outside, on the near face of the slab of the block there (of the block of s,
+// where that one holds no point; a block that is not flat leaves the place as it
+// is: on its middle plane instead, 300,000 hinted queries in a volume of a million
+// points took 139 us, 93 now, in a thick shell 185, now 143); the
 // points of the 2^3 cells nearest to that place are scanned, or those of the
 // whole block where these are empty.  A query without a hint tends to lie on
 // the surface (a mesh scored against a cloud); within half a cell of the plane
@@ -447,7 +450,8 @@ __device__ __forceinline__ int nn_first(const float q[3], int hint, int64_t J, c
   const float4 A = __ldg(g.blk + 2 * (int64_t)bi), B = __ldg(g.blk + 2 * (int64_t)bi + 1);
   const NNBlock k = nn_block(B);
   const float n[3] = {A.x, A.y, A.z};
-  const float off = 0.5f * (A.w + B.x) - (A.x * f[0] + A.y * f[1] + A.z * f[2]);
+  const float nf = A.x * f[0] + A.y * f[1] + A.z * f[2];
+  const float off = fminf(fmaxf(nf, A.w), B.x) - nf;
   const int corner[3] = {4 * bx, 4 * by, 4 * bz};
   const float h = n[0] * q[0] + n[1] * q[1] + n[2] * q[2] - 0.5f * (A.w + B.x);
   int how = !hinted && fabsf(h) < 0.5f * g.cs ? 2 : 0;
