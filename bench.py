@@ -79,9 +79,8 @@ def alg_bytes(name, n, J, Vs, Vt):
         "k_seed_points": 28 * J,  # a band without normals: points read, seeds written (at set-up)
         "k_count_valid": 24 * n,
         "k_tv": 8 * Vs,
-        # the sweep without a gradient, and with the fixed-point sums folded in,
-        # under the names and bytes of the two passes that stored 1/TV between
-        # them (the first now only reads D: 4 bytes a slot)
+        # two passes that stored 1/TV between them; sweeps are traced under their
+        # names now (launch_bytes)
         "k_tv_inv": 8 * Vs,
         "k_tv_grad": 12 * Vs,
         "k_query": 24 * n + 8 * Vt,
@@ -92,8 +91,16 @@ def alg_bytes(name, n, J, Vs, Vt):
     }.get(name, 0)
 
 
-# The nearest-point kernels are bound by issue and SIMT divergence in their
-# float32 distance arithmetic, not by bytes: their roofline is the FP32 pipe,
+def launch_bytes(name, n, J, Vs, Vt):
+    """The bytes of a traced launch: alg_bytes, but for the L_TV sweep without a
+    gradient (D read), traced as k_tv_inv, and the one that folds the
+    fixed-point sums in (D read, gradient written; per trainable vertex two
+    64-bit sums read and cleared), traced as k_tv_grad."""
+    return {"k_tv_inv": 4 * Vs, "k_tv_grad": 8 * Vs + 32 * Vt}.get(name, alg_bytes(name, n, J, Vs, Vt))
+
+
+# The nearest-point kernels are bound by the L1's wavefronts and by latency in
+# reaching their candidates, not by bytes of DRAM: they are rated on the FP32 pipe,
 # in the flops of the candidate distances they evaluate (counted by
 # gp_nn_work): per candidate 3 subtractions, 1 multiply and 2 FMAs = 8 flops
 # (FMA = 2).  Peak: 152 SMs x 128 FP32 lanes x 2 flops x the maximum SM clock.
@@ -590,7 +597,7 @@ def run_ours(args, world, rank, local):
     per_kernel = {}
     for name, (cnt, tot) in kern.items():
         per_step_n = q_prof / args.steps
-        by = alg_bytes(name, per_step_n, J, Vs, Vt)
+        by = launch_bytes(name, per_step_n, J, Vs, Vt)
         avg_ms = tot / cnt
         per_kernel[name] = {"launches": cnt, "avg_us": round(1e3 * avg_ms, 2),
                             "share": round(tot / max(sum(v[1] for v in kern.values()), 1e-12), 4),
@@ -983,7 +990,7 @@ def run_collection(args, world, rank, local):
     per_kernel = {}
     tot_all = max(sum(v[1] for v in kern.values()), 1e-12)
     for name, (cnt, tot) in kern.items():
-        by = alg_bytes(name.replace("k_m_", "k_"), q_prof / Kp, J, Vs, Vt)
+        by = launch_bytes(name.replace("k_m_", "k_"), q_prof / Kp, J, Vs, Vt)
         if name == "k_m_perm":
             by = 8 * J / wl["batches_per_epoch"]  # an epoch's order, once per epoch
         avg_ms = tot / cnt
