@@ -92,9 +92,9 @@ cudaError_t gp_shown_take(int device, size_t bytes, gp_shown* block) {
   if (scope.err != cudaSuccess) return scope.err;
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, bytes);
-  if (e == cudaErrorMemoryAllocation && d.idle_bytes > 0) {
+  if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();
-    drop_idle(d);
+    empty_pool(d);
     e = cudaMalloc(&p, bytes);
   }
   if (e == cudaSuccess) *block = gp_shown{p, bytes};
@@ -115,6 +115,11 @@ void gp_shown_give(int device, gp_shown* block) {
         return;
       }
   cudaFree(b.p);
+}
+
+void gp_drop_kept(int device) {
+  std::lock_guard<std::mutex> lock(g_pool_mutex);
+  empty_pool(device_pools()[device]);
 }
 
 void gp_free_idle_done(int device) {

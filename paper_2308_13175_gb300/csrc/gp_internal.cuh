@@ -62,6 +62,9 @@ struct gp_shown {
 };
 cudaError_t gp_shown_take(int device, size_t bytes, gp_shown* block);
 void gp_shown_give(int device, gp_shown* block);
+// What the device keeps of freed memory is given up: for an allocation that
+// found no memory.
+void gp_drop_kept(int device);
 
 // After the last gp_free_idle of an object: a pool gives back what exceeds the
 // bytes it keeps, and a trim finds the rest, only once the host has seen the
@@ -174,6 +177,11 @@ gp_status gp_alloc(gp_ctx* ctx, T** p, size_t count, const char* what) {
   *p = nullptr;
   if (count == 0) count = 1;
   cudaError_t e = cudaMallocFromPoolAsync((void**)p, count * sizeof(T), ctx->pool, ctx->stream);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    gp_drop_kept(ctx->device);
+    e = cudaMallocFromPoolAsync((void**)p, count * sizeof(T), ctx->pool, ctx->stream);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;

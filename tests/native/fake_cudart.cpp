@@ -81,6 +81,7 @@ void forget(void* p, const Stream& order) {
 }  // namespace
 
 namespace fake {
+size_t capacity = ~size_t(0);
 int races = 0, wrong_device = 0, fail_set_attribute = 0;
 std::map<std::string, unsigned> last_grid;
 
@@ -90,6 +91,11 @@ size_t reserved() {
     n += p.second.live + p.second.held;
     for (auto& f : p.second.freed) n += f.second;
   }
+  return n;
+}
+size_t used() {
+  size_t n = reserved();
+  for (auto& b : g_blocks) n += b.second.pool ? 0 : b.second.bytes;
   return n;
 }
 uint64_t lowest_threshold() {
@@ -216,13 +222,22 @@ cudaError_t cudaMemPoolTrimTo(cudaMemPool_t pool, size_t keep) {
   if (p.held > keep) p.held = keep;  // frees that the host has not seen complete stay
   return cudaSuccess;
 }
+static bool full(size_t n) { return fake::used() + n > fake::capacity; }
 cudaError_t cudaMallocFromPoolAsync(void** p, size_t n, cudaMemPool_t pool, cudaStream_t) {
+  Pool& from = g_pools.at(pool);
+  const size_t reuse = from.held < n ? from.held : n;
+  from.held -= reuse;
+  if (full(n)) {
+    from.held += reuse;
+    return cudaErrorMemoryAllocation;
+  }
   *p = calloc(n, 1);
   g_blocks[*p] = Block{n, g_pools.at(pool).device, pool};
   g_pools.at(pool).live += n;
   return cudaSuccess;
 }
 cudaError_t cudaMalloc(void** p, size_t n) {
+  if (full(n)) return cudaErrorMemoryAllocation;
   *p = calloc(n, 1);
   g_blocks[*p] = Block{n, g_device, nullptr};
   return cudaSuccess;

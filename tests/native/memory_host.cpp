@@ -125,6 +125,23 @@ int main(int argc, char** argv) {
     gp_multi_get_info(m, &i);
     printf("records_per_tile %d\ntuned %d\n", i.records_per_tile,
            (int)fake::last_grid["k_m_nn"] - 8 * i.blocks_per_sm_nn);
+  } else if (!strcmp(what, "full")) {
+    // Allocations that fit only once kept memory is given up: a band's from the
+    // pool with blocks kept, then a multi's blocks with the pool's memory kept.
+    gp_ctx* ctx = nullptr;
+    gp_create(&ctx, 0, s1);
+    gp_band* b = make_band(ctx, 100);
+    gp_multi* m = make_multi(ctx, b, 4000000);
+    gp_multi_destroy(m);
+    gp_band_destroy(b);
+    fake::capacity = fake::used() + (size_t(60) << 20);
+    b = make_band(ctx, 2000000);
+    printf("band %d\n", b != nullptr);
+    gp_band_destroy(b);
+    b = make_band(ctx, 100);
+    fake::capacity = fake::used() + (size_t(20) << 20);
+    m = make_multi(ctx, b, 2000000);
+    printf("multi %d\n", m != nullptr);
   }
   return 0;
 }

@@ -68,3 +68,8 @@ def test_search_runs_the_blocks_that_were_tuned(run):
     """The search's blocks per SM stay what gp_multi_info says and what the
     autotuner timed, whichever tile length the query stage then takes."""
     assert run("tuned") == {"default": 0, "records_per_tile": 512, "tuned": 0}
+
+
+def test_kept_memory_is_given_up_for_an_allocation(run):
+    """On a full device what is kept does not make an allocation fail."""
+    assert run("full") == {"band": 1, "multi": 1}
