@@ -418,8 +418,9 @@ constexpr int NN_THREADS = 128;
 
 // One lane per query (nn_search works on a warp's 32 together).  Queries with a
 // NaN, infinite or huge coordinate (whose squared distances would overflow
-// float32) get -1 and a NaN surface point.  COUNT: also add the number of point distances evaluated (seeds, cells and
-// tie-break) to *work_total, for measurement; the search is the same.
+// float32) get -1 and a NaN surface point.  COUNT: also add the number of point
+// distances evaluated (seeds, cells and tie-break) to *work_total, for
+// measurement; the search is the same.
 template <bool COUNT>
 __global__ void __launch_bounds__(NN_THREADS, 8) k_nn(NNGrid g, const float* __restrict__ qin, int64_t n,
                                                       const int32_t* __restrict__ hint, int64_t J,

@@ -29,7 +29,7 @@ constexpr float NN_FAR_HINT = 8.f;
 // instructions with the points as records of four floats).  The parts are
 // rotated by the chunk's number (nn_part), so that lanes reading the same part
 // of chunks anywhere spread over the banks: 1,500,001 queries among 2 M points
-// take 491 us, 520 us in a fixed order.
+// took 491 us with it, 520 us in a fixed order.
 //
 // A block with points has a record of two float4,
 //   (n.x, n.y, n.z, lo), (hi, first occupied cell, occupancy mask: 2 words),
@@ -518,8 +518,10 @@ struct NNWarp {
 // Measured (GB300, seeded batches, whole search): with one thread walking its
 // query's rows of cells, 8 of 32 lanes active, 1,116 us for 2,097,152 queries
 // among 10 M points and 206 us for 262,144 among 100,000; with step 2 lane by
-// lane 730 and 210; shared 503 and 111.  It is then bound by the L1 (81% of its
-// wavefronts: a lane's chunk is a line of its own) and by issue (56%).
+// lane 730 and 210; shared 503 and 111 (488 and 86 as the search stands).  It is
+// then bound by the L1, for which a lane's chunk is a line of its own, and by issue
+// (75% of the L1's throughput and 64% of the issue slots with 1,500,001 queries; 52%
+// and 64% with 262,144, which leave latency).
 // Sorting a block's queries by radius instead of sharing gave 700 and 190.
 template <bool COUNT>
 __device__ __forceinline__ void nn_rest(const float q[3], const NNGrid& g, bool go, int first, NNTop& t, NNWarp& sh,

@@ -425,7 +425,7 @@ __device__ __forceinline__ bool query_record(const Grid& G, const float q[3], co
 // VALUES, out() their own values.
 constexpr int TV_SWEEP_THREADS = 128;
 constexpr int TV_SWEEP_WARPS = TV_SWEEP_THREADS / 32;
-constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM: 43 KB of shared memory, 102 registers a thread
+constexpr int TV_BLOCKS_PER_SM = 5;  // resident blocks per SM: 43 KB of shared memory; at most 102 registers (92 to 96 used)
 constexpr int TV_DENSE = 144 * 8;    // rows (y, z) in [-2, 9]^2, x in [0, 8)
 constexpr int TV_SIDE = 100 * 2;     // rows (y, z) in [-1, 8]^2: x = -2, -1 or x = 8, 9
 constexpr int TV_COPIES = 264 + 192; // 16-byte pieces of rows, 8-byte pieces of the sides

@@ -101,12 +101,12 @@ class FitStep:
         the grid values, so only the record buffers need ordering (two of
         them, alternating).  With the separate descent (gp_step, then
         gp_update) the next draw starts once the current gp_step is done and
-        overlaps its Adam update: measured on the 10M-point scene, letting it
-        overlap gp_step's L_TV passes and query pass too made the step slower
-        than running everything in turn (the search and those passes contend
-        for L2), while overlapping Adam only made it faster.  With the fused
-        descent (gp_step_update, whose sweep holds every SM) the draw is
-        issued beside the whole descent.  The calling stream waits for
+        overlaps its Adam update (on the 10M-point scene 1.27 ms a step, 1.29
+        with everything in turn and the L2 flushed between steps: the order
+        dates from kernels that are gone, when also overlapping gp_step lost
+        time, and gains little now).  With the fused descent (gp_step_update,
+        whose sweep holds every SM) the draw is issued beside the whole
+        descent.  The calling stream waits for
         everything before this returns (asynchronously, as every call here).
         Returns the loss buffer of the last step."""
         if K <= 0:
